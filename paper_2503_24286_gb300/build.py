@@ -21,12 +21,20 @@ CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
-def _embed_devmath() -> str:
-    src = open(os.path.join(CSRC, "pyro_device_math.cuh")).read()
+# device sources compiled at run time (NVRTC), embedded as strings
+EMBED = {"pyro_device_math.cuh": "kDeviceMathSource", "pyro_fixed_math.cuh": "kFixedMathSource",
+         "pyro_tile.cuh": "kTileSource"}
+
+
+def _embed_sources() -> str:
     out = os.path.join(BUILD, "pyro_devmath_src.cpp")
-    text = ('// generated from pyro_device_math.cuh\nnamespace pyro {\n'
-            'extern const char* kDeviceMathSource;\n'
-            'const char* kDeviceMathSource = R"PYRODM(' + src + ')PYRODM";\n}\n')
+    text = "// generated from " + ", ".join(EMBED) + "\nnamespace pyro {\n"
+    for name, var in EMBED.items():
+        src = open(os.path.join(CSRC, name)).read()
+        # adjacent literals: compilers need not accept one of more than 64 KB
+        parts = ['R"PYRODM(' + src[i:i + 15000] + ')PYRODM"' for i in range(0, len(src), 15000)]
+        text += "extern const char* %s;\nconst char* %s =\n%s;\n" % (var, var, "\n".join(parts))
+    text += "}\n"
     if not os.path.exists(out) or open(out).read() != text:
         with open(out, "w") as f:
             f.write(text)
@@ -45,7 +53,7 @@ def build(verbose: bool = False) -> str:
     os.makedirs(os.path.dirname(LIB), exist_ok=True)
     headers = glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         glob.glob(os.path.join(INCLUDE, "*.h"))
-    cpp = sorted(glob.glob(os.path.join(CSRC, "*.cpp"))) + [_embed_devmath()]
+    cpp = sorted(glob.glob(os.path.join(CSRC, "*.cpp"))) + [_embed_sources()]
     cu = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     jobs = []
     for s in cpp:

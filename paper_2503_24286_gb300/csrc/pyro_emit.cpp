@@ -30,6 +30,7 @@
 //    Newton slope until |dT| <= tol T, plus one further step.
 #include "pyro_emit.h"
 #include "pyro_emit_common.h"
+#include "pyro_emit_tile.h"
 #include "pyro_emit_warp.h"
 
 #include <algorithm>
@@ -2178,10 +2179,17 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
 
   // ---- net production rates (Eq. production_rates) ------------------------------
   Src r;   // count the forward per-point path separately
-  r << "\nextern \"C\" __global__ void __launch_bounds__(BLK, MINB) pyro_omega(i64 n, const double* __restrict__ g_rho,\n"
+  r << "\n#define TILE_OPEN " << kTileOpen << "\n";
+  r << "extern \"C\" __global__ void __launch_bounds__(BLK, MINB) pyro_omega(i64 n, const double* __restrict__ g_rho,\n"
        "    const double* __restrict__ g_Tin, int energy_mode, const double* __restrict__ g_Y,\n"
        "    double* __restrict__ g_Tout, double* __restrict__ g_omega, double T_guess, int max_iter, double tol,\n"
-       "    unsigned long long* __restrict__ g_fail, double* __restrict__ g_store) {\n"
+       "    unsigned long long* __restrict__ g_fail, double* __restrict__ g_store, int open_only) {\n"
+       "  // open_only: only the states that the tile kernel left open (pyro_tile.cuh)\n"
+       "  if (open_only) {\n    bool any = false;\n"
+       "    #pragma unroll 8\n"
+       "    for (i64 p = (i64)blockIdx.x * BLK + threadIdx.x; p < n; p += (i64)gridDim.x * BLK)\n"
+       "      any |= __double_as_longlong(g_omega[p]) == TILE_OPEN;\n"
+       "    if (!__syncthreads_or(any)) return;\n  }\n"
        "  __shared__ double s_exp[512];\n  __shared__ double s_log[256];\n"
        "  extern __shared__ double s_dyn[];\n"
        "  double* sL = " << (opt.gstore ? "g_store + (i64)blockIdx.x * 2 * NSP * BLK" : "s_dyn") << ";\n"
@@ -2189,6 +2197,7 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
        "  pyro_load_tables(s_exp, s_log);\n  __syncthreads();\n"
        "  const int t = threadIdx.x;\n  const float tolf = (float)tol;\n"
        "  for (i64 p = (i64)blockIdx.x * BLK + t; p < n; p += (i64)gridDim.x * BLK) {\n"
+       "    if (open_only && __double_as_longlong(g_omega[p]) != TILE_OPEN) continue;\n"
        "    const double* Yp = g_Y + p;\n    const double rho = g_rho[p];\n"
        "    double T;\n"
        "    if (energy_mode) {\n      int it;\n"
@@ -2303,6 +2312,19 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
     out.warp_wpb = w.wpb;
     out.smem_dyn_bytes_warp = w.smem;
     out.stats["deriv_warp_per_state"] = 1;
+  }
+  {
+    // tile kernel of the net production rates (the form that evaluates almost every state)
+    const TileEmit t = emit_tile_unit(m);
+    out.stats["tile"] = t.source.empty() ? 0 : 1;
+    if (!t.source.empty()) {
+      out.group_sources["tile"] = t.source;
+      out.tile_warps = t.warps;
+      out.smem_dyn_bytes_tile = t.smem_bytes;
+      out.stats["tile_t_lo"] = t.t_lo;
+      out.stats["tile_warps"] = t.warps;
+      out.stats["tile_chunks"] = t.chunks;
+    }
   }
   out.stats["deriv_block"] = opt.deriv_block;
 

@@ -41,6 +41,8 @@ struct EmitResult {
   int smem_dyn_bytes_cn_solve = 0;        // dynamic shared memory of the Crank-Nicolson solve kernel
   int smem_dyn_bytes_transport = 0;       // dynamic shared memory of the transport kernel
   int smem_dyn_bytes_jac = 0;             // dynamic shared memory of the Jacobian-type kernels
+  int tile_warps = 0;                     // warps per block of the tile kernel
+  int smem_dyn_bytes_tile = 0;            // dynamic shared memory of the tile kernel
   int cn_solve_warps = 4;                 // states (warps) per block of the Crank-Nicolson solve kernel
   // warp-per-state kernels ("wfwd", "wjvp", "wvjp"): states (warps) per block and
   // dynamic shared memory per block
@@ -54,6 +56,10 @@ constexpr int kTransportBlock = 32;
 // States per group of the Crank-Nicolson Newton-matrix layout [n/G][N^2][G]
 // (also the warps per block of the batched solve).
 constexpr int kCnGroup = 4;
+
+// First output of a state that the tile kernel leaves to the FP64 kernels: a NaN no
+// computation produces (and if one did, the state would only be evaluated again).
+constexpr const char* kTileOpen = "0x7ff8005059524f31ll";
 
 EmitResult emit_module(const Mechanism& m, const EmitOptions& opt);
 

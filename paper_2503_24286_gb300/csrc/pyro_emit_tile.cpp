@@ -1,0 +1,455 @@
+// Emitter of the tile kernel's tables (see pyro_tile.cuh for the kernel and
+// pyro_fixed_math.cuh for the number formats).
+#include "pyro_emit_tile.h"
+
+#include <algorithm>
+#include <cmath>
+#include <functional>
+#include <map>
+#include <sstream>
+#include <vector>
+
+#include "pyro_emit_common.h"
+
+namespace pyro {
+
+namespace {
+using namespace emitc;
+
+typedef long long i64;
+typedef unsigned long long u64;
+typedef long double ld;
+
+const ld LOG2E = 1.442695040888963407359924681001892137L;
+const ld T_HI = 5000.0L, T_T = 5000.5L;
+
+// fixed-point conversions; `bad` is set where a value does not fit
+struct Fix {
+  bool bad = false;
+  i64 lg(ld v) {          // f = 50, lowest bit clear
+    if (!(std::fabs((double)v) < 8000.0)) { bad = true; return 0; }
+    return (i64)llroundl(v * 562949953421312.0L) * 2;
+  }
+  i64 lg_any(ld v) {      // f = 50, all bits
+    if (!(std::fabs((double)v) < 8000.0)) { bad = true; return 0; }
+    return (i64)llroundl(v * 1125899906842624.0L);
+  }
+  i64 coef(ld v) {        // f = 51 as two signed halves
+    if (!(std::fabs((double)v) < 4000.0)) { bad = true; return 0; }
+    const i64 x = (i64)llroundl(v * 2251799813685248.0L);
+    const int lo = (int)(unsigned)(u64)x;
+    const i64 hi = (x - lo) / 4294967296ll;
+    return (i64)(((u64)hi << 32) | (unsigned)lo);
+  }
+};
+
+i64 dbits(double v) {
+  i64 b;
+  static_assert(sizeof b == sizeof v, "");
+  __builtin_memcpy(&b, &v, 8);
+  return b;
+}
+
+// log2 of lambda_k = phi_k/W_k as a function of T in range r (long double)
+ld lambda(const Species& s, int r, ld T) {
+  const double* a = r == 0 ? s.low : s.high;
+  const ld L = ((ld)a[0] - a[6] + logl(R_GAS / P_ATM) - logl((ld)s.W)) + (1.0L - a[0]) * logl(T) + a[5] / T -
+               T * ((ld)a[1] / 2 + T * ((ld)a[2] / 6 + T * ((ld)a[3] / 12 + T * (ld)a[4] / 20)));
+  return L * LOG2E;
+}
+
+struct Arr { ld c, b, theta; };     // log2 k = c + b log2 T - theta log2(e)/T
+ld arr_at(const Arr& a, ld T) { return a.c + a.b * log2l(T) - a.theta * LOG2E / T; }
+
+int classes(const Reaction& r) {   // tile_other's kinds; 0: plain
+  switch (r.kind) {
+    case RX_ARRHENIUS: return 0;
+    case RX_THREEBODY: return 1;
+    case RX_PLOG: return 5;
+    default: return r.n_sri >= 3 ? 4 : r.n_troe >= 3 ? 3 : 2;
+  }
+}
+
+template <class T>
+void array(std::ostringstream& o, const char* type, const char* name, const std::vector<T>& v) {
+  o << "__device__ const " << type << " " << name << "[" << std::max<size_t>(v.size(), 1) << "] = {";
+  for (size_t i = 0; i < v.size(); ++i) o << (i ? "," : "") << (i % 16 == 15 ? "\n" : "") << v[i];
+  if (v.empty()) o << "0";
+  o << "};\n";
+}
+
+std::vector<std::string> as_ll(const std::vector<i64>& v) {
+  std::vector<std::string> s;
+  for (i64 x : v) s.push_back(std::to_string(x) + "ll");
+  return s;
+}
+std::vector<std::string> as_d(const std::vector<double>& v) {
+  std::vector<std::string> s;
+  for (double x : v) s.push_back(lit(x));
+  return s;
+}
+
+}  // namespace
+
+TileEmit emit_tile_unit(const Mechanism& m) {
+  TileEmit out;
+  const int N = m.n_species(), NR = m.n_reactions();
+  if (N < 1 || N > 1022 || NR < 1) { out.why = "no reactions, or more than 1022 species"; return out; }
+  for (auto& r : m.reactions)
+    if (side_factors(r.reactants).size() > 3 || side_factors(r.products).size() > 3 ||
+        side_factors(r.reactants).empty() || (r.reversible && side_factors(r.products).empty())) {
+      out.why = "a reaction has more than three factors on a side";
+      return out;
+    }
+  const double tmid = m.species[0].t_mid;      // the range switch of every species, as in the other kernels
+
+  // ---- temperature range: the lowest T_LO from which every rate's exponent at unit
+  // concentrations is below 1190 (a product with one zero, 2^-2400, then vanishes) and
+  // above -8150 + 2460 per factor (a product of zeros stays in range: |lg| < 8192)
+  auto folded = [&](const Reaction& r, double A, double b, double theta) {
+    Arr a{log2l((ld)A), (ld)b, (ld)theta};
+    for (auto& p : r.reactants) a.c -= p.second * log2l((ld)m.species[p.first].W);
+    return a;
+  };
+  std::vector<std::vector<Arr>> forms(NR);       // the Arrhenius forms of each reaction
+  for (int j = 0; j < NR; ++j) {
+    const Reaction& r = m.reactions[j];
+    if (r.kind == RX_PLOG)
+      for (auto& q : r.plog) forms[j].push_back(folded(r, q.A, q.b, q.theta));
+    else
+      forms[j].push_back(folded(r, r.A, r.b, r.theta));
+    if (r.kind == RX_FALLOFF) {                  // the low-pressure limit bounds the falloff rate from below
+      Arr a = folded(r, r.A0, r.b0, r.theta0);
+      forms[j].push_back(a);
+    }
+  }
+  auto fits_from = [&](double lo) {
+    std::vector<ld> lam(N);
+    for (int i = 0; i <= 200; ++i) {
+      const ld T = lo * powl(T_HI / lo, i / 200.0L);
+      const int rg = T >= tmid ? 1 : 0;
+      for (int k = 0; k < N; ++k) lam[k] = lambda(m.species[k], rg, T);
+      for (int j = 0; j < NR; ++j) {
+        ld f = 0, g = 0;
+        for (auto& p : m.reactions[j].reactants) { f += p.second * lam[p.first]; g += p.second * logl((ld)m.species[p.first].W) * LOG2E; }
+        ld r = 0;
+        for (auto& p : m.reactions[j].products) r += p.second * lam[p.first];
+        for (auto& a : forms[j]) {
+          const ld K = arr_at(a, T) + g;         // log2 of the rate constant
+          const ld X = arr_at(a, T) - f + r;     // reverse exponent at unit products
+          const ld nf = (ld)side_factors(m.reactions[j].reactants).size(), np = (ld)side_factors(m.reactions[j].products).size();
+          if (!(K > -8150 + 2460 * nf && K < 1190 && X > -8150 + 2460 * np && X < 1190)) return false;
+        }
+      }
+    }
+    return true;
+  };
+  double t_lo = 0.0;
+  for (double lo : {200.0, 225.0, 250.0, 275.0, 300.0, 350.0, 400.0}) if (fits_from(lo)) { t_lo = lo; break; }
+  if (t_lo == 0.0) { out.why = "rate constants out of range above 400 K"; return out; }
+  const ld T_V = 0.9999L * (ld)t_lo;
+
+  // ---- species tables ----------------------------------------------------------
+  Fix fx;
+  std::vector<i64> sp((size_t)N * 16);
+  std::vector<double> ed((size_t)N * 12), iw(N);
+  std::ostringstream ef;
+  for (int k = 0; k < N; ++k) {
+    const Species& s = m.species[k];
+    const SpeciesCoef C = species_coef(s);
+    iw[k] = 1.0 / s.W;
+    for (int r = 0; r < 2; ++r) {
+      const double* a = r == 0 ? s.low : s.high;
+      const ld c0 = ((ld)a[0] - a[6] + logl(R_GAS / P_ATM) - logl((ld)s.W)) * LOG2E;
+      const ld c[4] = {-(ld)a[1] / 2 * T_T * LOG2E, -(ld)a[2] / 6 * T_T * T_T * LOG2E,
+                       -(ld)a[3] / 12 * T_T * T_T * T_T * LOG2E, -(ld)a[4] / 20 * T_T * T_T * T_T * T_T * LOG2E};
+      ld sum = fabsl(c0);
+      for (ld x : c) sum += fabsl(x);
+      if (!(sum < 4000)) fx.bad = true;
+      i64* q = &sp[((size_t)k * 2 + r) * 8];
+      q[0] = fx.lg_any(c[3]); q[1] = fx.lg_any(c[2]); q[2] = fx.lg_any(c[1]); q[3] = fx.lg_any(c[0]);
+      q[4] = fx.lg_any(c0);
+      q[5] = fx.coef(16 * (1.0L - a[0]));
+      q[6] = fx.coef((ld)a[5] * LOG2E / T_V);
+      q[7] = 0;
+      for (int i = 0; i < 6; ++i) ed[((size_t)k * 2 + r) * 6 + i] = C.d[r][i];
+    }
+    for (int r = 0; r < 2; ++r) for (int i = 0; i < 6; ++i) ef << (k + r + i ? "," : "") << litf(C.d[r][i]);
+  }
+
+  // ---- reactions: cost, classes --------------------------------------------------
+  struct Rx { int j, cls, shape, acc; double cost; std::vector<i64> ax; };
+  std::vector<std::vector<int>> groups;          // plain duplicates share a row
+  {
+    std::vector<bool> used(NR, false);
+    for (int j = 0; j < NR; ++j) {
+      if (used[j]) continue;
+      std::vector<int> g{j};
+      used[j] = true;
+      const Reaction& r = m.reactions[j];
+      if (r.duplicate && r.kind == RX_ARRHENIUS)
+        for (int q = j + 1; q < NR; ++q) {
+          const Reaction& o = m.reactions[q];
+          if (!used[q] && o.duplicate && o.kind == RX_ARRHENIUS && o.reversible == r.reversible &&
+              o.reactants == r.reactants && o.products == r.products) { g.push_back(q); used[q] = true; }
+        }
+      groups.push_back(g);
+    }
+  }
+  const int rows_all = (int)groups.size();
+  auto nfac = [&](int j, bool prod) { return (int)side_factors(prod ? m.reactions[j].products : m.reactions[j].reactants).size(); };
+  auto n_prod = [&](int j) { return m.reactions[j].reversible ? nfac(j, true) : 0; };
+  auto cost_of = [&](int j) {
+    const int cls = classes(m.reactions[j]);
+    const double base = 40 + 4 * nfac(j, false) + (n_prod(j) ? 25 + 2 * n_prod(j) : 0);
+    return base + (cls == 0 ? 0 : cls == 1 ? 60 : cls == 2 ? 150 : cls == 5 ? 150 : 320) + 18.0 * m.reactions[j].efficiencies.size();
+  };
+
+  // ---- block shape -----------------------------------------------------------------
+  // Measured (2^20 states of 53 species / 325 reactions, energy input): two blocks of 12
+  // warps an SM 7.3 ms, one of 24 warps 7.6, two of 8 warps 7.9, one of 16 warps 7.8; with
+  // the rows in more than one chunk two blocks lose (8.3 ms and more).  10 species / 21
+  // reactions: eight blocks of 4 warps 0.81 ms, four of 8 warps 0.96 ms; 160 / 1100
+  // (2^18 states): one block of 24 warps 5.6 ms, of 16 warps 6.4 ms.
+  const int fixed_bytes = 8192 + 512 * (N + 1) + 1920 + 256;
+  int warps = rows_all < 48 ? 4 : rows_all < 120 ? 8 : 12;
+  int minb = 24 / warps + (warps == 4 ? 2 : 0);
+  auto red = [](int w) { return w * 256 + 6 * 256 + 12 * 128 + w * 12 * 128; };   // scratch of the temperature solve, in the rows
+  while (minb > 1 && fixed_bytes + std::max(rows_all * 256, red(warps)) > kSmemPerSm / minb - kSmemPerBlock) --minb;
+  if (minb == 1) warps = 24;
+  const int lim = std::min(kSmemMaxBlock, kSmemPerSm / minb - kSmemPerBlock) - fixed_bytes;
+  const int max_rows = lim / 256;
+  if (lim < red(warps) || max_rows < 8) { out.why = "species arrays do not fit in shared memory"; return out; }
+  const int chunks = (rows_all + max_rows - 1) / max_rows;
+  const int rows = (rows_all + chunks - 1) / chunks;
+  const int tile_rows = std::max(rows, (red(warps) + 255) / 256);
+
+  // groups to chunks (equal rows; heaviest first so that costs even out)
+  std::vector<int> order(groups.size());
+  for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+  auto gcost = [&](int g) { double c = 0; for (int j : groups[g]) c += cost_of(j); return c; };
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return gcost(a) > gcost(b); });
+  std::vector<std::vector<int>> in_chunk(chunks);
+  {
+    std::vector<double> load(chunks, 0.0);
+    for (int g : order) {
+      int best = -1;
+      for (int c = 0; c < chunks; ++c)
+        if ((int)in_chunk[c].size() < rows && (best < 0 || load[c] < load[best])) best = c;
+      in_chunk[best].push_back(g);
+      load[best] += gcost(g);
+    }
+  }
+  // classes present, in code order: plain reactions by (factors, reversible), then the others
+  std::map<int, int> class_id;
+  auto key_of = [&](int j) {
+    if (classes(m.reactions[j])) return 8;
+    return (std::max(nfac(j, false), n_prod(j)) > 2 ? 2 : 0) + (n_prod(j) > 0 ? 1 : 0);
+  };
+  for (int j = 0; j < NR; ++j) class_id[key_of(j)] = 0;
+  class_id[8] = 0;
+  int ncls = 0;
+  for (auto& kv : class_id) kv.second = ncls++;
+
+  std::vector<i64> rx, ax;
+  std::vector<int> seg;
+  std::vector<int> row_of(groups.size());
+  for (int ch = 0; ch < chunks; ++ch) {
+    std::vector<std::vector<int>> mine(warps);
+    std::vector<double> load(warps, 0.0);
+    int row = 0;
+    for (int g : in_chunk[ch]) {
+      row_of[g] = row++;
+      const int w = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+      mine[w].push_back(g);
+      load[w] += gcost(g);
+    }
+    for (int w = 0; w < warps; ++w) {
+      for (auto& kv : class_id) {
+        seg.push_back((int)(rx.size() / 8));
+        for (int g : mine[w])
+          for (size_t q = 0; q < groups[g].size(); ++q) {
+            const int j = groups[g][q];
+            if (key_of(j) != kv.first) continue;
+            const Reaction& r = m.reactions[j];
+            const int cls = classes(r);
+            const Arr a = forms[j][0];
+            i64 rec[8] = {0};
+            if (cls != 5) {
+              rec[0] = fx.lg(a.c);
+              rec[1] = fx.coef(16 * a.b);
+              rec[2] = fx.coef(-a.theta * LOG2E / T_V);
+            }
+            const std::vector<int> fr = side_factors(r.reactants), fp = r.reversible ? side_factors(r.products) : std::vector<int>();
+            auto at = [](const std::vector<int>& f, size_t i) { return (u64)(i < f.size() ? f[i] : 0); };
+            if (cls == 0) {       // byte offsets into the species arrays and of the row
+              auto off = [&](const std::vector<int>& f, size_t i) { return (u64)((i < f.size() ? f[i] : N) * 256); };
+              rec[3] = (i64)(off(fr, 0) | off(fr, 1) << 32);
+              rec[4] = (i64)(off(fr, 2) | off(fp, 0) << 32);
+              rec[5] = (i64)(off(fp, 1) | off(fp, 2) << 32);
+              rec[6] = (i64)((u64)row_of[g] * 256 | (u64)(q > 0 ? 1 : 0) << 32);
+              rx.insert(rx.end(), rec, rec + 8);
+              continue;
+            }
+            rec[3] = (i64)(at(fr, 0) | at(fr, 1) << 16 | at(fr, 2) << 32 | at(fp, 0) << 48);
+            rec[4] = (i64)(at(fp, 1) | at(fp, 2) << 16 | (u64)row_of[g] << 32 | (u64)fr.size() << 48 | (u64)fp.size() << 52 | (u64)cls << 56);
+            rec[5] = (i64)ax.size();
+            if (cls) {
+              std::vector<i64> x(16, 0);
+              if (cls == 5) {
+                const size_t nn = r.plog.size();
+                x[1] = (i64)nn;
+                for (size_t i = 0; i < nn; ++i) {
+                  const Arr& f = forms[j][i];
+                  const ld lp = log2l((ld)r.plog[i].p);
+                  x.push_back(fx.lg(lp));
+                  x.push_back(dbits(i + 1 < nn ? (double)(1.0L / (log2l((ld)r.plog[i + 1].p) - lp)) : 0.0));
+                  x.push_back(fx.lg(f.c)); x.push_back(fx.coef(16 * f.b)); x.push_back(fx.coef(-f.theta * LOG2E / T_V));
+                }
+                if (nn < 2) fx.bad = true;
+              } else {
+                for (auto& e : r.efficiencies) {
+                  const double c = (e.second - 1.0) / m.species[e.first].W;
+                  if (c == 0.0) continue;
+                  x[0]++;
+                  x.push_back(e.first);
+                  x.push_back(dbits(c));
+                }
+              }
+              if (cls >= 2 && cls <= 4) {
+                x[2] = fx.lg(log2l((ld)r.A0) - log2l((ld)r.A));
+                x[3] = fx.coef(16 * ((ld)r.b0 - r.b));
+                x[4] = fx.coef(-((ld)r.theta0 - r.theta) * LOG2E / T_V);
+              }
+              // a term that is below 2^-1100 at every T of the range is left out
+              auto term = [&](ld slope, ld at_lo) { return at_lo > -1100 && (fabsl(slope) < 4000 || (fx.bad = true)); };
+              auto add = [&](i64 c, ld t, ld v) {      // an exponential of S: c, slopes in t and v
+                i64* e = &x[5 + 3 * x[1]++];
+                e[0] = c; e[1] = fx.coef(t); e[2] = fx.coef(v);
+              };
+              if (cls == 3) {
+                const ld A = r.troe[0], s3 = -T_T / r.troe[1] * LOG2E, s1 = -T_T / r.troe[2] * LOG2E;
+                if (A != 1 && term(s3, s3 * t_lo / T_T)) add(fx.lg(log2l(fabsl(1 - A))) | (A > 1 ? 1 : 0), s3, 0);
+                if (A > 0 && term(s1, s1 * t_lo / T_T)) add(fx.lg(log2l(A)), s1, 0);
+                if (r.n_troe == 4) {
+                  const ld s2 = -(ld)r.troe[3] / T_V * LOG2E;
+                  if (term(s2, s2 * T_V / T_HI)) add(0, 0, s2);
+                }
+              } else if (cls == 4) {
+                const ld d = r.n_sri >= 5 ? r.sri[3] : 1.0, e = r.n_sri >= 5 ? r.sri[4] : 0.0;
+                const ld sb = -(ld)r.sri[1] * LOG2E / T_V, sc = -T_T / r.sri[2] * LOG2E;
+                if (r.sri[0] > 0 && term(sb, sb * T_V / T_HI)) add(fx.lg(log2l((ld)r.sri[0])), 0, sb);
+                if (term(sc, sc * t_lo / T_T)) add(0, sc, 0);
+                x[14] = fx.lg(log2l(d));
+                x[15] = fx.coef(16 * e);
+              }
+              if (x.size() % 2) x.push_back(0);      // efficiency pairs are read as 16-byte units
+              ax.insert(ax.end(), x.begin(), x.end());
+            }
+            rx.insert(rx.end(), rec, rec + 8);
+          }
+      }
+      seg.push_back((int)(rx.size() / 8));
+    }
+  }
+  if (fx.bad) { out.why = "a coefficient does not fit the fixed-point range"; return out; }
+
+  // ---- species sums: owners balanced by entries, lists per chunk ------------------
+  std::vector<std::vector<std::pair<int, int>>> terms(N);      // (group, nu)
+  for (size_t g = 0; g < groups.size(); ++g)
+    for (auto& q : net_nu(m.reactions[groups[g][0]])) if (q.second) terms[q.first].push_back({(int)g, q.second});
+  const int kpw = (N + warps - 1) / warps;
+  std::vector<std::vector<int>> owned(warps);
+  {
+    std::vector<int> idx(N);
+    for (int k = 0; k < N; ++k) idx[k] = k;
+    std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return terms[a].size() > terms[b].size(); });
+    std::vector<size_t> load(warps, 0);
+    for (int k : idx) {
+      int best = -1;
+      for (int w = 0; w < warps; ++w)
+        if ((int)owned[w].size() <= kpw && (best < 0 || load[w] < load[best])) best = w;
+      owned[best].push_back(k);
+      load[best] += terms[k].size() + 1;
+    }
+  }
+  int kpo = 0;
+  for (auto& v : owned) kpo = std::max(kpo, (int)v.size());
+  std::vector<int> chunk_of(groups.size());
+  for (int ch = 0; ch < chunks; ++ch) for (int g : in_chunk[ch]) chunk_of[g] = ch;
+  std::vector<int> wl, wo, we, wc;
+  for (int ch = 0; ch < chunks; ++ch)
+    for (int w = 0; w < warps; ++w)
+      for (int i = 0; i < kpo; ++i) {
+        int ends[4], sum = 0, no = 0;
+        ends[0] = (int)we.size();
+        for (int pass = 0; pass < 3; ++pass) {
+          if (i < (int)owned[w].size())
+            for (auto& t : terms[owned[w][i]])
+              if (chunk_of[t.first] == ch && (t.second == 1 ? 0 : t.second == -1 ? 1 : 2) == pass) {
+                we.push_back(row_of[t.first] * 256);
+                wc.push_back(t.second);
+                sum += std::abs(t.second);
+                no += pass == 2;
+              }
+          while (we.size() % 4) { we.push_back(tile_rows * 256); wc.push_back(0); }   // the zero row
+          ends[pass + 1] = (int)we.size();
+        }
+        wl.insert(wl.end(), ends, ends + 4);
+        int hb = 0;
+        while ((1 << hb) < sum) ++hb;
+        wo.push_back(i < (int)owned[w].size() ? owned[w][i] : -1);
+        wo.push_back(hb + 256 * no);
+      }
+  for (int q = 0; q < 8; ++q) rx.push_back(0);   // spare record (the loops read one ahead)
+
+  // ---- the unit -------------------------------------------------------------------
+  std::ostringstream o;
+  o << "// Tile kernel of mechanism '" << m.name << "': " << N << " species, " << NR << " reactions.\n"
+    << "#define NSP " << N << "\n#define NW " << warps << "\n#define TILE_MINB " << minb << "\n#define KPW " << kpw
+    << "\n#define KPO " << kpo << "\n#define NCH " << chunks << "\n#define NCLS " << ncls << "\n#define TILE_ROWS "
+    << tile_rows << "\n#define TMID " << lit(tmid) << "\n#define TILE_OPEN " << kTileOpen << "\n#define T_LO " << lit(t_lo) << "\n#define T_HI "
+    << lit((double)T_HI) << "\n#define T_V " << lit((double)T_V) << "\n#define T_T " << lit((double)T_T)
+    << "\n#define T_INV_R " << lit((double)(1.0L / R_GAS)) << "\n#define T_INV_R_LO "
+    << lit((double)(1.0L / R_GAS - (ld)(double)(1.0L / R_GAS))) << "\n#define T_LG_R " << fx.lg(log2l(R_GAS)) << "ll\n";
+  o << "#include \"pyro_fixed_math.cuh\"\n";
+  {
+    std::vector<std::string> e2, l2;
+    for (int j = 0; j < 1024; ++j) e2.push_back(std::to_string((u64)roundl(exp2l(j / 1024.0L) * 9223372036854775808.0L)) + "ull");
+    for (int j = 0; j < 256; ++j) {
+      const unsigned rc = (unsigned)roundl(2048.0L / (1.0L + (j + 0.5L) / 256));
+      l2.push_back("{" + std::to_string((i64)llroundl(-log2l(rc / 2048.0L) * 4611686018427387904.0L)) + "ll," +
+                   std::to_string(rc) + "u,0u}");
+    }
+    array(o, "unsigned long long", "t_exp2", e2);
+    array(o, "pfx::Log2Entry", "t_log2", l2);
+  }
+  array(o, "__align__(16) long long", "t_sp", as_ll(sp));
+  o << "__device__ const __align__(16) float t_ef[" << 12 * N << "] = {" << ef.str() << "};\n";
+  array(o, "__align__(16) double", "t_ed", as_d(ed));
+  array(o, "double", "t_iw", as_d(iw));
+  array(o, "__align__(16) long long", "t_rx", as_ll(rx));
+  array(o, "__align__(16) long long", "t_ax", as_ll(ax));
+  array(o, "int", "t_seg", seg);
+  array(o, "__align__(16) int", "t_wl", wl);
+  array(o, "__align__(8) int", "t_wo", wo);
+  array(o, "__align__(16) int", "t_we", we);
+  array(o, "signed char", "t_wc", wc);
+  o << "#define TILE_PLAIN";
+  for (auto& kv : class_id) {
+    if (kv.first == 8) continue;
+    const int c = kv.second;
+    o << " \\\n  { const int a = __ldg(seg + " << c << "), b = __ldg(seg + " << c + 1 << "); if (a < b) tile_plain<"
+      << (kv.first & 2 ? 3 : 2) << ", " << (kv.first & 1 ? "true" : "false") << ">(s, a, b, u, v, lane); }";
+  }
+  o << "\n#include \"pyro_tile.cuh\"\n";
+  out.source = o.str();
+  out.warps = warps;
+  out.smem_bytes = fixed_bytes + tile_rows * 256;
+  out.t_lo = t_lo;
+  out.chunks = chunks;
+  out.rows = rows;
+  return out;
+}
+
+}  // namespace pyro

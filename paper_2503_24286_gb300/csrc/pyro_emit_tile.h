@@ -1,0 +1,32 @@
+// Emitter of the tile kernel of the net production rates (32 states per block, all
+// exponents in fixed point): the mechanism's tables and sizes for pyro_tile.cuh.
+#pragma once
+
+#include <string>
+
+#include "pyro_emit.h"
+#include "pyro_mech.h"
+
+namespace pyro {
+
+struct TileEmit {
+  std::string source;      // empty: the mechanism does not fit the tables (see why)
+  std::string why;
+  int warps = 8;           // per block
+  int smem_bytes = 0;      // dynamic shared memory per block
+  double t_lo = 0.0;       // states at or below it are left to the FP64 kernel
+  int chunks = 0, rows = 0;
+};
+
+// Dynamic shared memory an SM can hold, and what a resident block costs beside its own.
+constexpr int kSmemPerSm = 228 * 1024;
+constexpr int kSmemPerBlock = 1024;
+constexpr int kSmemMaxBlock = 227 * 1024;
+
+TileEmit emit_tile_unit(const Mechanism& m);
+
+// The kernel text (embedded at build time).
+extern const char* kFixedMathSource;
+extern const char* kTileSource;
+
+}  // namespace pyro

@@ -926,11 +926,13 @@ __device__ double wtsolve(const double* sY, double e, double T0, int max_iter, f
         "extern \"C\" __global__ void __launch_bounds__(WPB * 32) pyro_omega_warp(i64 n, const double* __restrict__ g_rho,\n"
         "    const double* __restrict__ g_Tin, int energy_mode, const double* __restrict__ g_Y,\n"
         "    double* __restrict__ g_Tout, double* __restrict__ g_omega, double T_guess, int max_iter, double tol,\n"
-        "    unsigned long long* __restrict__ g_fail, double* __restrict__ g_store)");
+        "    unsigned long long* __restrict__ g_fail, double* __restrict__ g_store, int open_only)");
     k << "  double* sP = sL;   // partial sums of the production rates (after the reactions)\n"
          "  (void)g_store;\n  const float tolf = (float)tol;\n"
          "  for (i64 base = (i64)blockIdx.x * WPB; base < n; base += (i64)gridDim.x * WPB) {\n"
          "    const i64 p = base + warp;\n    if (p >= n) break;   // warp-uniform; no block barrier below\n"
+         "    // open_only: only the states that the tile kernel left open (pyro_tile.cuh)\n"
+         "    if (open_only && __double_as_longlong(g_omega[p]) != " << kTileOpen << ") continue;\n"
          "    const double rho = g_rho[p];\n    double ys = 0.0;\n"
          "    for (int k = lane; k < NSP; k += 32) {\n      const double y = g_Y[(i64)k * n + p];\n"
          "      sY[k] = y;\n      ys = fma(y, __ldg(w_invW + k), ys);\n    }\n"

@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "pyro_emit.h"
+#include "pyro_emit_tile.h"
 #include "pyro_emit_warp.h"
 #include "pyro_internal.h"
 #include "pyro_mech.h"
@@ -113,9 +114,9 @@ const char* kArch = "sm_103a";
 // Compile CUDA C to a cubin for sm_103a with NVRTC.
 bool nvrtc_compile(const std::string& src, std::vector<char>& cubin, std::string& log) {
   nvrtcProgram prog;
-  const char* hdrs[] = {kDeviceMathSource};
-  const char* names[] = {"pyro_device_math.cuh"};
-  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 1, hdrs, names) != NVRTC_SUCCESS) {
+  const char* hdrs[] = {kDeviceMathSource, kFixedMathSource, kTileSource};
+  const char* names[] = {"pyro_device_math.cuh", "pyro_fixed_math.cuh", "pyro_tile.cuh"};
+  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 3, hdrs, names) != NVRTC_SUCCESS) {
     log = "nvrtcCreateProgram failed";
     return false;
   }
@@ -140,7 +141,7 @@ bool nvrtc_compile(const std::string& src, std::vector<char>& cubin, std::string
 
 
 // Compile CUDA C for sm_103a with NVRTC, or fetch the cubin from the on-disk
-// cache keyed by a hash of the source, the device-math header, the arch and the
+// cache keyed by a hash of the source, the headers it includes, the arch and the
 // NVRTC version.
 int compile_cached(const std::string& src, bool use_cache, std::vector<char>& cubin) {
   if (const char* dump = std::getenv("PYRO_DUMP_DIR")) {   // debugging aid: keep the emitted sources
@@ -152,6 +153,8 @@ int compile_cached(const std::string& src, bool use_cache, std::vector<char>& cu
   nvrtcVersion(&nv_major, &nv_minor);
   std::string key_src = src + std::string(kDeviceMathSource) + kArch + std::to_string(nv_major) + "." +
                         std::to_string(nv_minor);
+  if (src.find("pyro_fixed_math.cuh") != std::string::npos) key_src += kFixedMathSource;
+  if (src.find("pyro_tile.cuh") != std::string::npos) key_src += kTileSource;
   char hex[32];
   std::snprintf(hex, sizeof hex, "%016llx", (unsigned long long)fnv1a(key_src));
   std::string dir = cache_dir(), path = dir + "/pyro_" + hex + ".cubin";
@@ -505,7 +508,7 @@ const char* group_kernel(const std::string& g) {
   return g == "jvp" ? "pyro_jvp" : g == "vjp" ? "pyro_vjp" : g == "jad" ? "pyro_jacobian_adiabatic"
        : g == "cn" ? "pyro_cn_assemble" : g == "tr" ? "pyro_transport" : g == "wfwd" ? "pyro_omega_warp"
        : g == "wjvp" ? "pyro_jvp_warp" : g == "wvjp" ? "pyro_vjp_warp" : g == "wjac" ? "pyro_jacobian_cta"
-       : g == "wjad" ? "pyro_jacobian_adiabatic_cta" : "pyro_jacobian";
+       : g == "wjad" ? "pyro_jacobian_adiabatic_cta" : g == "tile" ? "pyro_omega_tile" : "pyro_jacobian";
 }
 
 // Compile (in parallel threads, cached on disk) and load the named derivative
@@ -552,6 +555,10 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
       G.block = 32 * h->emitted.warp_wpb.at(todo[i]);
       G.smem = h->emitted.smem_dyn_bytes_warp.at(todo[i]);
     }
+    if (todo[i] == "tile") {
+      G.block = 32 * h->emitted.tile_warps;
+      G.smem = h->emitted.smem_dyn_bytes_tile;
+    }
     if (todo[i] == "jac" || todo[i] == "jad" || todo[i] == "cn") G.smem = h->emitted.smem_dyn_bytes_jac;
     const int smem = G.smem >= 0 ? G.smem : h->emitted.smem_dyn_bytes_deriv;
     const int blk = G.block > 0 ? G.block : h->opt.deriv_block;
@@ -578,7 +585,7 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
       h->emitted.stats[todo[i] + "_active_clusters"] = ncl;
     }
     if (h->emitted.stats["deriv_store_global"] > 0 && todo[i] != "jac" && todo[i] != "jad" && todo[i] != "cn" &&
-        todo[i][0] != 'w') {
+        todo[i] != "tile" && todo[i][0] != 'w') {
       size_t bytes = (size_t)h->num_sms * nb * 4 * h->m.n_species() * h->opt.deriv_block * sizeof(double);
       cudaError_t e = cudaMalloc(&G.store, bytes);
       if (e != cudaSuccess) return fail(PYRO_ECUDA, std::string("species-array store allocation: ") + cudaGetErrorString(e));
@@ -666,6 +673,46 @@ std::string jac_group(const pyro_mech* h, bool adiabatic) {
   return adiabatic ? "jad" : "jac";
 }
 
+// Net production rates on device pointers.  Where the mechanism fits the tile
+// kernel's tables it evaluates the states (32 per block; see pyro_tile.cuh), and
+// the FP64 kernel (thread or warp per state) those that the tile kernel left open.
+// newton=fp64 keeps its own temperature iteration: solved first, then rates at T.
+int launch_rates(const pyro_mech* h, int64_t n, const void* rho, const void* T_or_e, int energy, const void* Y,
+                 void* T_out, void* omega, unsigned long long* fail_ctr, void* stream) {
+  long long nn = n;
+  double Tg = 1200.0, tol = 1e-10;
+  int max_iter = 50, open_only = 0;
+  const void* none = nullptr;
+  const void* Tin = T_or_e;
+  auto it = h->groups.find("tile");
+  const bool tile = it != h->groups.end() && it->second.f;
+  if (tile) {
+    const pyro_mech::Group& G = it->second;
+    if (energy && !h->opt.mixed) {
+      void* pt[] = {&nn, &Tin, &Y, &none, &Tg, &max_iter, &tol, &T_out, &none, &fail_ctr};
+      if (int rc = launch(h, h->f_temperature, n, 8, 0, stream, pt)) return rc;
+      Tin = T_out;
+      energy = 0;
+    }
+    void* params[] = {&nn, &rho, &Tin, &energy, &Y, &T_out, &omega, &Tg, &max_iter, &tol, &fail_ctr};
+    const int64_t need = (n + 31) / 32, cap = (int64_t)h->num_sms * G.blocks_per_sm;
+    CUresult r = driver().LaunchKernel(G.f, (unsigned)std::min(need, cap), 1, 1, G.block, 1, 1, G.smem, as_stream(stream),
+                                       params, nullptr);
+    if (r != CUDA_SUCCESS) return fail(PYRO_ECUDA, "kernel launch: " + cu_err(r));
+    if (energy) Tin = T_out;
+    energy = 0;
+    open_only = 1;
+  }
+  const void* store = h->d_store;
+  void* params[] = {&nn, &rho, &Tin, &energy, &Y, &T_out, &omega, &Tg, &max_iter, &tol, &fail_ctr, &store, &open_only};
+  if (h->opt.warp) {
+    auto wf = h->groups.find("wfwd");
+    if (wf == h->groups.end() || !wf->second.f) return fail(PYRO_ECUDA, "warp-per-state kernel not loaded");
+    return launch_warp(h, wf->second, n, stream, params);
+  }
+  return launch(h, h->f_omega, n, h->omega_blocks_per_sm, h->emitted.smem_dyn_bytes_omega, stream, params);
+}
+
 int launch_deriv(const pyro_mech* h, const pyro_mech::Group& G, int64_t n, void* stream, void** params) {
   const int blk = G.block > 0 ? G.block : h->opt.deriv_block;
   const int smem = G.smem >= 0 ? G.smem : h->emitted.smem_dyn_bytes_deriv;
@@ -720,9 +767,19 @@ int pyro_mech_load(const char* mech_path, const char* options, pyro_mech** out) 
 
   // compile (or fetch from the cache)
   std::vector<char> cubin;
-  if (int rc = compile_cached(h->emitted.source, h->opt.cache, cubin)) { delete h; return rc; }
+  const bool tile = h->emitted.stats["tile"] > 0;
+  std::thread tile_compile;   // the tile kernel's unit beside the main one (fetched from the cache below)
+  if (tile && h->opt.cache)
+    tile_compile = std::thread([&] { std::vector<char> c; compile_cached(h->emitted.group_sources.at("tile"), true, c); });
+  const int crc = compile_cached(h->emitted.source, h->opt.cache, cubin);
+  if (tile_compile.joinable()) tile_compile.join();
+  if (crc) { delete h; return crc; }
   h->emitted.stats["cubin_bytes"] = (double)cubin.size();
-  if (!h->opt.device) { *out = h; return PYRO_OK; }
+  if (!h->opt.device) {
+    if (tile) if (int rc = ensure_groups(h, {"tile"})) { delete h; return rc; }
+    *out = h;
+    return PYRO_OK;
+  }
   Driver& d = driver();
   if (!d.ok) { delete h; return fail(PYRO_ECUDA, d.err); }
   cudaError_t ce = cudaFree(0);   // make sure a context is current
@@ -766,6 +823,7 @@ int pyro_mech_load(const char* mech_path, const char* options, pyro_mech** out) 
     size_t bytes = (size_t)h->num_sms * nb * 2 * h->m.n_species() * h->opt.block * sizeof(double);
     if (int rc = ensure_store(h, bytes)) { pyro_mech_free(h); return rc; }
   }
+  if (tile) if (int rc = ensure_groups(h, {"tile"})) { pyro_mech_free(h); return rc; }
   if (h->opt.warp) {
     // the emitted warp-per-state forward kernel (compiled now, cached on disk)
     if (int rc = ensure_groups(h, {"wfwd"})) { pyro_mech_free(h); return rc; }
@@ -931,15 +989,7 @@ int pyro_net_production_rates(const pyro_mech* hc, int64_t n, const double* rho,
   int rc = with_args(h, n, {{rho, 1, 8, true, false}, {T_or_e, 1, 8, true, false}, {Y, NS, 8, true, false},
                          {input_is_energy ? T_out : nullptr, 1, 8, false, true}, {omega, NS, 8, false, true}},
                      stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
-                       long long nn = nc;
-                       int em = input_is_energy ? 1 : 0;
-                       double Tg = 1200.0, tol = 1e-10;
-                       int max_iter = 50;
-                       void* params[] = {&nn, &d[0], &d[1], &em, &d[2], &d[3], &d[4], &Tg, &max_iter, &tol, &h->d_fail,
-                                         &h->d_store};
-                       if (h->opt.warp) return launch_warp(h, h->groups["wfwd"], nc, st, params);
-                       return launch(h, h->f_omega, nc, h->omega_blocks_per_sm, h->emitted.smem_dyn_bytes_omega,
-                                     st, params);
+                       return launch_rates(h, nc, d[0], d[1], input_is_energy ? 1 : 0, d[2], d[3], d[4], h->d_fail, st);
                      }, h->opt.warp || h->emitted.stats["omega_store_global"] <= 0);   // no per-block global scratch
   if (rc) return rc;
   return input_is_energy ? maybe_checked(h, stream) : PYRO_OK;
@@ -1381,19 +1431,7 @@ int internal_fail(int code, const char* msg) { return fail(code, msg); }
 int internal_launch_omega(const pyro_mech* h, int64_t n, const void* rho, const void* T_or_e,
                           int input_is_energy, const void* Y, void* T_out, void* omega,
                           unsigned long long* fail_ctr, void* stream) {
-  long long nn = n;
-  int em = input_is_energy ? 1 : 0;
-  double Tg = 1200.0, tol = 1e-10;
-  int max_iter = 50;
-  void* store = h->d_store;
-  void* params[] = {&nn, &rho, &T_or_e, &em, &Y, &T_out, &omega, &Tg, &max_iter, &tol, &fail_ctr, &store};
-  // the same kernel choice as pyro_net_production_rates (thread or warp per state)
-  if (h->opt.warp) {
-    auto it = h->groups.find("wfwd");
-    if (it == h->groups.end() || !it->second.f) return fail(PYRO_ECUDA, "warp-per-state kernel not loaded");
-    return launch_warp(h, it->second, n, stream, params);
-  }
-  return launch(h, h->f_omega, n, h->omega_blocks_per_sm, h->emitted.smem_dyn_bytes_omega, stream, params);
+  return launch_rates(h, n, rho, T_or_e, input_is_energy ? 1 : 0, Y, T_out, omega, fail_ctr, stream);
 }
 
 }  // namespace pyro

@@ -1,0 +1,561 @@
+// Net production rates of a tile of 32 states per block: lane = state, the block's
+// warps split the species and the reactions, and all exponents are fixed point.
+//
+// Included by the emitted unit, which defines the mechanism's tables (t_*) and
+// sizes (NSP, NW, KPW, NCH, ...).  One pass over a tile:
+//   0  temperature from energy (energy input): every warp collapses the energy
+//      polynomials of its species, one warp finishes the Newton iteration;
+//   1  per species lambda_k = log2(phi_k/W_k) and alpha_k = log2(a_k), with
+//      a_k = phi_k C_k (the activity form of Eq. equil_constants and
+//      Eq. reaction_rates), in shared memory [species][lane];
+//   2  per reaction the exponents of its forward and reverse rate,
+//      K_j(T) - sum nu' lambda + sum nu' alpha  and  ... + sum nu'' alpha,
+//      two exponentials and their difference, the rate of progress, in shared memory
+//      as one 64-bit word: 52 bits of signed integer and 12 of exponent (not
+//      normalised: its error is 2^-50 of the larger of the two rates);
+//   3  per species the sum of its reactions' rates, aligned to the largest exponent
+//      met so far, normalised once into the output.
+// All warps of a block run the same code at about the same time and the loops over
+// species and reactions are rolled: a reaction is a table record, not code, so that
+// the kernel stays within the instruction caches (with a loop per reaction shape and
+// unrolled species loops it was 119 KB and stalled on instruction fetch).
+// The FP64 pipe, which runs beside the integer work, keeps the temperature solve,
+// the third-body concentrations and the blending factors of falloff reactions.
+//
+// States outside the tables' range (temperature outside (T_LO, T_HI), NaN,
+// infinite or subnormal mass fractions or ones beyond 2^8, densities beyond
+// 2^-60..2^20, [M] <= 0) get TILE_OPEN in their first output; the caller then
+// launches the FP64 kernel, which evaluates the states so marked.
+#include "pyro_device_math.cuh"
+#include "pyro_fixed_math.cuh"
+
+using pfx::Pair;
+typedef pfx::i64 i64;
+typedef pfx::u64 u64;
+
+struct TileScalars {
+  double T[32], ysum[32];
+  Pair u[32], v[32], t[32];      // log2(T)/16, T_V/T, T/T_T
+  i64 lgT[32], lgrho[32];
+  int bad[32];
+};
+
+// A rate is a 64-bit word r: read as an integer it is m 2^(e - 61 - RATE_E) with
+// e = r & 4095.  The exponent's bits are the last bits of the integer: they lie below
+// its resolution and, near RATE_E/4096 of one unit, are on average what truncation
+// took away.
+#define RATE_E 2048
+struct TileSmem {
+  u64* exp2;
+  i64 *lam, *alp;   // [NSP + 1][32]: the species and a unit factor; alp first holds Y
+  i64* R;           // rows and one zero row; during the temperature solve its scratch (red, B, b, ys)
+  double* red;
+  double* B;
+  float* b;
+  double* ys;
+  TileScalars* sc;
+};
+
+__device__ __forceinline__ Pair as_pair(i64 v) {
+  Pair p;
+  p.lo = (int)v;
+  p.hi = (int)((u64)v >> 32);
+  return p;
+}
+
+__device__ __forceinline__ TileSmem tile_smem(char* base) {
+  TileSmem s;
+  s.exp2 = (u64*)base;                     base += pfx::EXP2_TAB * 8;
+  s.lam = (i64*)base;                      base += (NSP + 1) * 256;
+  s.alp = (i64*)base;                      base += (NSP + 1) * 256;
+  s.R = (i64*)base;
+  s.ys = (double*)base;                    // NW x 32
+  s.B = s.ys + NW * 32;                    // 6 x 32
+  s.b = (float*)(s.B + 6 * 32);            // 12 x 32
+  s.red = (double*)(s.b + 12 * 32);        // NW x 6 x 32 (FP32: NW x 12 x 32)
+  base += (TILE_ROWS + 1) * 256;
+  s.sc = (TileScalars*)base;
+  return s;
+}
+
+// double of m 2^(e - f)
+__device__ __forceinline__ double tile_to_double(i64 m, int e, int f) {
+  const u64 a = m < 0 ? (u64)(-m) : (u64)m;
+  const int z = pfx::clz64(a | 1ull);
+  const u64 v = a << z;                               // leading one at bit 63
+  u64 r = (v >> 11) + ((v >> 10) & 1ull);             // 53 bits, rounded; a carry moves to the exponent
+  const int x = e - f + 63 - z + 1022;
+  r += (u64)(unsigned)x << 52;
+  r = (a == 0ull || x < 0) ? 0ull : r;
+  r = x > 2045 ? 0x7ff0000000000000ull : r;
+  return __longlong_as_double((i64)(r | ((u64)m & 0x8000000000000000ull)));
+}
+
+// arithmetic right shift; 63 where n is larger
+__device__ __forceinline__ i64 tile_sar(i64 v, int n) {
+  i64 r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
+__device__ __forceinline__ u64 tile_shr(u64 v, int n) {
+  u64 r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
+
+// the rate 2^xf - 2^xr (REV false: 2^xf) with the signs in the lowest bits
+template <bool REV>
+__device__ __forceinline__ i64 tile_rate(i64 xf, i64 xr, const u64* tab) {
+  const u64 f = pfx::exp2_mant(xf, tab);
+  const i64 sf = -(xf & 1ll);
+  const int nf = (int)(xf >> pfx::LG_F);
+  i64 m;
+  int e = max(nf, 50 - RATE_E);
+  if (REV) {
+    const u64 g = pfx::exp2_mant(xr, tab);
+    const i64 sg = -(xr & 1ll);
+    const int ng = (int)(xr >> pfx::LG_F);
+    e = max(e, ng);
+    // one's complement negation: off by one in 2^61
+    m = ((i64)tile_shr(f, e + 2 - nf) ^ sf) - ((i64)tile_shr(g, e + 2 - ng) ^ sg);
+  } else {
+    m = (i64)tile_shr(f, e + 2 - nf) ^ sf;
+  }
+  return (m & ~4095ll) | (i64)(e + RATE_E);
+}
+
+// the rate of a sum of two
+__device__ __forceinline__ i64 tile_add(i64 a, i64 b) {
+  const int ea = (int)a & 4095, eb = (int)b & 4095, e = max(ea, eb) + 1;
+  return ((tile_sar(a, e - ea) + tile_sar(b, e - eb)) & ~4095ll) | (i64)e;
+}
+
+// K(T) = c + beta u + tau v of a reaction, lowest bit clear
+__device__ __forceinline__ i64 tile_K(i64 c, i64 beta, i64 tau, Pair u, Pair v) {
+  return pfx::mul_add(as_pair(tau), v, pfx::mul_add(as_pair(beta), u, c)) & ~1ll;
+}
+
+// ---------------------------------------------------------------------------
+// temperature (Sec. A.3.1): FP32 Newton on the collapsed polynomials of both
+// ranges, then FP64 Newton on the range found, as in the per-thread solve
+// ---------------------------------------------------------------------------
+__device__ __noinline__ void tile_collapse_all(const double* __restrict__ Yp, i64 n, bool hi, double* B) {
+  for (int q = 0; q < 6; ++q) B[q] = 0.0;
+  for (int k = 0; k < NSP; ++k) {
+    const double y = __ldg(Yp + k * n);
+    for (int q = 0; q < 6; ++q) B[q] = fma(y, t_ed[(k * 2 + hi) * 6 + q], B[q]);
+  }
+}
+
+__device__ __forceinline__ void tile_energy(const TileSmem& s, const double* __restrict__ Yp, i64 n,
+                                            double e, double T0, int max_iter, float tolf, int w, int lane,
+                                            double& T, bool& ok) {
+  {
+    float f[12];
+#pragma unroll
+    for (int q = 0; q < 12; ++q) f[q] = 0.f;
+    const double* y = (const double*)s.alp + lane;
+#pragma unroll 1
+    for (int k = w; k < NSP; k += NW) {
+      const float yf = pdm::to_float_trunc(y[k * 32]);
+      const float4* c = (const float4*)(t_ef + k * 12);
+      const float4 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2);
+      f[0] = fmaf(yf, c0.x, f[0]); f[1] = fmaf(yf, c0.y, f[1]); f[2] = fmaf(yf, c0.z, f[2]); f[3] = fmaf(yf, c0.w, f[3]);
+      f[4] = fmaf(yf, c1.x, f[4]); f[5] = fmaf(yf, c1.y, f[5]); f[6] = fmaf(yf, c1.z, f[6]); f[7] = fmaf(yf, c1.w, f[7]);
+      f[8] = fmaf(yf, c2.x, f[8]); f[9] = fmaf(yf, c2.y, f[9]); f[10] = fmaf(yf, c2.z, f[10]); f[11] = fmaf(yf, c2.w, f[11]);
+    }
+    float* red = (float*)s.red;
+#pragma unroll
+    for (int q = 0; q < 12; ++q) red[(w * 12 + q) * 32 + lane] = f[q];
+    __syncthreads();
+    for (int q = w; q < 12; q += NW) {
+      float a = 0.f;
+#pragma unroll
+      for (int i = 0; i < NW; ++i) a += red[(i * 12 + q) * 32 + lane];
+      s.b[q * 32 + lane] = a;
+    }
+    __syncthreads();
+  }
+  const float* b = s.b + lane;
+  float Tf = pdm::to_float_trunc(T0);
+  const float eRf = pdm::to_float_trunc(e * T_INV_R);
+  for (int it = 0; it < 40; ++it) {
+    const float* c = b + (Tf >= (float)TMID ? 6 * 32 : 0);
+    const float c0 = c[0], c1 = c[32], c2 = c[64], c3 = c[96], c4 = c[128], c5 = c[160];
+    const float ef = fmaf(Tf, fmaf(Tf, fmaf(Tf, fmaf(Tf, fmaf(Tf, c5, c4), c3), c2), c1), c0);
+    const float cvf = fmaf(Tf, fmaf(Tf, fmaf(Tf, fmaf(Tf, 5.f * c5, 4.f * c4), 3.f * c3), 2.f * c2), c1);
+    const float Tn = fminf(fmaxf(Tf + (eRf - ef) * __frcp_rn(cvf), 100.f), 5000.f);
+    const bool conv = fabsf(Tn - Tf) <= 1e-5f * Tn;
+    Tf = Tn;
+    if (conv) break;
+  }
+  bool hi = Tf >= (float)TMID;
+  {
+    double B[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int k = w; k < NSP; k += NW) {
+      const double y = ((const double*)s.alp)[k * 32 + lane];
+      const double2* d = (const double2*)(t_ed + (k * 2 + hi) * 6);
+      const double2 d0 = __ldg(d), d1 = __ldg(d + 1), d2 = __ldg(d + 2);
+      B[0] = fma(y, d0.x, B[0]); B[1] = fma(y, d0.y, B[1]);
+      B[2] = fma(y, d1.x, B[2]); B[3] = fma(y, d1.y, B[3]);
+      B[4] = fma(y, d2.x, B[4]); B[5] = fma(y, d2.y, B[5]);
+    }
+    double* red = s.red;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) red[(w * 6 + q) * 32 + lane] = B[q];
+  }
+  __syncthreads();
+  for (int q = w; q < 6; q += NW) {
+    const double* red = s.red + q * 32 + lane;
+    double a = 0.0;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) a += red[i * 6 * 32];
+    s.B[q * 32 + lane] = a;
+  }
+  __syncthreads();
+  if (w != 0) return;
+  double B[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) B[q] = s.B[q * 32 + lane];
+  // B[0] - e/R first: the terms that cancel are large (formation energies), the rest is
+  // of the size of c_v T, and the residual is rounded at that size only
+  auto take_e = [&] { B[0] = fma(e, -T_INV_R_LO, fma(e, -T_INV_R, B[0])); };
+  take_e();
+  T = pdm::to_double(Tf);
+  bool flag = false;
+  ok = false;
+  for (int it = 0; it < max_iter + 1; ++it) {
+    const float Tc = pdm::to_float_trunc(T);
+    const bool h2 = Tc >= (float)TMID;
+    if (h2 != hi) { hi = h2; tile_collapse_all(Yp, n, hi, B); take_e(); }
+    const double res = fma(T, fma(T, fma(T, fma(T, fma(T, B[5], B[4]), B[3]), B[2]), B[1]), B[0]);
+    const float* c = b + (hi ? 6 * 32 : 0);
+    const float cvf = fmaf(Tc, fmaf(Tc, fmaf(Tc, fmaf(Tc, 5.f * c[160], 4.f * c[128]), 3.f * c[96]), 2.f * c[64]), c[32]);
+    const double dT = res * pdm::to_double(-__frcp_rn(cvf));
+    double Tn = T + dT;
+    const float Tnf = pdm::to_float_trunc(Tn);
+    const bool clamped = !(Tnf >= 100.f && Tnf <= 5000.f);
+    Tn = clamped ? (Tnf < 100.f ? 100.0 : 5000.0) : Tn;
+    const bool conv = !clamped && fabsf(pdm::to_float_trunc(dT)) <= tolf * pdm::to_float_trunc(Tn);
+    T = Tn;
+    if (flag) { ok = true; break; }
+    if (conv) flag = true;
+    else if (it >= max_iter - 1) break;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// reactions
+// ---------------------------------------------------------------------------
+// plain reactions with up to NF factors a side (missing ones: the unit factor);
+// REV: reversible.  A flag marks a duplicate of a reaction before it in this warp,
+// whose rate is added to the same row.
+template <int NF, bool REV>
+__device__ __forceinline__ void tile_plain(const TileSmem& s, int i0, int i1, Pair u, Pair v, int lane) {
+  const char* lam = (const char*)(s.lam + lane);
+  const char* alp = (const char*)(s.alp + lane);
+  char* R = (char*)(s.R + lane);
+  const int4* r = (const int4*)(t_rx + i0 * 8);
+  int4 r0 = __ldg(r), r1 = __ldg(r + 1), r2 = __ldg(r + 2), r3 = __ldg(r + 3);
+#pragma unroll 1
+  for (int i = i0; i < i1; ++i) {
+    const int4 c0 = r0, c1 = r1, c2 = r2, c3 = r3;
+    r += 4;                                    // the next record (the table ends with a spare one)
+    r0 = __ldg(r); r1 = __ldg(r + 1); r2 = __ldg(r + 2); r3 = __ldg(r + 3);
+    // c0: c, beta; c1: tau, reactants 0 and 1; c2: reactant 2, products 0 to 2; c3: the row
+    // (byte offsets), the flag
+    Pair beta, tau;
+    beta.lo = c0.z; beta.hi = c0.w;
+    tau.lo = c1.x; tau.hi = c1.y;
+    const i64 c = (i64)(((u64)(unsigned)c0.y << 32) | (unsigned)c0.x);
+    auto at = [](const char* b, int o) { return *(const i64*)(b + o); };
+    i64 X = (pfx::mul_add(tau, v, pfx::mul_add(beta, u, c)) & ~1ll) - at(lam, c1.z);
+    X -= at(lam, c1.w);
+    if (NF > 2) X -= at(lam, c2.x);
+    i64 Xf = X + at(alp, c1.z) + at(alp, c1.w);
+    if (NF > 2) Xf += at(alp, c2.x);
+    i64 Xr = X;
+    if (REV) {
+      Xr += at(alp, c2.y) + at(alp, c2.z);
+      if (NF > 2) Xr += at(alp, c2.w);
+    }
+    i64 rate = tile_rate<REV>(Xf, Xr, s.exp2);
+    i64* o = (i64*)(R + c3.x);
+    if (c3.y) rate = tile_add(*o, rate);
+    *o = rate;
+  }
+}
+
+__device__ __forceinline__ double ax_d(i64 v) { return __longlong_as_double(v); }
+
+// sum_k eps_k Y_k/W_k of a reaction from its efficiency list
+__device__ __forceinline__ double tile_mS(const i64* ax, int ne, double ysum, const double* __restrict__ Yp, i64 n) {
+  double m = ysum;
+#pragma unroll 4
+  for (int q = 0; q < ne; ++q) {
+    const longlong2 c = __ldg((const longlong2*)ax + q);
+    m = fma(__ldg(Yp + c.x * n), ax_d(c.y), m);
+  }
+  return m;
+}
+
+__device__ __forceinline__ bool tile_normal_pos(double x) {
+  const int h = __double2hiint(x);
+  return h >= 0x00100000 && h < 0x7ff00000;
+}
+
+enum { TK_THREEBODY = 1, TK_LINDEMANN = 2, TK_TROE = 3, TK_SRI = 4, TK_PLOG = 5 };
+
+// f l for 0 <= f <= 1 and a logarithm l
+__device__ __forceinline__ i64 tile_part(double f, i64 l) {
+  const bool near_one = f >= 0.9999;
+  const double g = fmax(near_one ? 1.0 - f : f, 1e-300);
+  const i64 p = pfx::mul_add(pfx::split(2 * l), pfx::split(pfx::frac_of(g)), 0ll);
+  return near_one ? l - p : p;
+}
+
+// reactions of the other classes: auxiliary data ax (see the emitter for the layout)
+__device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, int lane, double rho,
+                                           const double* __restrict__ Yp, i64 n) {
+  const Pair u = s.sc->u[lane], v = s.sc->v[lane], t = s.sc->t[lane];
+  const double ysum = s.sc->ysum[lane];
+  const i64* lam = s.lam + lane;
+  const i64* alp = s.alp + lane;
+#pragma unroll 1
+  for (int i = i0; i < i1; ++i) {
+    const i64* r = t_rx + i * 8;
+    const i64 fa = __ldg(r + 3), fb = __ldg(r + 4);
+    const int nr = (int)((fb >> 48) & 0xf), np = (int)((fb >> 52) & 0xf), kind = (int)((fb >> 56) & 0xf);
+    const i64* ax = t_ax + __ldg(r + 5);
+    const int ne = (int)__ldg(ax);
+    // log2 [M] of the reaction (PLOG: of the total concentration)
+    const double M = rho * tile_mS(ax + 16, ne, ysum, Yp, n);
+    if (!tile_normal_pos(M)) s.sc->bad[lane] = 1;
+    const i64 lgM = pfx::log2_of(M, t_log2);
+    i64 X;
+    if (kind == TK_PLOG) {
+      // log2 k linear in log2 p between the bracketing nodes, end nodes outside
+      const int nn = (int)__ldg(ax + 1);
+      const i64* nd = ax + 16;               // nodes {lg p, 1/(lg p_next - lg p), c, beta, tau}
+      const i64 lgp = s.sc->lgT[lane] + lgM + T_LG_R;
+      int q = 0;
+      for (int j = 1; j + 1 < nn; ++j) if (lgp >= __ldg(nd + 5 * j)) q = j;
+      const i64* a = nd + 5 * q;
+      const i64 xa = tile_K(__ldg(a + 2), __ldg(a + 3), __ldg(a + 4), u, v);
+      const i64 xb = tile_K(__ldg(a + 7), __ldg(a + 8), __ldg(a + 9), u, v);
+      const double pf = fmin(fmax(pfx::to_double(lgp - __ldg(a)) * ax_d(__ldg(a + 1)), 0.0), 1.0);
+      X = pf > 0.0 ? xa + tile_part(pf, xb - xa) : xa;
+    } else {
+      X = tile_K(__ldg(r), __ldg(r + 1), __ldg(r + 2), u, v);
+    }
+    if (kind == TK_THREEBODY) X += lgM;
+    if (kind >= TK_LINDEMANN && kind <= TK_SRI) {
+      const i64 lgPr = tile_K(__ldg(ax + 2), __ldg(ax + 3), __ldg(ax + 4), u, v) + lgM;
+      // log2(Pr/(1+Pr)) = min(lgPr, 0) - log2(1 + 2^-|lgPr|)
+      const i64 am = lgPr < 0 ? lgPr : -lgPr;
+      u64 q = 0x4000000000000000ull + tile_shr(pfx::exp2_mant(am, s.exp2), 1 - (int)(am >> pfx::LG_F));   // [1, 2], f = 62
+      q = q > 0x7fffffffffffffffull ? 0x7fffffffffffffffull : q;
+      X += (lgPr < 0 ? lgPr : 0ll) - ((pfx::log2_mant(q >> 10, t_log2) + 0x800ll) >> 12);
+      if (kind != TK_LINDEMANN) {
+        // the sum of up to three exponentials (Troe: F_cent, SRI: a e^(-b/T) + e^(-T/c)),
+        // exponents c + beta t + gamma v
+        double S = 0.0;
+        const int nt = (int)__ldg(ax + 1);
+#pragma unroll 1
+        for (int j = 0; j < nt; ++j) {
+          const i64* e = ax + 5 + 3 * j;
+          const i64 x = pfx::mul_add(as_pair(__ldg(e + 1)), t, pfx::mul_add(as_pair(__ldg(e + 2)), v, 0ll)) & ~1ll;
+          S += pfx::exp2_lg(x + __ldg(e), s.exp2);
+        }
+        if (!tile_normal_pos(S)) s.sc->bad[lane] = 1;
+        const i64 lS = pfx::log2_of(S, t_log2);
+        // Troe: log F = log F_cent den^2/(den^2 + x^2), all logarithms to base 10;
+        // SRI: F = d S^(1/(1 + log10^2 Pr)) T^e
+        double x = pfx::to_double(lgPr) * 0.30102999566398119521, den2 = 1.0;
+        if (kind == TK_TROE) {
+          const double lf10 = pfx::to_double(lS) * 0.30102999566398119521;
+          x += fma(-0.67, lf10, -0.4);
+          const double den = fma(-0.14, x, fma(-1.27, lf10, 0.75));
+          den2 = den * den;
+        }
+        X += tile_part(den2 * pdm::rcp(fma(x, x, den2)), lS);
+        if (kind == TK_SRI) X += pfx::mul_add(as_pair(__ldg(ax + 15)), u, __ldg(ax + 14));
+      }
+    }
+    X &= ~1ll;
+    // factors
+    i64 Xf = 0, Xr = np ? 0ll : pfx::LG_ZERO;
+    for (int q = 0; q < nr; ++q) {
+      const int k = (int)((fa >> (16 * q)) & 0xffff) * 32;
+      X -= lam[k];
+      Xf += alp[k];
+    }
+    for (int q = 0; q < np; ++q) {
+      const int k = (int)((q == 0 ? (fa >> 48) : (fb >> (16 * (q - 1)))) & 0xffff) * 32;
+      Xr += alp[k];
+    }
+    s.R[(int)((fb >> 32) & 0xffff) * 32 + lane] = tile_rate<true>(X + Xf, X + Xr, s.exp2);
+  }
+}
+
+struct TilePlus { static constexpr bool minus = false; };
+struct TileMinus { static constexpr bool minus = true; };
+
+extern "C" __global__ void __launch_bounds__(32 * NW, TILE_MINB)
+pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict__ g_Tin, int energy_mode,
+                const double* __restrict__ g_Y, double* __restrict__ g_Tout, double* __restrict__ g_omega,
+                double T_guess, int max_iter, double tol, unsigned long long* __restrict__ g_fail) {
+  extern __shared__ __align__(16) char s_raw[];
+  const TileSmem s = tile_smem(s_raw);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < pfx::EXP2_TAB; i += 32 * NW) s.exp2[i] = t_exp2[i];
+  const i64 tiles = (n + 31) >> 5;
+  if (w == 0) {                                 // the zero row that pads the lists of the species sums
+    s.R[TILE_ROWS * 32 + lane] = 0;
+    s.lam[NSP * 32 + lane] = 0;                 // the unit factor
+    s.alp[NSP * 32 + lane] = 0;
+  }
+#pragma unroll 1
+  for (i64 tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const i64 p = tile * 32 + lane;
+    const i64 pc = p < n ? p : n - 1;
+    const double* Yp = g_Y + pc;
+    const double rho = __ldg(g_rho + pc);
+    {
+      {
+        double y[KPW];
+        double ys = 0.0;
+#pragma unroll
+        for (int i = 0; i < KPW; ++i) {
+          const int k = w + i * NW;
+          y[i] = k < NSP ? __ldg(Yp + k * n) : 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < KPW; ++i) {
+          const int k = w + i * NW;
+          if (k < NSP) {
+            ys = fma(y[i], __ldg(t_iw + k), ys);
+            s.alp[k * 32 + lane] = __double_as_longlong(y[i]);
+          }
+        }
+        s.ys[w * 32 + lane] = ys;
+      }
+      bool bad = false;
+      double T;
+      bool ok = true;
+      if (energy_mode) {
+        tile_energy(s, Yp, n, __ldg(g_Tin + pc), T_guess, max_iter, (float)tol, w, lane, T, ok);
+      } else {
+        T = __ldg(g_Tin + pc);
+        __syncthreads();
+      }
+      if (w == 0) {
+        if (energy_mode && p < n) {
+          if (!ok) atomicAdd(g_fail, 1ull);
+          g_Tout[p] = T;
+        }
+        // state scalars; states outside the tables' range are left to the FP64 kernel
+        const unsigned re = ((unsigned)__double2hiint(rho) >> 20) & 0x7ff;
+        const bool in = T > T_LO && T < T_HI && re >= 1023 - 60 && re <= 1023 + 20;
+        const double Ts = in ? T : 1000.0;
+        const i64 lgT = pfx::log2_of(Ts, t_log2);
+        s.sc->T[lane] = Ts;
+        s.sc->lgT[lane] = lgT;
+        s.sc->lgrho[lane] = pfx::log2_of(in ? fabs(rho) : 1.0, t_log2) | (i64)((u64)__double_as_longlong(rho) >> 63);
+        s.sc->u[lane] = pfx::split(lgT << 9);
+        s.sc->v[lane] = pfx::split(pfx::frac_of(T_V * pdm::rcp(Ts)));
+        s.sc->t[lane] = pfx::split(pfx::frac_of(Ts * (1.0 / T_T)));
+        s.sc->bad[lane] = in ? 0 : 1;
+      }
+      if (w == NW - 1) {
+        double a = 0.0;
+#pragma unroll
+        for (int i = 0; i < NW; ++i) a += s.ys[i * 32 + lane];
+        s.sc->ysum[lane] = a;
+      }
+      __syncthreads();
+      // species: lambda_k and alpha_k
+      const Pair u = s.sc->u[lane], v = s.sc->v[lane], t = s.sc->t[lane];
+      const i64 lgrho = s.sc->lgrho[lane];
+      const int hi = pdm::to_float_trunc(s.sc->T[lane]) >= (float)TMID ? 1 : 0;
+#pragma unroll 1
+      for (int k = w; k < NSP; k += NW) {
+        const longlong2* c = (const longlong2*)(t_sp + (k * 2 + hi) * 8);
+        const longlong2 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2), c3 = __ldg(c + 3);   // c4 c3 | c2 c1 | c0 cl | ci -
+        i64 q = pfx::horner(c0.x, t, c0.y);
+        q = pfx::horner(q, t, c1.x);
+        q = pfx::horner(q, t, c1.y);
+        q = pfx::horner(q, t, c2.x);
+        q = tile_K(q, c2.y, c3.x, u, v);
+        const u64 yb = (u64)s.alp[k * 32 + lane];
+        const int ye = (int)(yb >> 52) & 0x7ff;
+        const bool zero = (yb << 1) == 0ull;
+        bad |= (ye == 0 && !zero) || ye > 1023 + 8;
+        i64 ly = pfx::log2_of(__longlong_as_double((i64)(yb & 0x7fffffffffffffffull)), t_log2);
+        ly = zero ? pfx::LG_ZERO : (ly | (i64)(yb >> 63));
+        s.lam[k * 32 + lane] = q;
+        s.alp[k * 32 + lane] = q + ly + lgrho;
+      }
+      if (bad) s.sc->bad[lane] = 1;
+      __syncthreads();
+    }
+    const Pair u = s.sc->u[lane], v = s.sc->v[lane];
+    const bool open = s.sc->bad[lane] != 0;
+#pragma unroll 1
+    for (int ch = 0; ch < NCH; ++ch) {
+      const int* seg = t_seg + (ch * NW + w) * (NCLS + 1);
+      // every other warp takes the plain reactions last: they load the integer pipes, the
+      // others the FP64 pipe
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        if ((w & 1) == half) {
+          TILE_PLAIN
+        } else {
+          const int a = __ldg(seg + NCLS - 1), b = __ldg(seg + NCLS);
+          if (a < b) tile_other(s, a, b, lane, rho, Yp, n);
+        }
+      }
+      __syncthreads();
+      // species sums: per owned species the rows with nu = +1, with -1 (both padded to
+      // multiples of 4 with the zero row) and with other nu
+      const char* R = (const char*)(s.R + lane);
+#pragma unroll 1
+      for (int i = 0; i < KPO; ++i) {
+        const int4 q = __ldg((const int4*)t_wl + (ch * NW + w) * KPO + i);   // first entry, ends of the three lists
+        const int2 o = __ldg((const int2*)t_wo + (ch * NW + w) * KPO + i);   // species, head-room bits + 256 others
+        if (o.x < 0) break;
+        const int hb = o.y & 0xff;
+        i64 a = 0;
+        int e = 0;
+        auto quad = [&](int j, auto sign) {
+          const int4 r = __ldg((const int4*)(t_we + j));
+          const i64 v0 = *(const i64*)(R + r.x), v1 = *(const i64*)(R + r.y), v2 = *(const i64*)(R + r.z),
+                    v3 = *(const i64*)(R + r.w);
+          const int e0 = (int)v0 & 4095, e1 = (int)v1 & 4095, e2 = (int)v2 & 4095, e3 = (int)v3 & 4095;
+          const int en = max(max(e, max(e0, e1)), max(e2, e3)), t = en + hb;
+          a = tile_sar(a, en - e);
+          e = en;
+          const i64 b = (tile_sar(v0, t - e0) + tile_sar(v1, t - e1)) + (tile_sar(v2, t - e2) + tile_sar(v3, t - e3));
+          if (decltype(sign)::minus) a -= b; else a += b;
+        };
+        for (int j = q.x; j < q.y; j += 4) quad(j, TilePlus());
+        for (int j = q.y; j < q.z; j += 4) quad(j, TileMinus());
+        for (int j = q.z; j < q.z + (o.y >> 8); ++j) {
+          const i64 x = *(const i64*)(R + __ldg(t_we + j));
+          const int e0 = (int)x & 4095, en = max(e, e0);
+          a = tile_sar(a, en - e) + (i64)__ldg(t_wc + j) * tile_sar(x, en + hb - e0);
+          e = en;
+        }
+        double v = tile_to_double(a, e + hb - RATE_E, 61);
+        if (p < n) {
+          double* out = g_omega + o.x * n + p;
+          if (ch > 0) v += *out;
+          if (open && o.x == 0) v = __longlong_as_double(TILE_OPEN);
+          *out = v;
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
