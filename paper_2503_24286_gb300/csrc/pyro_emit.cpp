@@ -88,30 +88,121 @@ __device__ __forceinline__ void pyro_load_tables(double* se, double* sl) {
 
 void emit_tsolve(Src& s, const Mechanism& m, const std::vector<SpeciesCoef>& C, const EmitOptions& opt,
                  std::map<std::string, double>& st) {
-  int N = m.n_species();
-  // FP32 collapse (both ranges) and FP64 collapse (one range)
-  s << "// Newton inversion of e = sum_k Y_k e_k(T) (Sec. A.3.1, Eq. delta_temp), or with\n"
-       "// ENTH of h = sum_k Y_k h_k(T) (the enthalpy variant: the linear coefficient of each\n"
-       "// species polynomial gains 1/W_k, c_v becomes c_p); returns T, writes the iteration\n"
-       "// count (FP32 + FP64 steps) or -1 if max_iter FP64 steps did not meet |dT| <= tol T.\n";
-  s << "template <bool ENTH>\n__device__ __forceinline__ double pyro_tsolve(const double* __restrict__ Yp, i64 n, double e,\n"
-       "    double T0, int max_iter, float tolf, int* iters) {\n";
-  s << "  const double eR = e * " << lit((double)(1.0L / R_GAS)) << ";\n";
-  Src dummy;
-  s << "  float bl0=0.f,bl1=0.f,bl2=0.f,bl3=0.f,bl4=0.f,bl5=0.f,bh0=0.f,bh1=0.f,bh2=0.f,bh3=0.f,bh4=0.f,bh5=0.f;\n";
-  for (int k = 0; k < N; ++k) {
-    const double invW = 1.0 / m.species[k].W;
-    auto cf = [&](int r, int q) {
-      if (q != 1) return litf(C[k].d[r][q]);
-      return "(ENTH ? " + litf(C[k].d[r][1] + invW) + " : " + litf(C[k].d[r][1]) + ")";
-    };
-    s << "  { float y = pdm::to_float_trunc(__ldg(Yp + (i64)" << k << " * n));";
-    for (int q = 0; q < 6; ++q) s << " bl" << q << " = fmaf(y, " << cf(0, q) << ", bl" << q << ");";
-    for (int q = 0; q < 6; ++q) s << " bh" << q << " = fmaf(y, " << cf(1, q) << ", bh" << q << ");";
-    s << " }\n";
+  const int N = m.n_species(), NP = (N + 7) / 8 * 8;
+  // Tables, one row per species (rows past the last one are zero).  FP32: the energy
+  // coefficients d_0..d_5 of both ranges and the enthalpy's d_1 + 1/W.  FP64 and integer:
+  // per range d_0..d_5, d_1 + 1/W.  An integer column m is scaled by 2^s_m with its largest
+  // coefficient in [2^(hb-1), 2^hb), hb = min(57, 62 - ceil(log2 N)): the sums of
+  // products of halves, the high one shifted by 7, then stay below 2^63 while sum |Y| < 2.
+  int hb = 57;
+  while ((1 << (62 - hb)) < N) --hb;
+  auto coef = [&](int k, int r, int q) { return q < 6 ? C[k].d[r][q] : C[k].d[r][1] + 1.0 / m.species[k].W; };
+  int sc[7];
+  for (int q = 0; q < 7; ++q) {
+    double mx = 0.0;
+    for (int k = 0; k < N; ++k) for (int r = 0; r < 2; ++r) mx = std::max(mx, std::fabs(coef(k, r, q)));
+    sc[q] = mx > 0.0 ? hb - 1 - std::ilogb(mx) : 0;
   }
-  s << R"(  float Tf = pdm::to_float_trunc(T0);
-  const float eRf = pdm::to_float_trunc(eR);
+  std::ostringstream tf, td, tx;
+  for (int k = 0; k < NP; ++k) {
+    for (int q = 0; q < 16; ++q) {
+      const double v = k >= N || q > 13 ? 0.0 : q < 12 ? coef(k, q / 6, q % 6) : coef(k, q - 12, 6);
+      tf << (k || q ? "," : "") << litf(v);
+    }
+    for (int r = 0; r < 2; ++r)
+      for (int q = 0; q < 8; ++q) {
+        const double v = k >= N || q > 6 ? 0.0 : coef(k, r, q);
+        td << (k || r || q ? "," : "") << lit(v);
+        const long long x = q > 6 ? 0 : llroundl(ldexpl((long double)v, sc[q]));
+        const int lo = (int)(unsigned)(unsigned long long)x;      // two signed halves (pfx::Pair)
+        const long long hi = (x - lo) / 4294967296ll;
+        tx << (k || r || q ? "," : "") << (long long)(((unsigned long long)hi << 32) | (unsigned)lo) << "ll";
+      }
+  }
+  s << "#include \"pyro_fixed_math.cuh\"\n#define TS_ROWS " << NP << "\n#define TS_INV_R " << lit((double)(1.0L / R_GAS))
+    << "\n#define TS_INV_R_LO " << lit((double)(1.0L / R_GAS - (long double)(double)(1.0L / R_GAS))) << "\n";
+  s << "__device__ const __align__(16) float ts_f[" << 16 * NP << "] = {" << tf.str() << "};\n";
+  s << "__device__ const __align__(16) double ts_d[" << 16 * NP << "] = {" << td.str() << "};\n";
+  s << "__device__ const __align__(16) long long ts_x[" << 16 * NP << "] = {" << tx.str() << "};\n";
+  s << "__device__ const int ts_s[8] = {";
+  for (int q = 0; q < 7; ++q) s << sc[q] + 61 << ",";   // f of the sums: the column's scale and Y's 61
+  s << "0};\n";
+  s << R"(
+// Collapse of the species polynomials into the mixture polynomial of one range,
+// B_m = sum_k Y_k d_km, in FP64: for mass fractions outside the integer form's range.
+template <bool ENTH>
+__device__ __noinline__ void ts_collapse64(const double* __restrict__ Yp, i64 n, bool hi, double* B) {
+  for (int q = 0; q < 6; ++q) B[q] = 0.0;
+  for (int k = 0; k < NSP; ++k) {
+    const double y = __ldg(Yp + (i64)k * n);
+    const double* d = ts_d + (k * 2 + hi) * 8;
+    for (int q = 0; q < 6; ++q) B[q] = fma(y, d[ENTH && q == 1 ? 6 : q], B[q]);
+  }
+}
+
+// The same on the integer pipe, exact up to the 2^-61 of Y and the coefficients' 2^-hb.
+// The FP64 form takes 6 N = 318 FP64 instructions for 53 species, 6,000 cycles of an SM per
+// warp against ~2,000 of the integer form: 2^20 temperatures 0.72 ms with FP64.
+template <bool ENTH>
+__device__ __forceinline__ void ts_collapse(const double* __restrict__ Yp, i64 n, bool hi, double (&B)[6]) {
+  i64 h[6], l[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) h[q] = l[q] = 0;
+#pragma unroll 1
+  for (int k0 = 0; k0 < NSP; k0 += 8) {
+    double y[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) y[i] = k0 + i < NSP ? __ldg(Yp + (i64)(k0 + i) * n) : 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const longlong2* c = (const longlong2*)(ts_x + ((k0 + i) * 2 + hi) * 8);
+      const longlong2 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2);
+      const i64 x[6] = {c0.x, ENTH ? __ldg((const i64*)c + 6) : c0.y, c1.x, c1.y, c2.x, c2.y};
+      const pfx::Pair v = pfx::split(pfx::fix61(y[i]));
+#pragma unroll
+      for (int q = 0; q < 6; ++q) {
+        const int ch = (int)(x[q] >> 32), cl = (int)x[q];
+        h[q] += (i64)ch * v.hi;
+        l[q] += (i64)ch * v.lo;
+        l[q] += (i64)cl * v.hi;
+        l[q] += (i64)pfx::mulhi_s(cl, v.lo);
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 6; ++q)      // h 2^64 + l 2^32 = (h 2^7 + l 2^-25) 2^57
+    B[q] = pfx::scaled((h[q] << 7) + ((l[q] + 0x1000000ll) >> 25), 57 - __ldg(ts_s + (ENTH && q == 1 ? 6 : q)));
+}
+
+// Newton inversion of e = sum_k Y_k e_k(T) (Sec. A.3.1, Eq. delta_temp), or with
+// ENTH of h = sum_k Y_k h_k(T) (the enthalpy variant: the linear coefficient of each
+// species polynomial gains 1/W_k, c_v becomes c_p); returns T, writes the iteration
+// count (FP32 + FP64 steps) or -1 if max_iter FP64 steps did not meet |dT| <= tol T.
+template <bool ENTH>
+__device__ __forceinline__ double pyro_tsolve(const double* __restrict__ Yp, i64 n, double e,
+    double T0, int max_iter, float tolf, int* iters) {
+  float bl0=0.f,bl1=0.f,bl2=0.f,bl3=0.f,bl4=0.f,bl5=0.f,bh0=0.f,bh1=0.f,bh2=0.f,bh3=0.f,bh4=0.f,bh5=0.f;
+  float ysum = 0.f;
+#pragma unroll 1
+  for (int k0 = 0; k0 < NSP; k0 += 8) {
+    double yd[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) yd[i] = k0 + i < NSP ? __ldg(Yp + (i64)(k0 + i) * n) : 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float4* c = (const float4*)(ts_f + (k0 + i) * 16);
+      const float4 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2);
+      const float y = pdm::to_float_trunc(yd[i]);
+      float d1l = c0.y, d1h = c1.w;
+      if (ENTH) { const float2 g = __ldg((const float2*)(c + 3)); d1l = g.x; d1h = g.y; }
+      ysum += fabsf(y);
+      bl0 = fmaf(y, c0.x, bl0); bl1 = fmaf(y, d1l, bl1); bl2 = fmaf(y, c0.z, bl2); bl3 = fmaf(y, c0.w, bl3);
+      bl4 = fmaf(y, c1.x, bl4); bl5 = fmaf(y, c1.y, bl5); bh0 = fmaf(y, c1.z, bh0); bh1 = fmaf(y, d1h, bh1);
+      bh2 = fmaf(y, c2.x, bh2); bh3 = fmaf(y, c2.y, bh3); bh4 = fmaf(y, c2.z, bh4); bh5 = fmaf(y, c2.w, bh5);
+    }
+  }
+  float Tf = pdm::to_float_trunc(T0);
+  const float eRf = pdm::to_float_trunc(e * TS_INV_R);
   int it32 = 0;
   if (opt_mixed) {
     for (; it32 < 40; ) {
@@ -130,43 +221,30 @@ void emit_tsolve(Src& s, const Mechanism& m, const std::vector<SpeciesCoef>& C, 
   }
   double T = opt_mixed ? pdm::to_double(Tf) : T0;
   bool hi = pdm::to_float_trunc(T) >= (float)TMID;
-  double B0, B1, B2, B3, B4, B5;
-)";
-  // collapse macro for a given range flag 'hi'
-  s << "  auto collapse = [&](bool hi) {\n    B0 = 0.0; B1 = 0.0; B2 = 0.0; B3 = 0.0; B4 = 0.0; B5 = 0.0;\n";
-  for (int k = 0; k < N; ++k) {
-    const double invW = 1.0 / m.species[k].W;
-    s << "    { double y = __ldg(Yp + (i64)" << k << " * n);";
-    for (int q = 0; q < 6; ++q) {
-      double v[2] = {C[k].d[0][q], C[k].d[1][q]};
-      if (q == 1) {
-        double vh[2] = {C[k].d[0][1] + invW, C[k].d[1][1] + invW};
-        s << " B1 = fma(y, (ENTH ? " << sel(vh) << " : " << sel(v) << "), B1);";
-      } else {
-        s << " B" << q << " = fma(y, " << sel(v) << ", B" << q << ");";
-      }
-    }
-    s << " }\n";
-  }
-  s << "  };\n";
-  st["tsolve_collapse_fp64_ops"] = 6.0 * N;
-  s << R"(  collapse(hi);
+  double B[6];
+  const bool small = ysum > 0.25f && ysum < 2.f;          // sum |Y|; false for NaN
+  auto collapse = [&] {
+    if (small) ts_collapse<ENTH>(Yp, n, hi, B);
+    else { double b[6]; ts_collapse64<ENTH>(Yp, n, hi, b); for (int q = 0; q < 6; ++q) B[q] = b[q]; }
+    // B_0 - e/R first: the formation energies cancel there, and the residual is rounded
+    // at the size of c_v T only
+    B[0] = fma(e, -TS_INV_R_LO, fma(e, -TS_INV_R, B[0]));
+  };
   int it64 = 0;
-  bool flag = false, ok = false;
+  bool flag = false, ok = false, have = false;
   for (int it = 0; it < max_iter + 1; ++it) {
     ++it64;
     float Tcur = pdm::to_float_trunc(T);
     bool h2 = Tcur >= (float)TMID;
-    if (h2 != hi) { hi = h2; collapse(hi); }
-    double e64 = fma(T, fma(T, fma(T, fma(T, fma(T, B5, B4), B3), B2), B1), B0);
-    double res = e64 - eR;
+    if (h2 != hi || !have) { hi = h2; collapse(); have = true; }     // one copy of the collapse
+    double res = fma(T, fma(T, fma(T, fma(T, fma(T, B[5], B[4]), B[3]), B[2]), B[1]), B[0]);
     double dT;
     if (opt_mixed) {
       float c0 = hi ? bh1 : bl1, c1 = hi ? bh2 : bl2, c2 = hi ? bh3 : bl3, c3 = hi ? bh4 : bl4, c4 = hi ? bh5 : bl5;
       float cvf = fmaf(Tcur, fmaf(Tcur, fmaf(Tcur, fmaf(Tcur, 5.f * c4, 4.f * c3), 3.f * c2), 2.f * c1), c0);
       dT = res * pdm::to_double(-__frcp_rn(cvf));
     } else {
-      double cv = fma(T, fma(T, fma(T, 5.0 * B5 * T + 4.0 * B4, 3.0 * B3), 2.0 * B2), B1);
+      double cv = fma(T, fma(T, fma(T, 5.0 * B[5] * T + 4.0 * B[4], 3.0 * B[3]), 2.0 * B[2]), B[1]);
       dT = -res * pdm::rcp(cv);
     }
     double Tn = T + dT;
@@ -183,6 +261,7 @@ void emit_tsolve(Src& s, const Mechanism& m, const std::vector<SpeciesCoef>& C, 
   return T;
 }
 )";
+  st["tsolve_collapse_fp64_ops"] = 6.0 * N;
   // per-iteration FP64 costs
   st["tsolve_iter_fp64_ops_mixed"] = 5 + 1 + 1 + 1;            // Horner, res, dT, T+dT
   st["tsolve_iter_fp64_ops_fp64"] = 5 + 1 + 4 + 4 + 4 + 1 + 1;  // + cv Horner (4) + multiples (4) + rcp (4)
@@ -2320,6 +2399,7 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
     if (!t.source.empty()) {
       out.group_sources["tile"] = t.source;
       out.tile_warps = t.warps;
+      out.tile_chunks = t.chunks;
       out.smem_dyn_bytes_tile = t.smem_bytes;
       out.stats["tile_t_lo"] = t.t_lo;
       out.stats["tile_warps"] = t.warps;

@@ -42,6 +42,7 @@ struct EmitResult {
   int smem_dyn_bytes_transport = 0;       // dynamic shared memory of the transport kernel
   int smem_dyn_bytes_jac = 0;             // dynamic shared memory of the Jacobian-type kernels
   int tile_warps = 0;                     // warps per block of the tile kernel
+  int tile_chunks = 0;                    // reaction chunks per tile
   int smem_dyn_bytes_tile = 0;            // dynamic shared memory of the tile kernel
   int cn_solve_warps = 4;                 // states (warps) per block of the Crank-Nicolson solve kernel
   // warp-per-state kernels ("wfwd", "wjvp", "wvjp"): states (warps) per block and

@@ -36,7 +36,9 @@ struct Fix {
   }
   i64 coef(ld v) {        // f = 51 as two signed halves
     if (!(std::fabs((double)v) < 4000.0)) { bad = true; return 0; }
-    const i64 x = (i64)llroundl(v * 2251799813685248.0L);
+    return pair((i64)llroundl(v * 2251799813685248.0L));
+  }
+  i64 pair(i64 x) {       // two signed halves
     const int lo = (int)(unsigned)(u64)x;
     const i64 hi = (x - lo) / 4294967296ll;
     return (i64)(((u64)hi << 32) | (unsigned)lo);
@@ -153,6 +155,19 @@ TileEmit emit_tile_unit(const Mechanism& m) {
   Fix fx;
   std::vector<i64> sp((size_t)N * 16);
   std::vector<double> ed((size_t)N * 12), iw(N);
+  // integer energy coefficients: column q scaled by 2^xs[q], the largest in [2^(hb-1), 2^hb),
+  // so that sums over the species stay below 2^63 while sum |Y| < 2 (TileDot)
+  std::vector<i64> ex((size_t)N * 12);
+  std::vector<int> xs(6, 0);
+  {
+    int hb = 57;
+    while ((1 << (62 - hb)) < N) --hb;
+    for (int q = 0; q < 6; ++q) {
+      double mx = 0.0;
+      for (auto& sp : m.species) { const SpeciesCoef C = species_coef(sp); for (int r = 0; r < 2; ++r) mx = std::max(mx, std::fabs(C.d[r][q])); }
+      if (mx > 0.0) xs[q] = hb - 1 - std::ilogb(mx);
+    }
+  }
   std::ostringstream ef;
   for (int k = 0; k < N; ++k) {
     const Species& s = m.species[k];
@@ -172,7 +187,10 @@ TileEmit emit_tile_unit(const Mechanism& m) {
       q[5] = fx.coef(16 * (1.0L - a[0]));
       q[6] = fx.coef((ld)a[5] * LOG2E / T_V);
       q[7] = 0;
-      for (int i = 0; i < 6; ++i) ed[((size_t)k * 2 + r) * 6 + i] = C.d[r][i];
+      for (int i = 0; i < 6; ++i) {
+        ed[((size_t)k * 2 + r) * 6 + i] = C.d[r][i];
+        ex[((size_t)k * 2 + r) * 6 + i] = fx.pair(llroundl(ldexpl((ld)C.d[r][i], xs[i])));
+      }
     }
     for (int r = 0; r < 2; ++r) for (int i = 0; i < 6; ++i) ef << (k + r + i ? "," : "") << litf(C.d[r][i]);
   }
@@ -214,7 +232,7 @@ TileEmit emit_tile_unit(const Mechanism& m) {
   const int fixed_bytes = 8192 + 512 * (N + 1) + 1920 + 256;
   int warps = rows_all < 48 ? 4 : rows_all < 120 ? 8 : 12;
   int minb = 24 / warps + (warps == 4 ? 2 : 0);
-  auto red = [](int w) { return w * 256 + 6 * 256 + 12 * 128 + w * 12 * 128; };   // scratch of the temperature solve, in the rows
+  auto red = [](int w) { return w * 256 + 6 * 256 + 14 * 128 + w * 13 * 128; };   // scratch of the temperature solve, in the rows
   while (minb > 1 && fixed_bytes + std::max(rows_all * 256, red(warps)) > kSmemPerSm / minb - kSmemPerBlock) --minb;
   if (minb == 1) warps = 24;
   const int lim = std::min(kSmemMaxBlock, kSmemPerSm / minb - kSmemPerBlock) - fixed_bytes;
@@ -343,7 +361,7 @@ TileEmit emit_tile_unit(const Mechanism& m) {
                 x[14] = fx.lg(log2l(d));
                 x[15] = fx.coef(16 * e);
               }
-              if (x.size() % 2) x.push_back(0);      // efficiency pairs are read as 16-byte units
+              if (x.size() % 2) x.push_back(0);      // 16-byte units
               ax.insert(ax.end(), x.begin(), x.end());
             }
             rx.insert(rx.end(), rec, rec + 8);
@@ -401,7 +419,11 @@ TileEmit emit_tile_unit(const Mechanism& m) {
         wo.push_back(i < (int)owned[w].size() ? owned[w][i] : -1);
         wo.push_back(hb + 256 * no);
       }
-  for (int q = 0; q < 8; ++q) rx.push_back(0);   // spare record (the loops read one ahead)
+  // spare elements (the loops read one ahead)
+  for (int q = 0; q < 16; ++q) rx.push_back(0);
+  for (int q = 0; q < 4; ++q) { wl.push_back(0); we.push_back(tile_rows * 256); wc.push_back(0); }
+  for (int q = 0; q < 2; ++q) wo.push_back(-1);
+  for (int q = 0; q < 64; ++q) ax.push_back(0);  // and the prefetches touch up to 512 bytes
 
   // ---- the unit -------------------------------------------------------------------
   std::ostringstream o;
@@ -428,6 +450,9 @@ TileEmit emit_tile_unit(const Mechanism& m) {
   o << "__device__ const __align__(16) float t_ef[" << 12 * N << "] = {" << ef.str() << "};\n";
   array(o, "__align__(16) double", "t_ed", as_d(ed));
   array(o, "double", "t_iw", as_d(iw));
+  array(o, "__align__(16) long long", "t_ex", as_ll(ex));
+  for (int& q : xs) q += 61;                     // f of the sums: the column's scale and Y's 61
+  array(o, "int", "t_exs", xs);
   array(o, "__align__(16) long long", "t_rx", as_ll(rx));
   array(o, "__align__(16) long long", "t_ax", as_ll(ax));
   array(o, "int", "t_seg", seg);

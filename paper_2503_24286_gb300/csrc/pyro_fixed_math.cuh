@@ -89,6 +89,24 @@ PFX_FN i64 frac_of(double x) {
   return s > 62 ? 0ll : (i64)(m >> s);
 }
 
+// a double of |y| < 2 with f = 61 (truncated; undefined beyond)
+PFX_FN i64 fix61(double y) {
+  const u64 b = dbits(y);
+  const int s = 1024 - ((int)(b >> 52) & 0x7ff);
+  const u64 m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 10;   // f = 62, to shift by 1 - exponent
+  const i64 v = s > 62 ? 0ll : (i64)(m >> (s & 63));
+  return (b >> 63) ? -v : v;
+}
+
+// double of v 2^e, rounded (half up in magnitude), for results within the normal range
+PFX_FN double scaled(i64 v, int e) {
+  const u64 a = v < 0 ? (u64)(-v) : (u64)v;
+  const int z = clz64(a | 1ull);
+  const u64 m = a << z;                            // leading one at bit 63
+  const u64 b = ((u64)(unsigned)(e + 63 - z + 1022) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+  return bitsd(a == 0 ? 0ull : (b | ((u64)v & 0x8000000000000000ull)));
+}
+
 // double of a value with f = 50 (truncated to 53 significant bits)
 PFX_FN double to_double(i64 v) {
   const u64 a = v < 0 ? (u64)(-v) : (u64)v;

@@ -45,6 +45,7 @@ struct Driver {
   decltype(&cuModuleUnload) ModuleUnload = nullptr;
   decltype(&cuModuleGetFunction) ModuleGetFunction = nullptr;
   decltype(&cuLaunchKernel) LaunchKernel = nullptr;
+  decltype(&cuLaunchKernelEx) LaunchKernelEx = nullptr;
   decltype(&cuFuncSetAttribute) FuncSetAttribute = nullptr;
   decltype(&cuOccupancyMaxActiveBlocksPerMultiprocessor) Occupancy = nullptr;
   decltype(&cuOccupancyMaxActiveClusters) MaxActiveClusters = nullptr;
@@ -70,6 +71,7 @@ Driver& driver() {
            get("cuModuleUnload", (void**)&d.ModuleUnload) &&
            get("cuModuleGetFunction", (void**)&d.ModuleGetFunction) &&
            get("cuLaunchKernel", (void**)&d.LaunchKernel) &&
+           get("cuLaunchKernelEx", (void**)&d.LaunchKernelEx) &&
            get("cuFuncSetAttribute", (void**)&d.FuncSetAttribute) &&
            get("cuOccupancyMaxActiveBlocksPerMultiprocessor", (void**)&d.Occupancy) &&
            get("cuOccupancyMaxActiveClusters", (void**)&d.MaxActiveClusters) &&
@@ -504,6 +506,23 @@ int ensure_store(pyro_mech* h, size_t bytes) {
   return PYRO_OK;
 }
 
+// launch configuration of the tile kernel; split: one cluster of blocks per tile
+void tile_config(const pyro_mech* h, const pyro_mech::Group& G, CUlaunchConfig* cfg, CUlaunchAttribute* attr, bool split) {
+  std::memset(cfg, 0, sizeof(*cfg));
+  std::memset(attr, 0, sizeof(*attr));
+  cfg->gridDimX = cfg->gridDimY = cfg->gridDimZ = 1;
+  cfg->blockDimX = (unsigned)G.block;
+  cfg->blockDimY = cfg->blockDimZ = 1;
+  cfg->sharedMemBytes = (unsigned)G.smem;
+  if (split) {
+    attr->id = CU_LAUNCH_ATTRIBUTE_CLUSTER_DIMENSION;
+    attr->value.clusterDim.x = (unsigned)h->emitted.tile_chunks;
+    attr->value.clusterDim.y = attr->value.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+  }
+}
+
 const char* group_kernel(const std::string& g) {
   return g == "jvp" ? "pyro_jvp" : g == "vjp" ? "pyro_vjp" : g == "jad" ? "pyro_jacobian_adiabatic"
        : g == "cn" ? "pyro_cn_assemble" : g == "tr" ? "pyro_transport" : g == "wfwd" ? "pyro_omega_warp"
@@ -569,6 +588,14 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
     if (r != CUDA_SUCCESS || nb < 1) return fail(PYRO_ECUDA, std::string(group_kernel(todo[i])) + " does not fit on an SM");
     G.blocks_per_sm = nb;
     h->emitted.stats[todo[i] + "_blocks_per_sm"] = nb;
+    if (todo[i] == "tile" && h->emitted.tile_chunks > 1 && h->emitted.tile_chunks <= 8) {
+      CUlaunchConfig cfg;
+      CUlaunchAttribute attr;
+      tile_config(h, G, &cfg, &attr, true);
+      cfg.gridDimX = (unsigned)(h->emitted.tile_chunks * h->num_sms);
+      int ncl = 0;
+      if (d.MaxActiveClusters(&ncl, G.f, &cfg) == CUDA_SUCCESS) G.clusters = ncl;   // 0: one block a tile
+    }
     if (todo[i] == "wjac" || todo[i] == "wjad") {
       // persistent grid of the clusters that fit at once (a cluster's blocks share a GPC)
       CUlaunchConfig cfg;
@@ -694,10 +721,16 @@ int launch_rates(const pyro_mech* h, int64_t n, const void* rho, const void* T_o
       Tin = T_out;
       energy = 0;
     }
-    void* params[] = {&nn, &rho, &Tin, &energy, &Y, &T_out, &omega, &Tg, &max_iter, &tol, &fail_ctr};
     const int64_t need = (n + 31) / 32, cap = (int64_t)h->num_sms * G.blocks_per_sm;
-    CUresult r = driver().LaunchKernel(G.f, (unsigned)std::min(need, cap), 1, 1, G.block, 1, 1, G.smem, as_stream(stream),
-                                       params, nullptr);
+    // as long as every tile's cluster is resident at once, the chunks of a tile run in parallel
+    int split = need <= G.clusters ? 1 : 0;
+    void* params[] = {&nn, &rho, &Tin, &energy, &Y, &T_out, &omega, &Tg, &max_iter, &tol, &fail_ctr, &split};
+    CUlaunchConfig cfg;
+    CUlaunchAttribute attr;
+    tile_config(h, G, &cfg, &attr, split != 0);
+    cfg.gridDimX = (unsigned)(split ? need * h->emitted.tile_chunks : std::min(need, cap));
+    cfg.hStream = as_stream(stream);
+    CUresult r = driver().LaunchKernelEx(&cfg, G.f, params, nullptr);
     if (r != CUDA_SUCCESS) return fail(PYRO_ECUDA, "kernel launch: " + cu_err(r));
     if (energy) Tin = T_out;
     energy = 0;

@@ -19,13 +19,13 @@
 // species and reactions are rolled: a reaction is a table record, not code, so that
 // the kernel stays within the instruction caches (with a loop per reaction shape and
 // unrolled species loops it was 119 KB and stalled on instruction fetch).
-// The FP64 pipe, which runs beside the integer work, keeps the temperature solve,
-// the third-body concentrations and the blending factors of falloff reactions.
+// The FP64 pipe, which runs beside the integer work, keeps the Newton steps, the
+// third-body concentrations and the blending factors of falloff reactions.
 //
 // States outside the tables' range (temperature outside (T_LO, T_HI), NaN,
-// infinite or subnormal mass fractions or ones beyond 2^8, densities beyond
-// 2^-60..2^20, [M] <= 0) get TILE_OPEN in their first output; the caller then
-// launches the FP64 kernel, which evaluates the states so marked.
+// infinite or subnormal mass fractions or ones from 2, densities beyond 2^-60..2^20,
+// [M] <= 0) get TILE_OPEN in their first output; the caller then launches the FP64
+// kernel, which evaluates the states so marked.
 #include "pyro_device_math.cuh"
 #include "pyro_fixed_math.cuh"
 
@@ -49,8 +49,8 @@ struct TileSmem {
   u64* exp2;
   i64 *lam, *alp;   // [NSP + 1][32]: the species and a unit factor; alp first holds Y
   i64* R;           // rows and one zero row; during the temperature solve its scratch (red, B, b, ys)
-  double* red;
-  double* B;
+  i64* red;
+  i64* B;
   float* b;
   double* ys;
   TileScalars* sc;
@@ -70,13 +70,26 @@ __device__ __forceinline__ TileSmem tile_smem(char* base) {
   s.alp = (i64*)base;                      base += (NSP + 1) * 256;
   s.R = (i64*)base;
   s.ys = (double*)base;                    // NW x 32
-  s.B = s.ys + NW * 32;                    // 6 x 32
-  s.b = (float*)(s.B + 6 * 32);            // 12 x 32
-  s.red = (double*)(s.b + 12 * 32);        // NW x 6 x 32 (FP32: NW x 12 x 32)
+  s.B = (i64*)(s.ys + NW * 32);            // 6 x 32
+  s.b = (float*)(s.B + 6 * 32);            // 14 x 32
+  s.red = (i64*)(s.b + 14 * 32);           // NW x 6 x 32 (FP32: NW x 13 x 32)
   base += (TILE_ROWS + 1) * 256;
   s.sc = (TileScalars*)base;
   return s;
 }
+
+// sums of products of fixed-point values c (two signed halves) and Y (f = 61): h 2^64 + l 2^32
+struct TileDot {
+  i64 h, l;
+  __device__ __forceinline__ void add(i64 c, Pair y) {
+    const int ch = (int)(c >> 32), cl = (int)c;
+    h += (i64)ch * y.hi;
+    l += (i64)ch * y.lo;
+    l += (i64)cl * y.hi;
+    l += (i64)pfx::mulhi_s(cl, y.lo);
+  }
+  __device__ __forceinline__ i64 sum() const { return (h << 7) + ((l + 0x1000000ll) >> 25); }   // in units of 2^57
+};
 
 // double of m 2^(e - f)
 __device__ __forceinline__ double tile_to_double(i64 m, int e, int f) {
@@ -151,27 +164,28 @@ __device__ __forceinline__ void tile_energy(const TileSmem& s, const double* __r
                                             double e, double T0, int max_iter, float tolf, int w, int lane,
                                             double& T, bool& ok) {
   {
-    float f[12];
+    float f[13];
 #pragma unroll
-    for (int q = 0; q < 12; ++q) f[q] = 0.f;
+    for (int q = 0; q < 13; ++q) f[q] = 0.f;
     const double* y = (const double*)s.alp + lane;
-#pragma unroll 1
+#pragma unroll 2
     for (int k = w; k < NSP; k += NW) {
       const float yf = pdm::to_float_trunc(y[k * 32]);
       const float4* c = (const float4*)(t_ef + k * 12);
       const float4 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2);
+      f[12] += fabsf(yf);
       f[0] = fmaf(yf, c0.x, f[0]); f[1] = fmaf(yf, c0.y, f[1]); f[2] = fmaf(yf, c0.z, f[2]); f[3] = fmaf(yf, c0.w, f[3]);
       f[4] = fmaf(yf, c1.x, f[4]); f[5] = fmaf(yf, c1.y, f[5]); f[6] = fmaf(yf, c1.z, f[6]); f[7] = fmaf(yf, c1.w, f[7]);
       f[8] = fmaf(yf, c2.x, f[8]); f[9] = fmaf(yf, c2.y, f[9]); f[10] = fmaf(yf, c2.z, f[10]); f[11] = fmaf(yf, c2.w, f[11]);
     }
     float* red = (float*)s.red;
 #pragma unroll
-    for (int q = 0; q < 12; ++q) red[(w * 12 + q) * 32 + lane] = f[q];
+    for (int q = 0; q < 13; ++q) red[(w * 13 + q) * 32 + lane] = f[q];
     __syncthreads();
-    for (int q = w; q < 12; q += NW) {
+    for (int q = w; q < 13; q += NW) {
       float a = 0.f;
 #pragma unroll
-      for (int i = 0; i < NW; ++i) a += red[(i * 12 + q) * 32 + lane];
+      for (int i = 0; i < NW; ++i) a += red[(i * 13 + q) * 32 + lane];
       s.b[q * 32 + lane] = a;
     }
     __syncthreads();
@@ -191,33 +205,37 @@ __device__ __forceinline__ void tile_energy(const TileSmem& s, const double* __r
   }
   bool hi = Tf >= (float)TMID;
   {
-    double B[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    // the collapse of one range on the integer pipe (exact up to the 2^-61 of Y)
+    TileDot d[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) d[q].h = d[q].l = 0;
 #pragma unroll 1
     for (int k = w; k < NSP; k += NW) {
-      const double y = ((const double*)s.alp)[k * 32 + lane];
-      const double2* d = (const double2*)(t_ed + (k * 2 + hi) * 6);
-      const double2 d0 = __ldg(d), d1 = __ldg(d + 1), d2 = __ldg(d + 2);
-      B[0] = fma(y, d0.x, B[0]); B[1] = fma(y, d0.y, B[1]);
-      B[2] = fma(y, d1.x, B[2]); B[3] = fma(y, d1.y, B[3]);
-      B[4] = fma(y, d2.x, B[4]); B[5] = fma(y, d2.y, B[5]);
+      const Pair y = pfx::split(pfx::fix61(((const double*)s.alp)[k * 32 + lane]));
+      const longlong2* c = (const longlong2*)(t_ex + (k * 2 + hi) * 6);
+      const longlong2 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2);
+      d[0].add(c0.x, y); d[1].add(c0.y, y); d[2].add(c1.x, y);
+      d[3].add(c1.y, y); d[4].add(c2.x, y); d[5].add(c2.y, y);
     }
-    double* red = s.red;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) red[(w * 6 + q) * 32 + lane] = B[q];
-  }
-  __syncthreads();
-  for (int q = w; q < 6; q += NW) {
-    const double* red = s.red + q * 32 + lane;
-    double a = 0.0;
-#pragma unroll
-    for (int i = 0; i < NW; ++i) a += red[i * 6 * 32];
-    s.B[q * 32 + lane] = a;
+    for (int q = 0; q < 6; ++q) s.red[(w * 6 + q) * 32 + lane] = d[q].sum();
   }
   __syncthreads();
   if (w != 0) return;
   double B[6];
+  if (b[12 * 32] > 0.25f && b[12 * 32] < 2.f) {   // sum |Y| (false for NaN)
+#pragma unroll 1
+    for (int q = 0; q < 6; ++q) {
+      i64 a = 0;
 #pragma unroll
-  for (int q = 0; q < 6; ++q) B[q] = s.B[q * 32 + lane];
+      for (int i = 0; i < NW; ++i) a += s.red[(i * 6 + q) * 32 + lane];
+      s.B[q * 32 + lane] = a;
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) B[q] = pfx::scaled(s.B[q * 32 + lane], 57 - t_exs[q]);
+  } else {
+    tile_collapse_all(Yp, n, hi, B);
+  }
   // B[0] - e/R first: the terms that cancel are large (formation energies), the rest is
   // of the size of c_v T, and the residual is rounded at that size only
   auto take_e = [&] { B[0] = fma(e, -T_INV_R_LO, fma(e, -T_INV_R, B[0])); };
@@ -289,7 +307,8 @@ __device__ __forceinline__ void tile_plain(const TileSmem& s, int i0, int i1, Pa
 
 __device__ __forceinline__ double ax_d(i64 v) { return __longlong_as_double(v); }
 
-// sum_k eps_k Y_k/W_k of a reaction from its efficiency list
+// sum_k eps_k Y_k/W_k of a reaction from its efficiency list.  In FP64: the integer form
+// (TileDot) takes some 25 instructions a term and was slower (2^20 states 8.0 against 7.3 ms).
 __device__ __forceinline__ double tile_mS(const i64* ax, int ne, double ysum, const double* __restrict__ Yp, i64 n) {
   double m = ysum;
 #pragma unroll 4
@@ -322,12 +341,18 @@ __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, in
   const double ysum = s.sc->ysum[lane];
   const i64* lam = s.lam + lane;
   const i64* alp = s.alp + lane;
+  i64 an = __ldg(t_rx + i0 * 8 + 5);
 #pragma unroll 1
   for (int i = i0; i < i1; ++i) {
     const i64* r = t_rx + i * 8;
     const i64 fa = __ldg(r + 3), fb = __ldg(r + 4);
     const int nr = (int)((fb >> 48) & 0xf), np = (int)((fb >> 52) & 0xf), kind = (int)((fb >> 56) & 0xf);
-    const i64* ax = t_ax + __ldg(r + 5);
+    const i64* ax = t_ax + an;
+    an = __ldg(r + 13);                          // of the next reaction: its lines are fetched meanwhile
+    if (i + 1 < i1) {
+      const char* pre = (const char*)(t_ax + an) + (lane & 3) * 128;
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(pre));
+    }
     const int ne = (int)__ldg(ax);
     // log2 [M] of the reaction (PLOG: of the total concentration)
     const double M = rho * tile_mS(ax + 16, ne, ysum, Yp, n);
@@ -405,7 +430,11 @@ struct TileMinus { static constexpr bool minus = true; };
 extern "C" __global__ void __launch_bounds__(32 * NW, TILE_MINB)
 pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict__ g_Tin, int energy_mode,
                 const double* __restrict__ g_Y, double* __restrict__ g_Tout, double* __restrict__ g_omega,
-                double T_guess, int max_iter, double tol, unsigned long long* __restrict__ g_fail) {
+                double T_guess, int max_iter, double tol, unsigned long long* __restrict__ g_fail, int split) {
+  // split: a cluster of NCH blocks per tile, one chunk of reactions each (few tiles: the
+  // chunks' time is the call's; 160 species, 1024 states: 113 us by one block a tile).
+  // Every block solves the temperature and prepares the species itself; the sums are added
+  // in the order of the chunks, as by one block, so that both forms give the same bits.
   extern __shared__ __align__(16) char s_raw[];
   const TileSmem s = tile_smem(s_raw);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -416,8 +445,9 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
     s.lam[NSP * 32 + lane] = 0;                 // the unit factor
     s.alp[NSP * 32 + lane] = 0;
   }
+  const int rank = split ? (int)(blockIdx.x % NCH) : 0, blocks = split ? NCH : 1;
 #pragma unroll 1
-  for (i64 tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+  for (i64 tile = blockIdx.x / blocks; tile < tiles; tile += gridDim.x / blocks) {
     const i64 p = tile * 32 + lane;
     const i64 pc = p < n ? p : n - 1;
     const double* Yp = g_Y + pc;
@@ -451,7 +481,7 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         __syncthreads();
       }
       if (w == 0) {
-        if (energy_mode && p < n) {
+        if (energy_mode && p < n && rank == 0) {
           if (!ok) atomicAdd(g_fail, 1ull);
           g_Tout[p] = T;
         }
@@ -491,7 +521,7 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         const u64 yb = (u64)s.alp[k * 32 + lane];
         const int ye = (int)(yb >> 52) & 0x7ff;
         const bool zero = (yb << 1) == 0ull;
-        bad |= (ye == 0 && !zero) || ye > 1023 + 8;
+        bad |= (ye == 0 && !zero) || ye > 1023;
         i64 ly = pfx::log2_of(__longlong_as_double((i64)(yb & 0x7fffffffffffffffull)), t_log2);
         ly = zero ? pfx::LG_ZERO : (ly | (i64)(yb >> 63));
         s.lam[k * 32 + lane] = q;
@@ -503,7 +533,7 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
     const Pair u = s.sc->u[lane], v = s.sc->v[lane];
     const bool open = s.sc->bad[lane] != 0;
 #pragma unroll 1
-    for (int ch = 0; ch < NCH; ++ch) {
+    for (int ch = rank; ch < (split ? rank + 1 : NCH); ++ch) {
       const int* seg = t_seg + (ch * NW + w) * (NCLS + 1);
       // every other warp takes the plain reactions last: they load the integer pipes, the
       // others the FP64 pipe
@@ -520,16 +550,25 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
       // species sums: per owned species the rows with nu = +1, with -1 (both padded to
       // multiples of 4 with the zero row) and with other nu
       const char* R = (const char*)(s.R + lane);
+      // a warp's lists follow one another in the entry table: the next four entries and the
+      // next species' header are loaded while the last ones are summed (both tables end
+      // with a spare element)
+      int4 qn = __ldg((const int4*)t_wl + (ch * NW + w) * KPO);              // first entry, ends of the three lists
+      int2 on = __ldg((const int2*)t_wo + (ch * NW + w) * KPO);              // species, head-room bits + 256 others
+      int4 rn = __ldg((const int4*)(t_we + qn.x));
 #pragma unroll 1
       for (int i = 0; i < KPO; ++i) {
-        const int4 q = __ldg((const int4*)t_wl + (ch * NW + w) * KPO + i);   // first entry, ends of the three lists
-        const int2 o = __ldg((const int2*)t_wo + (ch * NW + w) * KPO + i);   // species, head-room bits + 256 others
+        const int4 q = qn;
+        const int2 o = on;
         if (o.x < 0) break;
+        qn = __ldg((const int4*)t_wl + (ch * NW + w) * KPO + i + 1);
+        on = __ldg((const int2*)t_wo + (ch * NW + w) * KPO + i + 1);
         const int hb = o.y & 0xff;
         i64 a = 0;
         int e = 0;
         auto quad = [&](int j, auto sign) {
-          const int4 r = __ldg((const int4*)(t_we + j));
+          const int4 r = rn;
+          rn = __ldg((const int4*)(t_we + j + 4));
           const i64 v0 = *(const i64*)(R + r.x), v1 = *(const i64*)(R + r.y), v2 = *(const i64*)(R + r.z),
                     v3 = *(const i64*)(R + r.w);
           const int e0 = (int)v0 & 4095, e1 = (int)v1 & 4095, e2 = (int)v2 & 4095, e3 = (int)v3 & 4095;
@@ -547,8 +586,11 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
           a = tile_sar(a, en - e) + (i64)__ldg(t_wc + j) * tile_sar(x, en + hb - e0);
           e = en;
         }
+        if (q.w > q.z) rn = __ldg((const int4*)(t_we + q.w));
         double v = tile_to_double(a, e + hb - RATE_E, 61);
-        if (p < n) {
+        if (split) {
+          ((double*)s.lam)[o.x * 32 + lane] = v;     // the species arrays are free after the only chunk
+        } else if (p < n) {
           double* out = g_omega + o.x * n + p;
           if (ch > 0) v += *out;
           if (open && o.x == 0) v = __longlong_as_double(TILE_OPEN);
@@ -557,5 +599,35 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
       }
       __syncthreads();
     }
+#if NCH > 1
+    if (split) {
+      auto barrier = [] {
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+      };
+      auto remote = [](const void* a, int r) {
+        unsigned b, l = (unsigned)__cvta_generic_to_shared(a);
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(l), "r"(r));
+        return b;
+      };
+      barrier();
+#pragma unroll 1
+      for (int k = rank + w * NCH; k < NSP; k += NW * NCH) {
+        double v = 0.0;
+        int any = 0;
+#pragma unroll
+        for (int r = 0; r < NCH; ++r) {
+          double x;
+          int b;
+          asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x) : "r"(remote(s.lam + k * 32 + lane, r)) : "memory");
+          asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(b) : "r"(remote(s.sc->bad + lane, r)) : "memory");
+          v = r ? x + v : x;
+          any |= b;
+        }
+        if (any && k == 0) v = __longlong_as_double(TILE_OPEN);
+        if (p < n) g_omega[k * n + p] = v;
+      }
+      barrier();                                 // the other blocks read this one's arrays
+    }
+#endif
   }
 }

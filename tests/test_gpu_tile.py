@@ -86,6 +86,25 @@ def test_absent_negative_and_tiny_mass_fractions(mechs, name, idx):
     assert np.all(w[G == 0.0] == 0.0)          # no reaction of these species runs: exactly zero
 
 
+def test_split_tiles_give_the_same_bits(mech_files):
+    """160 species: few tiles run one cluster of blocks per tile (a block per chunk of reactions),
+    many run one block per tile; both give the same bits, open states included."""
+    from paper_2503_24286_gb300 import binding as B
+    m, orc = B.Mechanism(mech_files[0][4], "variant=warp"), O.Oracle(mech_files[0][4])
+    assert m.stat("tile_chunks") > 1
+    n = 32 * 200
+    rho, T, Y = _states(orc, 4, n, 41)
+    T[[7, 40]] = [280.0, 4990.0]
+    assert m.stat("tile_t_lo") > 280.0
+    e = orc.internal_energy(T, Y)
+    full, Tf = m.net_production_rates(_t(rho), _t(Y), e=_t(e))
+    for a, b in ((0, 1), (0, 33), (64, 640), (n - 95, n)):
+        w, Ts = m.net_production_rates(_t(rho[a:b]), _t(Y[:, a:b]), e=_t(e[a:b]))
+        assert torch.equal(w, full[:, a:b]) and torch.equal(Ts, Tf[a:b])
+    m.nonconverged()
+    _check(m, orc, rho[:100], T[:100], Y[:, :100])
+
+
 def test_nan_stays_in_its_state(mechs):
     m, orc = mechs["gri"]
     rho, T, Y = _states(orc, 1, 100, 37)
