@@ -1506,12 +1506,20 @@ void emit_transport_kernel(Src& s, const Mechanism& m, int blk, bool gstore) {
   s << "\n// mu, kappa, D_km of the mixture-averaged model (each output nullable)\n";
   s << "extern \"C\" __global__ void __launch_bounds__(" << blk << ") pyro_transport(i64 n, const double* __restrict__ g_T,\n"
        "    const double* __restrict__ g_Y, double* __restrict__ g_mu, double* __restrict__ g_kappa,\n"
-       "    double* __restrict__ g_Dm, double* __restrict__ g_store) {\n"
+       "    double* __restrict__ g_Dm, double* __restrict__ g_store, int open_only) {\n"
+       "  // open_only: only the states that the tile kernel left open (pyro_transport.cuh)\n"
+       "  const double* mark = g_mu ? g_mu : g_kappa ? g_kappa : g_Dm;\n"
+       "  if (open_only) {\n    bool any = false;\n"
+       "    #pragma unroll 8\n"
+       "    for (i64 p = (i64)blockIdx.x * BLKD + threadIdx.x; p < n; p += (i64)gridDim.x * BLKD)\n"
+       "      any |= __double_as_longlong(mark[p]) == " << kTileOpen << ";\n"
+       "    if (!__syncthreads_or(any)) return;\n  }\n"
        "  __shared__ double s_exp[512];\n  __shared__ double s_log[256];\n  extern __shared__ double s_dyn[];\n"
        "  double* sX = " << (gstore ? "g_store + (i64)blockIdx.x * 3 * NSP * BLKD" : "s_dyn") << ";\n"
        "  double* sV = sX + NSP * BLKD; double* sW = sV + NSP * BLKD;\n"
        "  pyro_load_tables(s_exp, s_log);\n  __syncthreads();\n  const int t = threadIdx.x;\n"
        "  for (i64 p = (i64)blockIdx.x * BLKD + t; p < n; p += (i64)gridDim.x * BLKD) {\n"
+       "    if (open_only && __double_as_longlong(mark[p]) != " << kTileOpen << ") continue;\n"
        "    const double* Yp = g_Y + p;\n"
        "    const double T = g_T[p];\n    const double L = pdm::log(T, s_log);\n    const double sqT = sqrt(T);\n"
        "    double ys = 0.0;\n";
@@ -2357,6 +2365,15 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
     out.stats["transport_fp64_ops_per_point"] = 7 + 1 + N + 4 + N * 23.0 + 4 + 3.0 * N * N + 13.0 * N + 10.0 * npair + 6.0 * N;
   }
   out.stats["has_transport"] = m.has_transport ? 1 : 0;
+  {
+    const TransportTile t = emit_transport_tile(m);
+    out.stats["transport_tile"] = t.source.empty() ? 0 : 1;
+    if (!t.source.empty()) {
+      out.group_sources["ttr"] = t.source;
+      out.transport_warps = t.warps;
+      out.smem_dyn_bytes_transport_tile = t.smem_bytes;
+    }
+  }
   {
     // Crank-Nicolson: temperature solve + Newton-system assembly + batched solve
     int ns2 = 0;

@@ -25,8 +25,16 @@ constexpr int kSmemMaxBlock = 227 * 1024;
 
 TileEmit emit_tile_unit(const Mechanism& m);
 
-// The kernel text (embedded at build time).
+struct TransportTile {
+  std::string source;      // empty: no transport section, or its fits do not suit the tables
+  int warps = 0, smem_bytes = 0;
+};
+
+TransportTile emit_transport_tile(const Mechanism& m);
+
+// The kernel texts (embedded at build time).
 extern const char* kFixedMathSource;
 extern const char* kTileSource;
+extern const char* kTransportSource;
 
 }  // namespace pyro

@@ -116,9 +116,9 @@ const char* kArch = "sm_103a";
 // Compile CUDA C to a cubin for sm_103a with NVRTC.
 bool nvrtc_compile(const std::string& src, std::vector<char>& cubin, std::string& log) {
   nvrtcProgram prog;
-  const char* hdrs[] = {kDeviceMathSource, kFixedMathSource, kTileSource};
-  const char* names[] = {"pyro_device_math.cuh", "pyro_fixed_math.cuh", "pyro_tile.cuh"};
-  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 3, hdrs, names) != NVRTC_SUCCESS) {
+  const char* hdrs[] = {kDeviceMathSource, kFixedMathSource, kTileSource, kTransportSource};
+  const char* names[] = {"pyro_device_math.cuh", "pyro_fixed_math.cuh", "pyro_tile.cuh", "pyro_transport.cuh"};
+  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 4, hdrs, names) != NVRTC_SUCCESS) {
     log = "nvrtcCreateProgram failed";
     return false;
   }
@@ -156,7 +156,8 @@ int compile_cached(const std::string& src, bool use_cache, std::vector<char>& cu
   std::string key_src = src + std::string(kDeviceMathSource) + kArch + std::to_string(nv_major) + "." +
                         std::to_string(nv_minor);
   if (src.find("pyro_fixed_math.cuh") != std::string::npos) key_src += kFixedMathSource;
-  if (src.find("pyro_tile.cuh") != std::string::npos) key_src += kTileSource;
+  if (src.find("\"pyro_tile.cuh\"") != std::string::npos) key_src += kTileSource;
+  if (src.find("\"pyro_transport.cuh\"") != std::string::npos) key_src += kTransportSource;
   char hex[32];
   std::snprintf(hex, sizeof hex, "%016llx", (unsigned long long)fnv1a(key_src));
   std::string dir = cache_dir(), path = dir + "/pyro_" + hex + ".cubin";
@@ -527,7 +528,7 @@ const char* group_kernel(const std::string& g) {
   return g == "jvp" ? "pyro_jvp" : g == "vjp" ? "pyro_vjp" : g == "jad" ? "pyro_jacobian_adiabatic"
        : g == "cn" ? "pyro_cn_assemble" : g == "tr" ? "pyro_transport" : g == "wfwd" ? "pyro_omega_warp"
        : g == "wjvp" ? "pyro_jvp_warp" : g == "wvjp" ? "pyro_vjp_warp" : g == "wjac" ? "pyro_jacobian_cta"
-       : g == "wjad" ? "pyro_jacobian_adiabatic_cta" : g == "tile" ? "pyro_omega_tile" : "pyro_jacobian";
+       : g == "wjad" ? "pyro_jacobian_adiabatic_cta" : g == "tile" ? "pyro_omega_tile" : g == "ttr" ? "pyro_transport_tile" : "pyro_jacobian";
 }
 
 // Compile (in parallel threads, cached on disk) and load the named derivative
@@ -574,6 +575,10 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
       G.block = 32 * h->emitted.warp_wpb.at(todo[i]);
       G.smem = h->emitted.smem_dyn_bytes_warp.at(todo[i]);
     }
+    if (todo[i] == "ttr") {
+      G.block = 32 * h->emitted.transport_warps;
+      G.smem = h->emitted.smem_dyn_bytes_transport_tile;
+    }
     if (todo[i] == "tile") {
       G.block = 32 * h->emitted.tile_warps;
       G.smem = h->emitted.smem_dyn_bytes_tile;
@@ -612,7 +617,7 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
       h->emitted.stats[todo[i] + "_active_clusters"] = ncl;
     }
     if (h->emitted.stats["deriv_store_global"] > 0 && todo[i] != "jac" && todo[i] != "jad" && todo[i] != "cn" &&
-        todo[i] != "tile" && todo[i][0] != 'w') {
+        todo[i] != "tile" && todo[i] != "ttr" && todo[i][0] != 'w') {
       size_t bytes = (size_t)h->num_sms * nb * 4 * h->m.n_species() * h->opt.deriv_block * sizeof(double);
       cudaError_t e = cudaMalloc(&G.store, bytes);
       if (e != cudaSuccess) return fail(PYRO_ECUDA, std::string("species-array store allocation: ") + cudaGetErrorString(e));
@@ -1049,6 +1054,7 @@ int pyro_mech_prepare(const pyro_mech* hc, const char* kernels) {
       else if (item == "transport" || item == "tr") {
         if (h->emitted.stats["has_transport"] <= 0) return fail(PYRO_EMECH, "the mechanism has no transport section");
         names.push_back("tr");
+        if (h->emitted.stats["transport_tile"] > 0) names.push_back("ttr");
       }
       else if (!item.empty()) return fail(PYRO_EINVAL, "unknown kernel group '" + item + "'");
     }
@@ -1129,14 +1135,23 @@ int pyro_transport(const pyro_mech* hc, int64_t n, const double* T, const double
   if (h->emitted.stats["has_transport"] <= 0) return fail(PYRO_EMECH, "the mechanism has no transport section");
   if (n == 0) return PYRO_OK;
   if (int rc = check_device(h)) return rc;
-  if (int rc = ensure_groups(h, {"tr"})) return rc;
+  const bool tile = h->emitted.stats["transport_tile"] > 0;
+  if (int rc = ensure_groups(h, tile ? std::vector<std::string>{"tr", "ttr"} : std::vector<std::string>{"tr"})) return rc;
   pyro_mech::Group& G = h->groups["tr"];
   const int64_t NS = h->m.n_species();
   return with_args(h, n, {{T, 1, 8, true, false}, {Y, NS, 8, true, false}, {mu, 1, 8, false, true},
                           {kappa, 1, 8, false, true}, {D_mix, NS, 8, false, true}},
                    stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
                      long long nn = nc;
-                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &G.store};
+                     int open_only = tile ? 1 : 0;
+                     if (tile) {   // 32 states per block; the FP64 kernel then takes the states it left open
+                       const pyro_mech::Group& t = h->groups["ttr"];
+                       void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4]};
+                       const unsigned grid = (unsigned)std::min((nc + 31) / 32, (int64_t)h->num_sms * t.blocks_per_sm);
+                       CUresult r = driver().LaunchKernel(t.f, grid, 1, 1, t.block, 1, 1, t.smem, as_stream(st), params, nullptr);
+                       if (r != CUDA_SUCCESS) return fail(PYRO_ECUDA, "kernel launch: " + cu_err(r));
+                     }
+                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &G.store, &open_only};
                      return launch_deriv(h, G, nc, st, params);
                    });
 }
