@@ -229,7 +229,7 @@ TileEmit emit_tile_unit(const Mechanism& m) {
   // the rows in more than one chunk two blocks lose (8.3 ms and more).  10 species / 21
   // reactions: eight blocks of 4 warps 0.81 ms, four of 8 warps 0.96 ms; 160 / 1100
   // (2^18 states): one block of 24 warps 5.6 ms, of 16 warps 6.4 ms.
-  const int fixed_bytes = 8192 + 512 * (N + 1) + 1920 + 256;
+  const int fixed_bytes = 8192 + 512 * (N + 1) + 2064 + 256;
   int warps = rows_all < 48 ? 4 : rows_all < 120 ? 8 : 12;
   int minb = 24 / warps + (warps == 4 ? 2 : 0);
   auto red = [](int w) { return w * 256 + 6 * 256 + 14 * 128 + w * 13 * 128; };   // scratch of the temperature solve, in the rows
@@ -460,12 +460,12 @@ TileEmit emit_tile_unit(const Mechanism& m) {
   array(o, "__align__(8) int", "t_wo", wo);
   array(o, "__align__(16) int", "t_we", we);
   array(o, "signed char", "t_wc", wc);
-  o << "#define TILE_PLAIN";
+  o << "#define TILE_PLAIN(SGN)";
   for (auto& kv : class_id) {
     if (kv.first == 8) continue;
     const int c = kv.second;
     o << " \\\n  { const int a = __ldg(seg + " << c << "), b = __ldg(seg + " << c + 1 << "); if (a < b) tile_plain<"
-      << (kv.first & 2 ? 3 : 2) << ", " << (kv.first & 1 ? "true" : "false") << ">(s, a, b, u, v, lane); }";
+      << (kv.first & 2 ? 3 : 2) << ", " << (kv.first & 1 ? "true" : "false") << ", SGN>(s, a, b, u, v, lane); }";
   }
   o << "\n#include \"pyro_tile.cuh\"\n";
   out.source = o.str();

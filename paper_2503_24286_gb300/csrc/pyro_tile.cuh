@@ -37,7 +37,9 @@ struct TileScalars {
   double T[32], ysum[32];
   Pair u[32], v[32], t[32];      // log2(T)/16, T_V/T, T/T_T
   i64 lgT[32], lgrho[32];
+  float Tf[32];
   int bad[32];
+  int neg;                       // the tile has negative mass fractions or densities
 };
 
 // A rate is a 64-bit word r: read as an integer it is m 2^(e - 61 - RATE_E) with
@@ -116,17 +118,18 @@ __device__ __forceinline__ u64 tile_shr(u64 v, int n) {
   return r;
 }
 
-// the rate 2^xf - 2^xr (REV false: 2^xf) with the signs in the lowest bits
-template <bool REV>
+// the rate 2^xf - 2^xr (REV false: 2^xf) with the signs in the lowest bits (SGN false: all
+// are clear)
+template <bool REV, bool SGN>
 __device__ __forceinline__ i64 tile_rate(i64 xf, i64 xr, const u64* tab) {
   const u64 f = pfx::exp2_mant(xf, tab);
-  const i64 sf = -(xf & 1ll);
+  const i64 sf = SGN ? -(xf & 1ll) : 0ll;
   const int nf = (int)(xf >> pfx::LG_F);
   i64 m;
   int e = max(nf, 50 - RATE_E);
   if (REV) {
     const u64 g = pfx::exp2_mant(xr, tab);
-    const i64 sg = -(xr & 1ll);
+    const i64 sg = SGN ? -(xr & 1ll) : 0ll;
     const int ng = (int)(xr >> pfx::LG_F);
     e = max(e, ng);
     // one's complement negation: off by one in 2^61
@@ -191,18 +194,27 @@ __device__ __forceinline__ void tile_energy(const TileSmem& s, const double* __r
     __syncthreads();
   }
   const float* b = s.b + lane;
-  float Tf = pdm::to_float_trunc(T0);
-  const float eRf = pdm::to_float_trunc(e * T_INV_R);
-  for (int it = 0; it < 40; ++it) {
-    const float* c = b + (Tf >= (float)TMID ? 6 * 32 : 0);
-    const float c0 = c[0], c1 = c[32], c2 = c[64], c3 = c[96], c4 = c[128], c5 = c[160];
-    const float ef = fmaf(Tf, fmaf(Tf, fmaf(Tf, fmaf(Tf, fmaf(Tf, c5, c4), c3), c2), c1), c0);
-    const float cvf = fmaf(Tf, fmaf(Tf, fmaf(Tf, fmaf(Tf, 5.f * c5, 4.f * c4), 3.f * c3), 2.f * c2), c1);
-    const float Tn = fminf(fmaxf(Tf + (eRf - ef) * __frcp_rn(cvf), 100.f), 5000.f);
-    const bool conv = fabsf(Tn - Tf) <= 1e-5f * Tn;
-    Tf = Tn;
-    if (conv) break;
+  if (w == 0) {
+    float c[12];
+#pragma unroll
+    for (int q = 0; q < 12; ++q) c[q] = b[q * 32];
+    float Tf = pdm::to_float_trunc(T0);
+    const float eRf = pdm::to_float_trunc(e * T_INV_R);
+    for (int it = 0; it < 40; ++it) {
+      const bool h = Tf >= (float)TMID;
+      const float c0 = h ? c[6] : c[0], c1 = h ? c[7] : c[1], c2 = h ? c[8] : c[2];
+      const float c3 = h ? c[9] : c[3], c4 = h ? c[10] : c[4], c5 = h ? c[11] : c[5];
+      const float ef = fmaf(Tf, fmaf(Tf, fmaf(Tf, fmaf(Tf, fmaf(Tf, c5, c4), c3), c2), c1), c0);
+      const float cvf = fmaf(Tf, fmaf(Tf, fmaf(Tf, fmaf(Tf, 5.f * c5, 4.f * c4), 3.f * c3), 2.f * c2), c1);
+      const float Tn = fminf(fmaxf(Tf + (eRf - ef) * __frcp_rn(cvf), 100.f), 5000.f);
+      const bool conv = fabsf(Tn - Tf) <= 1e-5f * Tn;
+      Tf = Tn;
+      if (conv) break;
+    }
+    s.sc->Tf[lane] = Tf;
   }
+  __syncthreads();
+  const float Tf = s.sc->Tf[lane];
   bool hi = Tf >= (float)TMID;
   {
     // the collapse of one range on the integer pipe (exact up to the 2^-61 of Y)
@@ -269,14 +281,14 @@ __device__ __forceinline__ void tile_energy(const TileSmem& s, const double* __r
 // plain reactions with up to NF factors a side (missing ones: the unit factor);
 // REV: reversible.  A flag marks a duplicate of a reaction before it in this warp,
 // whose rate is added to the same row.
-template <int NF, bool REV>
+template <int NF, bool REV, bool SGN>
 __device__ __forceinline__ void tile_plain(const TileSmem& s, int i0, int i1, Pair u, Pair v, int lane) {
   const char* lam = (const char*)(s.lam + lane);
   const char* alp = (const char*)(s.alp + lane);
   char* R = (char*)(s.R + lane);
   const int4* r = (const int4*)(t_rx + i0 * 8);
   int4 r0 = __ldg(r), r1 = __ldg(r + 1), r2 = __ldg(r + 2), r3 = __ldg(r + 3);
-#pragma unroll 1
+#pragma unroll 2
   for (int i = i0; i < i1; ++i) {
     const int4 c0 = r0, c1 = r1, c2 = r2, c3 = r3;
     r += 4;                                    // the next record (the table ends with a spare one)
@@ -298,7 +310,7 @@ __device__ __forceinline__ void tile_plain(const TileSmem& s, int i0, int i1, Pa
       Xr += at(alp, c2.y) + at(alp, c2.z);
       if (NF > 2) Xr += at(alp, c2.w);
     }
-    i64 rate = tile_rate<REV>(Xf, Xr, s.exp2);
+    i64 rate = tile_rate<REV, SGN>(Xf, Xr, s.exp2);
     i64* o = (i64*)(R + c3.x);
     if (c3.y) rate = tile_add(*o, rate);
     *o = rate;
@@ -420,7 +432,7 @@ __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, in
       const int k = (int)((q == 0 ? (fa >> 48) : (fb >> (16 * (q - 1)))) & 0xffff) * 32;
       Xr += alp[k];
     }
-    s.R[(int)((fb >> 32) & 0xffff) * 32 + lane] = tile_rate<true>(X + Xf, X + Xr, s.exp2);
+    s.R[(int)((fb >> 32) & 0xffff) * 32 + lane] = tile_rate<true, true>(X + Xf, X + Xr, s.exp2);
   }
 }
 
@@ -497,6 +509,9 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         s.sc->v[lane] = pfx::split(pfx::frac_of(T_V * pdm::rcp(Ts)));
         s.sc->t[lane] = pfx::split(pfx::frac_of(Ts * (1.0 / T_T)));
         s.sc->bad[lane] = in ? 0 : 1;
+        if (lane == 0) s.sc->neg = 0;
+        __syncwarp();
+        if (__double_as_longlong(rho) < 0) s.sc->neg = 1;
       }
       if (w == NW - 1) {
         double a = 0.0;
@@ -524,6 +539,7 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         bad |= (ye == 0 && !zero) || ye > 1023;
         i64 ly = pfx::log2_of(__longlong_as_double((i64)(yb & 0x7fffffffffffffffull)), t_log2);
         ly = zero ? pfx::LG_ZERO : (ly | (i64)(yb >> 63));
+        if ((i64)yb < 0 && !zero) s.sc->neg = 1;
         s.lam[k * 32 + lane] = q;
         s.alp[k * 32 + lane] = q + ly + lgrho;
       }
@@ -531,7 +547,7 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
       __syncthreads();
     }
     const Pair u = s.sc->u[lane], v = s.sc->v[lane];
-    const bool open = s.sc->bad[lane] != 0;
+    const bool open = s.sc->bad[lane] != 0, signs = s.sc->neg != 0;
 #pragma unroll 1
     for (int ch = rank; ch < (split ? rank + 1 : NCH); ++ch) {
       const int* seg = t_seg + (ch * NW + w) * (NCLS + 1);
@@ -540,7 +556,11 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
 #pragma unroll 1
       for (int half = 0; half < 2; ++half) {
         if ((w & 1) == half) {
-          TILE_PLAIN
+          if (signs) {
+            TILE_PLAIN(true)
+          } else {
+            TILE_PLAIN(false)
+          }
         } else {
           const int a = __ldg(seg + NCLS - 1), b = __ldg(seg + NCLS);
           if (a < b) tile_other(s, a, b, lane, rho, Yp, n);
@@ -578,8 +598,8 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
           const i64 b = (tile_sar(v0, t - e0) + tile_sar(v1, t - e1)) + (tile_sar(v2, t - e2) + tile_sar(v3, t - e3));
           if (decltype(sign)::minus) a -= b; else a += b;
         };
-        for (int j = q.x; j < q.y; j += 4) quad(j, TilePlus());
-        for (int j = q.y; j < q.z; j += 4) quad(j, TileMinus());
+        _Pragma("unroll 2") for (int j = q.x; j < q.y; j += 4) quad(j, TilePlus());
+        _Pragma("unroll 2") for (int j = q.y; j < q.z; j += 4) quad(j, TileMinus());
         for (int j = q.z; j < q.z + (o.y >> 8); ++j) {
           const i64 x = *(const i64*)(R + __ldg(t_we + j));
           const int e0 = (int)x & 4095, en = max(e, e0);
