@@ -23,7 +23,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 # device sources compiled at run time (NVRTC), embedded as strings
 EMBED = {"pyro_device_math.cuh": "kDeviceMathSource", "pyro_fixed_math.cuh": "kFixedMathSource",
-         "pyro_tile.cuh": "kTileSource", "pyro_transport.cuh": "kTransportSource"}
+         "pyro_tile.cuh": "kTileSource", "pyro_transport.cuh": "kTransportSource",
+         "pyro_tile_jvp.cuh": "kTileJvpSource"}
 
 
 def _embed_sources() -> str:

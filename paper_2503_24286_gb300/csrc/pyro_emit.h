@@ -43,6 +43,8 @@ struct EmitResult {
   int smem_dyn_bytes_jac = 0;             // dynamic shared memory of the Jacobian-type kernels
   int transport_warps = 0;                // warps per block of the transport tile kernel
   int smem_dyn_bytes_transport_tile = 0;  // its dynamic shared memory
+  int jvp_tile_warps = 0;                 // warps per block of the JVP's tile kernel
+  int smem_dyn_bytes_jvp_tile = 0;        // its dynamic shared memory
   int tile_warps = 0;                     // warps per block of the tile kernel
   int tile_chunks = 0;                    // reaction chunks per tile
   int smem_dyn_bytes_tile = 0;            // dynamic shared memory of the tile kernel

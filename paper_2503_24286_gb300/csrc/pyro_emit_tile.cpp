@@ -93,7 +93,7 @@ std::vector<std::string> as_d(const std::vector<double>& v) {
 
 }  // namespace
 
-TileEmit emit_tile_unit(const Mechanism& m) {
+TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
   TileEmit out;
   const int N = m.n_species(), NR = m.n_reactions();
   if (N < 1 || N > 1022 || NR < 1) { out.why = "no reactions, or more than 1022 species"; return out; }
@@ -130,7 +130,10 @@ TileEmit emit_tile_unit(const Mechanism& m) {
     for (int i = 0; i <= 200; ++i) {
       const ld T = lo * powl(T_HI / lo, i / 200.0L);
       const int rg = T >= tmid ? 1 : 0;
-      for (int k = 0; k < N; ++k) lam[k] = lambda(m.species[k], rg, T);
+      for (int k = 0; k < N; ++k) {
+        lam[k] = lambda(m.species[k], rg, T);
+        if (deriv && !(fabsl(lam[k]) < 1000)) return false;      // exp(L_k) itself is used
+      }
       for (int j = 0; j < NR; ++j) {
         ld f = 0, g = 0;
         for (auto& p : m.reactions[j].reactants) { f += p.second * lam[p.first]; g += p.second * logl((ld)m.species[p.first].W) * LOG2E; }
@@ -154,6 +157,7 @@ TileEmit emit_tile_unit(const Mechanism& m) {
   // ---- species tables ----------------------------------------------------------
   Fix fx;
   std::vector<i64> sp((size_t)N * 16);
+  std::vector<double> hc;                        // h_k/(RT) = h0 + ... + h4 T^4 + h5/T
   std::vector<double> ed((size_t)N * 12), iw(N);
   // integer energy coefficients: column q scaled by 2^xs[q], the largest in [2^(hb-1), 2^hb),
   // so that sums over the species stay below 2^63 while sum |Y| < 2 (TileDot)
@@ -187,6 +191,7 @@ TileEmit emit_tile_unit(const Mechanism& m) {
       q[5] = fx.coef(16 * (1.0L - a[0]));
       q[6] = fx.coef((ld)a[5] * LOG2E / T_V);
       q[7] = 0;
+      hc.insert(hc.end(), C.h[r], C.h[r] + 6);
       for (int i = 0; i < 6; ++i) {
         ed[((size_t)k * 2 + r) * 6 + i] = C.d[r][i];
         ex[((size_t)k * 2 + r) * 6 + i] = fx.pair(llroundl(ldexpl((ld)C.d[r][i], xs[i])));
@@ -229,7 +234,7 @@ TileEmit emit_tile_unit(const Mechanism& m) {
   // the rows in more than one chunk two blocks lose (8.3 ms and more).  10 species / 21
   // reactions: eight blocks of 4 warps 0.81 ms, four of 8 warps 0.96 ms; 160 / 1100
   // (2^18 states): one block of 24 warps 5.6 ms, of 16 warps 6.4 ms.
-  const int fixed_bytes = 8192 + 512 * (N + 1) + 2064 + 256;
+  const int fixed_bytes = deriv ? 8192 + 1024 * (N + 1) + 32 * (8 * 8 + 3 * 8 + 8 + 4) + 256 : 8192 + 512 * (N + 1) + 2064 + 256;
   int warps = rows_all < 48 ? 4 : rows_all < 120 ? 8 : 12;
   int minb = 24 / warps + (warps == 4 ? 2 : 0);
   auto red = [](int w) { return w * 256 + 6 * 256 + 14 * 128 + w * 13 * 128; };   // scratch of the temperature solve, in the rows
@@ -270,6 +275,7 @@ TileEmit emit_tile_unit(const Mechanism& m) {
   for (auto& kv : class_id) kv.second = ncls++;
 
   std::vector<i64> rx, ax;
+  std::vector<double> rd, fxa;                   // b, theta of a record; FP64 companions of ax
   std::vector<int> seg;
   std::vector<int> row_of(groups.size());
   for (int ch = 0; ch < chunks; ++ch) {
@@ -300,6 +306,8 @@ TileEmit emit_tile_unit(const Mechanism& m) {
             }
             const std::vector<int> fr = side_factors(r.reactants), fp = r.reversible ? side_factors(r.products) : std::vector<int>();
             auto at = [](const std::vector<int>& f, size_t i) { return (u64)(i < f.size() ? f[i] : 0); };
+            rd.push_back(r.b);
+            rd.push_back(r.theta);
             if (cls == 0) {       // byte offsets into the species arrays and of the row
               auto off = [&](const std::vector<int>& f, size_t i) { return (u64)((i < f.size() ? f[i] : N) * 256); };
               rec[3] = (i64)(off(fr, 0) | off(fr, 1) << 32);
@@ -314,6 +322,7 @@ TileEmit emit_tile_unit(const Mechanism& m) {
             rec[5] = (i64)ax.size();
             if (cls) {
               std::vector<i64> x(16, 0);
+              std::vector<double> fd(16, 0.0);
               if (cls == 5) {
                 const size_t nn = r.plog.size();
                 x[1] = (i64)nn;
@@ -322,6 +331,7 @@ TileEmit emit_tile_unit(const Mechanism& m) {
                   const ld lp = log2l((ld)r.plog[i].p);
                   x.push_back(fx.lg(lp));
                   x.push_back(dbits(i + 1 < nn ? (double)(1.0L / (log2l((ld)r.plog[i + 1].p) - lp)) : 0.0));
+                  for (double v : {0.0, 0.0, 0.0, r.plog[i].b, r.plog[i].theta}) fd.push_back(v);
                   x.push_back(fx.lg(f.c)); x.push_back(fx.coef(16 * f.b)); x.push_back(fx.coef(-f.theta * LOG2E / T_V));
                 }
                 if (nn < 2) fx.bad = true;
@@ -338,10 +348,14 @@ TileEmit emit_tile_unit(const Mechanism& m) {
                 x[2] = fx.lg(log2l((ld)r.A0) - log2l((ld)r.A));
                 x[3] = fx.coef(16 * ((ld)r.b0 - r.b));
                 x[4] = fx.coef(-((ld)r.theta0 - r.theta) * LOG2E / T_V);
+                fd[0] = r.b0 - r.b;
+                fd[1] = r.theta0 - r.theta;
               }
               // a term that is below 2^-1100 at every T of the range is left out
               auto term = [&](ld slope, ld at_lo) { return at_lo > -1100 && (fabsl(slope) < 4000 || (fx.bad = true)); };
               auto add = [&](i64 c, ld t, ld v) {      // an exponential of S: c, slopes in t and v
+                fd[2 + 2 * x[1]] = (double)(t / (T_T * LOG2E));            // its logarithmic slope in T: g0 + g2/T^2
+                fd[3 + 2 * x[1]] = (double)(-v * T_V / LOG2E);
                 i64* e = &x[5 + 3 * x[1]++];
                 e[0] = c; e[1] = fx.coef(t); e[2] = fx.coef(v);
               };
@@ -360,9 +374,12 @@ TileEmit emit_tile_unit(const Mechanism& m) {
                 if (term(sc, sc * t_lo / T_T)) add(0, sc, 0);
                 x[14] = fx.lg(log2l(d));
                 x[15] = fx.coef(16 * e);
+                fd[8] = (double)e;
               }
               if (x.size() % 2) x.push_back(0);      // 16-byte units
+              fd.resize(x.size(), 0.0);
               ax.insert(ax.end(), x.begin(), x.end());
+              fxa.insert(fxa.end(), fd.begin(), fd.end());
             }
             rx.insert(rx.end(), rec, rec + 8);
           }
@@ -460,14 +477,20 @@ TileEmit emit_tile_unit(const Mechanism& m) {
   array(o, "__align__(8) int", "t_wo", wo);
   array(o, "__align__(16) int", "t_we", we);
   array(o, "signed char", "t_wc", wc);
-  o << "#define TILE_PLAIN(SGN)";
+  if (deriv) {
+    array(o, "__align__(16) double", "t_rd", as_d(rd));
+    array(o, "double", "t_fx", as_d(fxa));
+    array(o, "double", "t_h", as_d(hc));
+  }
+  o << (deriv ? "#define TILE_PLAIN" : "#define TILE_PLAIN(SGN)");
   for (auto& kv : class_id) {
     if (kv.first == 8) continue;
     const int c = kv.second;
-    o << " \\\n  { const int a = __ldg(seg + " << c << "), b = __ldg(seg + " << c + 1 << "); if (a < b) tile_plain<"
-      << (kv.first & 2 ? 3 : 2) << ", " << (kv.first & 1 ? "true" : "false") << ", SGN>(s, a, b, u, v, lane); }";
+    o << " \\\n  { const int a = __ldg(seg + " << c << "), b = __ldg(seg + " << c + 1 << "); if (a < b) "
+      << (deriv ? "jvp_plain<" : "tile_plain<") << (kv.first & 2 ? 3 : 2) << ", " << (kv.first & 1 ? "true" : "false")
+      << (deriv ? ">(s, a, b, u, v, u1, u2, lane); }" : ", SGN>(s, a, b, u, v, lane); }");
   }
-  o << "\n#include \"pyro_tile.cuh\"\n";
+  o << (deriv ? "\n#include \"pyro_tile_jvp.cuh\"\n" : "\n#include \"pyro_tile.cuh\"\n");
   out.source = o.str();
   out.warps = warps;
   out.smem_bytes = fixed_bytes + tile_rows * 256;

@@ -23,7 +23,8 @@ constexpr int kSmemPerSm = 228 * 1024;
 constexpr int kSmemPerBlock = 1024;
 constexpr int kSmemMaxBlock = 227 * 1024;
 
-TileEmit emit_tile_unit(const Mechanism& m);
+// deriv: the unit of the Jacobian-vector product (pyro_tile_jvp.cuh) over the same tables
+TileEmit emit_tile_unit(const Mechanism& m, bool deriv = false);
 
 struct TransportTile {
   std::string source;      // empty: no transport section, or its fits do not suit the tables
@@ -36,5 +37,6 @@ TransportTile emit_transport_tile(const Mechanism& m);
 extern const char* kFixedMathSource;
 extern const char* kTileSource;
 extern const char* kTransportSource;
+extern const char* kTileJvpSource;
 
 }  // namespace pyro

@@ -116,9 +116,11 @@ const char* kArch = "sm_103a";
 // Compile CUDA C to a cubin for sm_103a with NVRTC.
 bool nvrtc_compile(const std::string& src, std::vector<char>& cubin, std::string& log) {
   nvrtcProgram prog;
-  const char* hdrs[] = {kDeviceMathSource, kFixedMathSource, kTileSource, kTransportSource};
-  const char* names[] = {"pyro_device_math.cuh", "pyro_fixed_math.cuh", "pyro_tile.cuh", "pyro_transport.cuh"};
-  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 4, hdrs, names) != NVRTC_SUCCESS) {
+  const char* hdrs[] = {kDeviceMathSource, kFixedMathSource, kTileSource, kTransportSource,
+                        kTileJvpSource};
+  const char* names[] = {"pyro_device_math.cuh", "pyro_fixed_math.cuh", "pyro_tile.cuh", "pyro_transport.cuh",
+                         "pyro_tile_jvp.cuh"};
+  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 5, hdrs, names) != NVRTC_SUCCESS) {
     log = "nvrtcCreateProgram failed";
     return false;
   }
@@ -157,6 +159,7 @@ int compile_cached(const std::string& src, bool use_cache, std::vector<char>& cu
                         std::to_string(nv_minor);
   if (src.find("pyro_fixed_math.cuh") != std::string::npos) key_src += kFixedMathSource;
   if (src.find("\"pyro_tile.cuh\"") != std::string::npos) key_src += kTileSource;
+  if (src.find("\"pyro_tile_jvp.cuh\"") != std::string::npos) key_src += std::string(kTileSource) + kTileJvpSource;
   if (src.find("\"pyro_transport.cuh\"") != std::string::npos) key_src += kTransportSource;
   char hex[32];
   std::snprintf(hex, sizeof hex, "%016llx", (unsigned long long)fnv1a(key_src));
@@ -528,7 +531,8 @@ const char* group_kernel(const std::string& g) {
   return g == "jvp" ? "pyro_jvp" : g == "vjp" ? "pyro_vjp" : g == "jad" ? "pyro_jacobian_adiabatic"
        : g == "cn" ? "pyro_cn_assemble" : g == "tr" ? "pyro_transport" : g == "wfwd" ? "pyro_omega_warp"
        : g == "wjvp" ? "pyro_jvp_warp" : g == "wvjp" ? "pyro_vjp_warp" : g == "wjac" ? "pyro_jacobian_cta"
-       : g == "wjad" ? "pyro_jacobian_adiabatic_cta" : g == "tile" ? "pyro_omega_tile" : g == "ttr" ? "pyro_transport_tile" : "pyro_jacobian";
+       : g == "wjad" ? "pyro_jacobian_adiabatic_cta" : g == "tile" ? "pyro_omega_tile" : g == "ttr" ? "pyro_transport_tile"
+       : g == "tjvp" ? "pyro_jvp_tile" : "pyro_jacobian";
 }
 
 // Compile (in parallel threads, cached on disk) and load the named derivative
@@ -575,6 +579,10 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
       G.block = 32 * h->emitted.warp_wpb.at(todo[i]);
       G.smem = h->emitted.smem_dyn_bytes_warp.at(todo[i]);
     }
+    if (todo[i] == "tjvp") {
+      G.block = 32 * h->emitted.jvp_tile_warps;
+      G.smem = h->emitted.smem_dyn_bytes_jvp_tile;
+    }
     if (todo[i] == "ttr") {
       G.block = 32 * h->emitted.transport_warps;
       G.smem = h->emitted.smem_dyn_bytes_transport_tile;
@@ -617,7 +625,7 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
       h->emitted.stats[todo[i] + "_active_clusters"] = ncl;
     }
     if (h->emitted.stats["deriv_store_global"] > 0 && todo[i] != "jac" && todo[i] != "jad" && todo[i] != "cn" &&
-        todo[i] != "tile" && todo[i] != "ttr" && todo[i][0] != 'w') {
+        todo[i] != "tile" && todo[i] != "ttr" && todo[i] != "tjvp" && todo[i][0] != 'w') {
       size_t bytes = (size_t)h->num_sms * nb * 4 * h->m.n_species() * h->opt.deriv_block * sizeof(double);
       cudaError_t e = cudaMalloc(&G.store, bytes);
       if (e != cudaSuccess) return fail(PYRO_ECUDA, std::string("species-array store allocation: ") + cudaGetErrorString(e));
@@ -694,6 +702,15 @@ int launch_cta(const pyro_mech* h, const pyro_mech::Group& G, int64_t n, void* s
   CUresult r = driver().LaunchKernel(G.f, grid, 1, 1, G.block, 1, 1, G.smem, as_stream(stream), params, nullptr);
   if (r != CUDA_SUCCESS) return fail(PYRO_ECUDA, "kernel launch: " + cu_err(r));
   return PYRO_OK;
+}
+
+// the kernels of a handle's JVP: the tile kernel with the per-thread kernel for the states
+// it leaves open, or (variant=warp, or a mechanism beyond the tables) one FP64 kernel
+std::vector<std::string> jvp_groups(const pyro_mech* h) {
+  if (h->opt.warp) return {"wjvp"};
+  auto it = h->emitted.stats.find("jvp_tile");
+  if (it == h->emitted.stats.end() || it->second <= 0) return {"jvp"};
+  return {"jvp", "tjvp"};
 }
 
 // the dense Jacobian groups of a handle: block per state (variant=warp, where
@@ -1040,13 +1057,15 @@ int pyro_mech_prepare(const pyro_mech* hc, const char* kernels) {
   std::string k = kernels ? kernels : "all";
   std::vector<std::string> names;
   if (k == "all") {
-    names = {h->opt.warp ? "wjvp" : "jvp", h->opt.warp ? "wvjp" : "vjp", jac_group(h, false)};
+    names = {h->opt.warp ? "wvjp" : "vjp", jac_group(h, false)};
+    for (auto& g : jvp_groups(h)) names.push_back(g);
   }
   else {
     std::string item;
     std::stringstream ss(k);
     while (std::getline(ss, item, ',')) {
-      if (item == "jvp" || item == "vjp") names.push_back(h->opt.warp ? "w" + item : item);
+      if (item == "jvp") { for (auto& g : jvp_groups(h)) names.push_back(g); }
+      else if (item == "vjp") names.push_back(h->opt.warp ? "wvjp" : "vjp");
       else if (item == "jacobian" || item == "jac") names.push_back(jac_group(h, false));
       else if (item == "jacobian_adiabatic" || item == "jad") names.push_back(jac_group(h, true));
       else if (item == "cn" || item == "crank_nicolson") names.push_back("cn");
@@ -1069,15 +1088,23 @@ int pyro_jvp(const pyro_mech* hc, int64_t n, const double* rho, const double* T,
     return fail(PYRO_EINVAL, "pyro_jvp: bad arguments");
   if (n == 0) return PYRO_OK;
   if (int rc = check_device(h)) return rc;
-  const std::string g = h->opt.warp ? "wjvp" : "jvp";   // one warp or one thread per state
-  if (int rc = ensure_groups(h, {g})) return rc;
+  const std::vector<std::string> gs = jvp_groups(h);
+  const std::string g = gs[0];
+  if (int rc = ensure_groups(h, gs)) return rc;
   const int64_t NS = h->m.n_species();
   return with_args(h, n, {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false}, {d_rho, 1, 8, true, false},
                        {d_T, 1, 8, true, false}, {d_Y, NS, 8, true, false}, {d_omega, NS, 8, false, true}},
                    stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
                      long long nn = nc;
-                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &d[5], &d[6], &h->groups[g].store};
+                     int open_only = gs.size() > 1 ? 1 : 0;
+                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &d[5], &d[6], &h->groups[g].store, &open_only};
                      if (h->opt.warp) return launch_warp(h, h->groups[g], nc, st, params);
+                     if (open_only) {
+                       const pyro_mech::Group& t = h->groups["tjvp"];
+                       const unsigned grid = (unsigned)std::min((nc + 31) / 32, (int64_t)h->num_sms * t.blocks_per_sm);
+                       CUresult r = driver().LaunchKernel(t.f, grid, 1, 1, t.block, 1, 1, t.smem, as_stream(st), params, nullptr);
+                       if (r != CUDA_SUCCESS) return fail(PYRO_ECUDA, "kernel launch: " + cu_err(r));
+                     }
                      return launch_deriv(h, h->groups[g], nc, st, params);
                    }, h->opt.warp);
 }

@@ -33,6 +33,7 @@ using pfx::Pair;
 typedef pfx::i64 i64;
 typedef pfx::u64 u64;
 
+#ifndef TILE_DERIV
 struct TileScalars {
   double T[32], ysum[32];
   Pair u[32], v[32], t[32];      // log2(T)/16, T_V/T, T/T_T
@@ -46,7 +47,9 @@ struct TileScalars {
 // e = r & 4095.  The exponent's bits are the last bits of the integer: they lie below
 // its resolution and, near RATE_E/4096 of one unit, are on average what truncation
 // took away.
+#ifndef RATE_E
 #define RATE_E 2048
+#endif
 struct TileSmem {
   u64* exp2;
   i64 *lam, *alp;   // [NSP + 1][32]: the species and a unit factor; alp first holds Y
@@ -58,6 +61,8 @@ struct TileSmem {
   TileScalars* sc;
 };
 
+#endif  // TILE_DERIV
+
 __device__ __forceinline__ Pair as_pair(i64 v) {
   Pair p;
   p.lo = (int)v;
@@ -65,6 +70,7 @@ __device__ __forceinline__ Pair as_pair(i64 v) {
   return p;
 }
 
+#ifndef TILE_DERIV
 __device__ __forceinline__ TileSmem tile_smem(char* base) {
   TileSmem s;
   s.exp2 = (u64*)base;                     base += pfx::EXP2_TAB * 8;
@@ -79,6 +85,8 @@ __device__ __forceinline__ TileSmem tile_smem(char* base) {
   s.sc = (TileScalars*)base;
   return s;
 }
+
+#endif  // TILE_DERIV
 
 // sums of products of fixed-point values c (two signed halves) and Y (f = 61): h 2^64 + l 2^32
 struct TileDot {
@@ -151,6 +159,7 @@ __device__ __forceinline__ i64 tile_K(i64 c, i64 beta, i64 tau, Pair u, Pair v) 
   return pfx::mul_add(as_pair(tau), v, pfx::mul_add(as_pair(beta), u, c)) & ~1ll;
 }
 
+#ifndef TILE_DERIV
 // ---------------------------------------------------------------------------
 // temperature (Sec. A.3.1): FP32 Newton on the collapsed polynomials of both
 // ranges, then FP64 Newton on the range found, as in the per-thread solve
@@ -275,9 +284,12 @@ __device__ __forceinline__ void tile_energy(const TileSmem& s, const double* __r
   }
 }
 
+#endif  // TILE_DERIV
+
 // ---------------------------------------------------------------------------
 // reactions
 // ---------------------------------------------------------------------------
+#ifndef TILE_DERIV
 // plain reactions with up to NF factors a side (missing ones: the unit factor);
 // REV: reversible.  A flag marks a duplicate of a reaction before it in this warp,
 // whose rate is added to the same row.
@@ -317,6 +329,8 @@ __device__ __forceinline__ void tile_plain(const TileSmem& s, int i0, int i1, Pa
   }
 }
 
+#endif  // TILE_DERIV
+
 __device__ __forceinline__ double ax_d(i64 v) { return __longlong_as_double(v); }
 
 // sum_k eps_k Y_k/W_k of a reaction from its efficiency list.  In FP64: the integer form
@@ -346,6 +360,7 @@ __device__ __forceinline__ i64 tile_part(double f, i64 l) {
   return near_one ? l - p : p;
 }
 
+#ifndef TILE_DERIV
 // reactions of the other classes: auxiliary data ax (see the emitter for the layout)
 __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, int lane, double rho,
                                            const double* __restrict__ Yp, i64 n) {
@@ -436,9 +451,57 @@ __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, in
   }
 }
 
+#endif  // TILE_DERIV
+
+// species sums of a chunk: per owned species the rows with nu = +1, with -1 (both padded to
+// multiples of 4 with the zero row) and with other nu; sink(species, sum)
 struct TilePlus { static constexpr bool minus = false; };
 struct TileMinus { static constexpr bool minus = true; };
+template <class F>
+__device__ __forceinline__ void tile_sums(const i64* rows, int ch, int w, F sink) {
+  const char* R = (const char*)rows;
+  // a warp's lists follow one another in the entry table: the next four entries and the
+  // next species' header are loaded while the last ones are summed (both tables end
+  // with a spare element)
+  int4 qn = __ldg((const int4*)t_wl + (ch * NW + w) * KPO);              // first entry, ends of the three lists
+  int2 on = __ldg((const int2*)t_wo + (ch * NW + w) * KPO);              // species, head-room bits + 256 others
+  int4 rn = __ldg((const int4*)(t_we + qn.x));
+#pragma unroll 1
+  for (int i = 0; i < KPO; ++i) {
+    const int4 q = qn;
+    const int2 o = on;
+    if (o.x < 0) break;
+    qn = __ldg((const int4*)t_wl + (ch * NW + w) * KPO + i + 1);
+    on = __ldg((const int2*)t_wo + (ch * NW + w) * KPO + i + 1);
+    const int hb = o.y & 0xff;
+    i64 a = 0;
+    int e = 0;
+    auto quad = [&](int j, auto sign) {
+      const int4 r = rn;
+      rn = __ldg((const int4*)(t_we + j + 4));
+      const i64 v0 = *(const i64*)(R + r.x), v1 = *(const i64*)(R + r.y), v2 = *(const i64*)(R + r.z),
+                v3 = *(const i64*)(R + r.w);
+      const int e0 = (int)v0 & 4095, e1 = (int)v1 & 4095, e2 = (int)v2 & 4095, e3 = (int)v3 & 4095;
+      const int en = max(max(e, max(e0, e1)), max(e2, e3)), t = en + hb;
+      a = tile_sar(a, en - e);
+      e = en;
+      const i64 b = (tile_sar(v0, t - e0) + tile_sar(v1, t - e1)) + (tile_sar(v2, t - e2) + tile_sar(v3, t - e3));
+      if (decltype(sign)::minus) a -= b; else a += b;
+    };
+    _Pragma("unroll 2") for (int j = q.x; j < q.y; j += 4) quad(j, TilePlus());
+    _Pragma("unroll 2") for (int j = q.y; j < q.z; j += 4) quad(j, TileMinus());
+    for (int j = q.z; j < q.z + (o.y >> 8); ++j) {
+      const i64 x = *(const i64*)(R + __ldg(t_we + j));
+      const int e0 = (int)x & 4095, en = max(e, e0);
+      a = tile_sar(a, en - e) + (i64)__ldg(t_wc + j) * tile_sar(x, en + hb - e0);
+      e = en;
+    }
+    if (q.w > q.z) rn = __ldg((const int4*)(t_we + q.w));
+    sink(o.x, tile_to_double(a, e + hb - RATE_E, 61));
+  }
+}
 
+#ifndef TILE_DERIV
 extern "C" __global__ void __launch_bounds__(32 * NW, TILE_MINB)
 pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict__ g_Tin, int energy_mode,
                 const double* __restrict__ g_Y, double* __restrict__ g_Tout, double* __restrict__ g_omega,
@@ -567,56 +630,16 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         }
       }
       __syncthreads();
-      // species sums: per owned species the rows with nu = +1, with -1 (both padded to
-      // multiples of 4 with the zero row) and with other nu
-      const char* R = (const char*)(s.R + lane);
-      // a warp's lists follow one another in the entry table: the next four entries and the
-      // next species' header are loaded while the last ones are summed (both tables end
-      // with a spare element)
-      int4 qn = __ldg((const int4*)t_wl + (ch * NW + w) * KPO);              // first entry, ends of the three lists
-      int2 on = __ldg((const int2*)t_wo + (ch * NW + w) * KPO);              // species, head-room bits + 256 others
-      int4 rn = __ldg((const int4*)(t_we + qn.x));
-#pragma unroll 1
-      for (int i = 0; i < KPO; ++i) {
-        const int4 q = qn;
-        const int2 o = on;
-        if (o.x < 0) break;
-        qn = __ldg((const int4*)t_wl + (ch * NW + w) * KPO + i + 1);
-        on = __ldg((const int2*)t_wo + (ch * NW + w) * KPO + i + 1);
-        const int hb = o.y & 0xff;
-        i64 a = 0;
-        int e = 0;
-        auto quad = [&](int j, auto sign) {
-          const int4 r = rn;
-          rn = __ldg((const int4*)(t_we + j + 4));
-          const i64 v0 = *(const i64*)(R + r.x), v1 = *(const i64*)(R + r.y), v2 = *(const i64*)(R + r.z),
-                    v3 = *(const i64*)(R + r.w);
-          const int e0 = (int)v0 & 4095, e1 = (int)v1 & 4095, e2 = (int)v2 & 4095, e3 = (int)v3 & 4095;
-          const int en = max(max(e, max(e0, e1)), max(e2, e3)), t = en + hb;
-          a = tile_sar(a, en - e);
-          e = en;
-          const i64 b = (tile_sar(v0, t - e0) + tile_sar(v1, t - e1)) + (tile_sar(v2, t - e2) + tile_sar(v3, t - e3));
-          if (decltype(sign)::minus) a -= b; else a += b;
-        };
-        _Pragma("unroll 2") for (int j = q.x; j < q.y; j += 4) quad(j, TilePlus());
-        _Pragma("unroll 2") for (int j = q.y; j < q.z; j += 4) quad(j, TileMinus());
-        for (int j = q.z; j < q.z + (o.y >> 8); ++j) {
-          const i64 x = *(const i64*)(R + __ldg(t_we + j));
-          const int e0 = (int)x & 4095, en = max(e, e0);
-          a = tile_sar(a, en - e) + (i64)__ldg(t_wc + j) * tile_sar(x, en + hb - e0);
-          e = en;
-        }
-        if (q.w > q.z) rn = __ldg((const int4*)(t_we + q.w));
-        double v = tile_to_double(a, e + hb - RATE_E, 61);
+      tile_sums(s.R + lane, ch, w, [&](int k, double v) {
         if (split) {
-          ((double*)s.lam)[o.x * 32 + lane] = v;     // the species arrays are free after the only chunk
+          ((double*)s.lam)[k * 32 + lane] = v;       // the species arrays are free after the only chunk
         } else if (p < n) {
-          double* out = g_omega + o.x * n + p;
+          double* out = g_omega + k * n + p;
           if (ch > 0) v += *out;
-          if (open && o.x == 0) v = __longlong_as_double(TILE_OPEN);
+          if (open && k == 0) v = __longlong_as_double(TILE_OPEN);
           *out = v;
         }
-      }
+      });
       __syncthreads();
     }
 #if NCH > 1
@@ -651,3 +674,4 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
 #endif
   }
 }
+#endif  // TILE_DERIV

@@ -1,0 +1,84 @@
+"""The JVP's tile kernel against the oracle where its dispatch or its number formats can go
+wrong: ragged tiles, states outside its tables beside ordinary ones, absent, negative and tiny
+mass fractions, zero and huge tangents, and every reaction class.  Tolerance: 1e-11 of each
+entry's gross scale (as in test_gpu_derivatives), with that suite's absolute floor of 1e-250."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2503_24286_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mechs(mech_files, mixed_reversibility_mech):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2503_24286_gb300 import binding as B
+    from paper_2503_24286_gb300 import build as BLD
+    BLD.build()
+    out = {}
+    for name, p in (("h2", mech_files[0][0]), ("gri", mech_files[0][1]), ("pdep", mixed_reversibility_mech)):
+        out[name] = (B.Mechanism(p), O.Oracle(p))
+        assert out[name][0].stat("jvp_tile") == 1
+    return out
+
+
+def _t(a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda:0")
+
+
+def _inputs(orc, idx, n, seed):
+    st = synth.config_states(idx, n=n, offset_seed=seed)
+    rng = np.random.default_rng(seed)
+    rho = orc.density(st.p, st.T, st.Y)
+    return [rho, st.T.copy(), st.Y.copy(), rng.standard_normal(n) * rho * 0.1, rng.standard_normal(n) * 10.0,
+            rng.standard_normal((orc.N, n)) * 1e-3]
+
+
+def _check(m, orc, a, skip=()):
+    g = m.jvp(*[_t(x) for x in a]).cpu().numpy()
+    o, sc = orc.jvp(*a), orc.jvp_scale(*a)
+    # states where the oracle's own numbers leave the double range ([M] = 0, 190 K) say nothing
+    fine = np.isfinite(o).all(axis=0) & np.isfinite(sc).all(axis=0)
+    keep = np.setdiff1d(np.arange(a[0].size)[fine], skip)
+    assert keep.size >= 0.9 * a[0].size
+    assert np.all(np.isfinite(g[:, keep]))
+    assert np.all(np.abs(g - o)[:, keep] <= 1e-11 * sc[:, keep] + 1e-250)
+    return g
+
+
+@pytest.mark.parametrize("name,idx", [("h2", 0), ("gri", 1), ("pdep", 7)])
+@pytest.mark.parametrize("n", [1, 31, 33, 70])
+def test_ragged_tiles(mechs, name, idx, n):
+    m, orc = mechs[name]
+    _check(m, orc, _inputs(orc, idx, n, 61 + n))
+
+
+@pytest.mark.parametrize("name,idx", [("h2", 0), ("gri", 1), ("pdep", 7)])
+def test_open_states_and_compositions(mechs, name, idx):
+    m, orc = mechs[name]
+    a = _inputs(orc, idx, 128, 62)
+    rho, T, Y, dr, dT, dY = a
+    rng = np.random.default_rng(63)
+    N = orc.N
+    T[[3, 40, 41]] = [190.0, 5000.0, 5400.0]
+    rho[5] = 1e-22
+    Y[:, 32:64] = np.where(rng.random((N, 32)) < 0.6, 0.0, Y[:, 32:64])
+    Y[:, 64:96] *= np.where(rng.random((N, 32)) < 0.3, -1e-6, 1.0)
+    Y[:, 96:112] = 10.0 ** rng.uniform(-60, -1, (N, 16))
+    dT[50], dr[51], dY[:, 52] = 0.0, 0.0, 0.0
+    dY[:, 53] *= 1e30
+    _check(m, orc, a)
+
+
+def test_nan_stays_in_its_state(mechs):
+    m, orc = mechs["gri"]
+    a = _inputs(orc, 1, 64, 64)
+    a[2][4, 10] = np.nan
+    a[5][4, 11] = np.nan
+    a[4][12] = np.inf
+    g = _check(m, orc, a, skip=(10, 11, 12))
+    assert np.isnan(g[4, 10]) and np.isnan(g[4, 11]) and not np.isfinite(g[:, 12]).all()
