@@ -834,12 +834,19 @@ void emit_vjp_kernel(Src& s, const Mechanism& m, const std::vector<SpeciesCoef>&
   s << "extern \"C\" __global__ void __launch_bounds__(" << blk << ") pyro_vjp(i64 n, const double* __restrict__ g_rho,\n"
        "    const double* __restrict__ g_T, const double* __restrict__ g_Y, const double* __restrict__ g_wb,\n"
        "    double* __restrict__ g_rhob, double* __restrict__ g_Tb, double* __restrict__ g_Yb,\n"
-       "    double* __restrict__ g_store) {\n"
+       "    double* __restrict__ g_store, int open_only) {\n"
+       "  // open_only: only the states that the tile kernel left open (pyro_tile_vjp.cuh)\n"
+       "  if (open_only) {\n    bool any = false;\n"
+       "    #pragma unroll 8\n"
+       "    for (i64 p = (i64)blockIdx.x * BLKD + threadIdx.x; p < n; p += (i64)gridDim.x * BLKD)\n"
+       "      any |= __double_as_longlong(g_rhob[p]) == " << kTileOpen << ";\n"
+       "    if (!__syncthreads_or(any)) return;\n  }\n"
        "  __shared__ double s_exp[512];\n  __shared__ double s_log[256];\n  extern __shared__ double s_dyn[];\n"
        "  double* sL = " << (opt.dgstore ? "g_store + (i64)blockIdx.x * 4 * NSP * BLKD" : "s_dyn") << ";\n"
        "  double* sA = sL + NSP * BLKD; double* sLp = sA + NSP * BLKD; double* sC = sLp + NSP * BLKD;\n"
        "  pyro_load_tables(s_exp, s_log);\n  __syncthreads();\n  const int t = threadIdx.x;\n"
        "  for (i64 p = (i64)blockIdx.x * BLKD + t; p < n; p += (i64)gridDim.x * BLKD) {\n"
+       "    if (open_only && __double_as_longlong(g_rhob[p]) != " << kTileOpen << ") continue;\n"
        "    const double* Yp = g_Y + p; const double* Wb = g_wb + p;\n"
        "    const double rho = g_rho[p], T = g_T[p];\n"
        "    const double lnT = pdm::log(T, s_log), invT = pdm::rcp(T), invT2 = invT * invT;\n"
@@ -2429,12 +2436,19 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
       out.stats["tile_warps"] = t.warps;
       out.stats["tile_chunks"] = t.chunks;
     }
-    const TileEmit j = emit_tile_unit(m, true);
+    const TileEmit j = emit_tile_unit(m, TileKind::Jvp);
     out.stats["jvp_tile"] = j.source.empty() ? 0 : 1;
     if (!j.source.empty()) {
       out.group_sources["tjvp"] = j.source;
       out.jvp_tile_warps = j.warps;
       out.smem_dyn_bytes_jvp_tile = j.smem_bytes;
+    }
+    const TileEmit v = emit_tile_unit(m, TileKind::Vjp);
+    out.stats["vjp_tile"] = v.source.empty() ? 0 : 1;
+    if (!v.source.empty()) {
+      out.group_sources["tvjp"] = v.source;
+      out.vjp_tile_warps = v.warps;
+      out.smem_dyn_bytes_vjp_tile = v.smem_bytes;
     }
   }
   out.stats["deriv_block"] = opt.deriv_block;

@@ -43,6 +43,7 @@ struct EmitResult {
   int smem_dyn_bytes_jac = 0;             // dynamic shared memory of the Jacobian-type kernels
   int transport_warps = 0;                // warps per block of the transport tile kernel
   int smem_dyn_bytes_transport_tile = 0;  // its dynamic shared memory
+  int vjp_tile_warps = 0, smem_dyn_bytes_vjp_tile = 0;   // the same of the VJP's
   int jvp_tile_warps = 0;                 // warps per block of the JVP's tile kernel
   int smem_dyn_bytes_jvp_tile = 0;        // its dynamic shared memory
   int tile_warps = 0;                     // warps per block of the tile kernel

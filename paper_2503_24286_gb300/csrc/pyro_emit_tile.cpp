@@ -93,13 +93,14 @@ std::vector<std::string> as_d(const std::vector<double>& v) {
 
 }  // namespace
 
-TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
+TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
+  const bool deriv = what != TileKind::Rates, vjp = what == TileKind::Vjp;
   TileEmit out;
   const int N = m.n_species(), NR = m.n_reactions();
   if (N < 1 || N > 1022 || NR < 1) { out.why = "no reactions, or more than 1022 species"; return out; }
   for (auto& r : m.reactions)
     if (side_factors(r.reactants).size() > 3 || side_factors(r.products).size() > 3 ||
-        side_factors(r.reactants).empty() || (r.reversible && side_factors(r.products).empty())) {
+        side_factors(r.reactants).empty() || (vjp && side_factors(r.products).empty()) || (r.reversible && side_factors(r.products).empty())) {
       out.why = "a reaction has more than three factors on a side";
       return out;
     }
@@ -234,7 +235,10 @@ TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
   // the rows in more than one chunk two blocks lose (8.3 ms and more).  10 species / 21
   // reactions: eight blocks of 4 warps 0.81 ms, four of 8 warps 0.96 ms; 160 / 1100
   // (2^18 states): one block of 24 warps 5.6 ms, of 16 warps 6.4 ms.
-  const int fixed_bytes = deriv ? 8192 + 1024 * (N + 1) + 32 * (8 * 8 + 3 * 8 + 8 + 4) + 256 : 8192 + 512 * (N + 1) + 2064 + 256;
+  int mrows = 0;                                 // reactions with an [M] adjoint
+  for (int j = 0; j < NR; ++j) if (classes(m.reactions[j])) ++mrows;
+  const int fixed_bytes = vjp ? 8192 + 1024 * (N + 1) + 256 * (mrows + 2) + 3 * 24 * 256 + 32 * (5 * 8 + 3 * 8 + 8 + 4) + 256
+                        : deriv ? 8192 + 1024 * (N + 1) + 32 * (8 * 8 + 3 * 8 + 8 + 4) + 256 : 8192 + 512 * (N + 1) + 2064 + 256;
   int warps = rows_all < 48 ? 4 : rows_all < 120 ? 8 : 12;
   int minb = 24 / warps + (warps == 4 ? 2 : 0);
   auto red = [](int w) { return w * 256 + 6 * 256 + 14 * 128 + w * 13 * 128; };   // scratch of the temperature solve, in the rows
@@ -244,6 +248,7 @@ TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
   const int max_rows = lim / 256;
   if (lim < red(warps) || max_rows < 8) { out.why = "species arrays do not fit in shared memory"; return out; }
   const int chunks = (rows_all + max_rows - 1) / max_rows;
+  if (vjp && chunks > 1) { out.why = "the reactions do not fit in shared memory at once"; return out; }
   const int rows = (rows_all + chunks - 1) / chunks;
   const int tile_rows = std::max(rows, (red(warps) + 255) / 256);
 
@@ -267,7 +272,7 @@ TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
   std::map<int, int> class_id;
   auto key_of = [&](int j) {
     if (classes(m.reactions[j])) return 8;
-    return (std::max(nfac(j, false), n_prod(j)) > 2 ? 2 : 0) + (n_prod(j) > 0 ? 1 : 0);
+    return (std::max(nfac(j, false), vjp ? nfac(j, true) : n_prod(j)) > 2 ? 2 : 0) + (n_prod(j) > 0 ? 1 : 0);
   };
   for (int j = 0; j < NR; ++j) class_id[key_of(j)] = 0;
   class_id[8] = 0;
@@ -277,7 +282,8 @@ TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
   std::vector<i64> rx, ax;
   std::vector<double> rd, fxa;                   // b, theta of a record; FP64 companions of ax
   std::vector<int> seg;
-  std::vector<int> row_of(groups.size());
+  std::vector<int> row_of(groups.size()), mrow_of(NR, -1);
+  int mrow = 0;
   for (int ch = 0; ch < chunks; ++ch) {
     std::vector<std::vector<int>> mine(warps);
     std::vector<double> load(warps, 0.0);
@@ -304,7 +310,9 @@ TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
               rec[1] = fx.coef(16 * a.b);
               rec[2] = fx.coef(-a.theta * LOG2E / T_V);
             }
-            const std::vector<int> fr = side_factors(r.reactants), fp = r.reversible ? side_factors(r.products) : std::vector<int>();
+            // the adjoint needs the products of an irreversible reaction too
+            const std::vector<int> fr = side_factors(r.reactants),
+                                   fp = r.reversible || vjp ? side_factors(r.products) : std::vector<int>();
             auto at = [](const std::vector<int>& f, size_t i) { return (u64)(i < f.size() ? f[i] : 0); };
             rd.push_back(r.b);
             rd.push_back(r.theta);
@@ -318,7 +326,10 @@ TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
               continue;
             }
             rec[3] = (i64)(at(fr, 0) | at(fr, 1) << 16 | at(fr, 2) << 32 | at(fp, 0) << 48);
-            rec[4] = (i64)(at(fp, 1) | at(fp, 2) << 16 | (u64)row_of[g] << 32 | (u64)fr.size() << 48 | (u64)fp.size() << 52 | (u64)cls << 56);
+            rec[4] = (i64)(at(fp, 1) | at(fp, 2) << 16 | (u64)row_of[g] << 32 | (u64)fr.size() << 48 | (u64)fp.size() << 52 | (u64)cls << 56 |
+                           (u64)(r.reversible ? 1 : 0) << 60);
+            rec[6] = (i64)mrow;
+            mrow_of[j] = mrow++;
             rec[5] = (i64)ax.size();
             if (cls) {
               std::vector<i64> x(16, 0);
@@ -442,6 +453,44 @@ TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
   for (int q = 0; q < 2; ++q) wo.push_back(-1);
   for (int q = 0; q < 64; ++q) ax.push_back(0);  // and the prefetches touch up to 512 bytes
 
+  // adjoint lists: per owned species its factor occurrences (row of Db, the other factors'
+  // offsets) and its efficiency terms (row of the [M] adjoint, coefficient)
+  std::vector<int> vl, v1, v2, v3;
+  if (vjp) {
+    for (int w = 0; w < warps; ++w)
+      for (int i = 0; i < kpo; ++i) {
+        if (i >= (int)owned[w].size()) { for (int q = 0; q < 8; ++q) vl.push_back(q ? 0 : -1); continue; }
+        const int k = owned[w][i];
+        int h[8] = {k, (int)v1.size() / 2, 0, 0, (int)v2.size() / 4, 0, (int)v3.size() / 4, 0};
+        for (int side = 0; side < 2; ++side) {
+          for (size_t g = 0; g < groups.size(); ++g) {
+            const Reaction& r = m.reactions[groups[g][0]];
+            if (side && !r.reversible) continue;
+            const std::vector<int> f = side_factors(side ? r.products : r.reactants);
+            for (size_t q = 0; q < f.size(); ++q) {
+              if (f[q] != k) continue;
+              std::vector<int> o;
+              for (size_t z = 0; z < f.size(); ++z) if (z != q) o.push_back(f[z] * 256);
+              if (o.empty()) o.push_back(N * 256);
+              if (o.size() == 1) { v1.push_back(row_of[g] * 256); v1.push_back(o[0]); }
+              else for (int x : {row_of[g] * 256, o[0], o[1], side}) v2.push_back(x);
+            }
+          }
+          h[2 + side] = (int)v1.size() / 2;
+        }
+        for (int j = 0; j < NR; ++j)
+          for (auto& e : m.reactions[j].efficiencies) {
+            const double c = (e.second - 1.0) / m.species[e.first].W;
+            if (e.first != k || c == 0.0 || mrow_of[j] < 0) continue;
+            const u64 b = (u64)dbits(c);
+            for (int x : {mrow_of[j] * 256, 0, (int)(unsigned)b, (int)(unsigned)(b >> 32)}) v3.push_back(x);
+          }
+        h[5] = (int)v2.size() / 4;
+        h[7] = (int)v3.size() / 4;
+        vl.insert(vl.end(), h, h + 8);
+      }
+  }
+
   // ---- the unit -------------------------------------------------------------------
   std::ostringstream o;
   o << "// Tile kernel of mechanism '" << m.name << "': " << N << " species, " << NR << " reactions.\n"
@@ -481,16 +530,23 @@ TileEmit emit_tile_unit(const Mechanism& m, bool deriv) {
     array(o, "__align__(16) double", "t_rd", as_d(rd));
     array(o, "double", "t_fx", as_d(fxa));
     array(o, "double", "t_h", as_d(hc));
+    if (vjp) {
+      o << "#define T_MROWS " << mrows << "\n";
+      array(o, "__align__(16) int", "t_vl", vl);
+      array(o, "__align__(8) int", "t_v1", v1);
+      array(o, "__align__(16) int", "t_v2", v2);
+      array(o, "__align__(16) int", "t_v3", v3);
+    }
   }
   o << (deriv ? "#define TILE_PLAIN" : "#define TILE_PLAIN(SGN)");
   for (auto& kv : class_id) {
     if (kv.first == 8) continue;
     const int c = kv.second;
     o << " \\\n  { const int a = __ldg(seg + " << c << "), b = __ldg(seg + " << c + 1 << "); if (a < b) "
-      << (deriv ? "jvp_plain<" : "tile_plain<") << (kv.first & 2 ? 3 : 2) << ", " << (kv.first & 1 ? "true" : "false")
-      << (deriv ? ">(s, a, b, u, v, u1, u2, lane); }" : ", SGN>(s, a, b, u, v, lane); }");
+      << (vjp ? "vjp_plain<" : deriv ? "jvp_plain<" : "tile_plain<") << (kv.first & 2 ? 3 : 2) << ", " << (kv.first & 1 ? "true" : "false")
+      << (vjp ? ">(s, a, b, u, v, invT, invT2, Tb, lane); }" : deriv ? ">(s, a, b, u, v, u1, u2, lane); }" : ", SGN>(s, a, b, u, v, lane); }");
   }
-  o << (deriv ? "\n#include \"pyro_tile_jvp.cuh\"\n" : "\n#include \"pyro_tile.cuh\"\n");
+  o << (vjp ? "\n#include \"pyro_tile_vjp.cuh\"\n" : deriv ? "\n#include \"pyro_tile_jvp.cuh\"\n" : "\n#include \"pyro_tile.cuh\"\n");
   out.source = o.str();
   out.warps = warps;
   out.smem_bytes = fixed_bytes + tile_rows * 256;

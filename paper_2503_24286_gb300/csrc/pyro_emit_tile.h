@@ -23,8 +23,10 @@ constexpr int kSmemPerSm = 228 * 1024;
 constexpr int kSmemPerBlock = 1024;
 constexpr int kSmemMaxBlock = 227 * 1024;
 
-// deriv: the unit of the Jacobian-vector product (pyro_tile_jvp.cuh) over the same tables
-TileEmit emit_tile_unit(const Mechanism& m, bool deriv = false);
+// Kernels over the tables: net production rates (pyro_tile.cuh), Jacobian-vector product
+// (pyro_tile_jvp.cuh), vector-Jacobian product (pyro_tile_vjp.cuh).
+enum class TileKind { Rates, Jvp, Vjp };
+TileEmit emit_tile_unit(const Mechanism& m, TileKind kind = TileKind::Rates);
 
 struct TransportTile {
   std::string source;      // empty: no transport section, or its fits do not suit the tables
@@ -38,5 +40,6 @@ extern const char* kFixedMathSource;
 extern const char* kTileSource;
 extern const char* kTransportSource;
 extern const char* kTileJvpSource;
+extern const char* kTileVjpSource;
 
 }  // namespace pyro

@@ -117,10 +117,10 @@ const char* kArch = "sm_103a";
 bool nvrtc_compile(const std::string& src, std::vector<char>& cubin, std::string& log) {
   nvrtcProgram prog;
   const char* hdrs[] = {kDeviceMathSource, kFixedMathSource, kTileSource, kTransportSource,
-                        kTileJvpSource};
+                        kTileJvpSource, kTileVjpSource};
   const char* names[] = {"pyro_device_math.cuh", "pyro_fixed_math.cuh", "pyro_tile.cuh", "pyro_transport.cuh",
-                         "pyro_tile_jvp.cuh"};
-  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 5, hdrs, names) != NVRTC_SUCCESS) {
+                         "pyro_tile_jvp.cuh", "pyro_tile_vjp.cuh"};
+  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 6, hdrs, names) != NVRTC_SUCCESS) {
     log = "nvrtcCreateProgram failed";
     return false;
   }
@@ -160,6 +160,7 @@ int compile_cached(const std::string& src, bool use_cache, std::vector<char>& cu
   if (src.find("pyro_fixed_math.cuh") != std::string::npos) key_src += kFixedMathSource;
   if (src.find("\"pyro_tile.cuh\"") != std::string::npos) key_src += kTileSource;
   if (src.find("\"pyro_tile_jvp.cuh\"") != std::string::npos) key_src += std::string(kTileSource) + kTileJvpSource;
+  if (src.find("\"pyro_tile_vjp.cuh\"") != std::string::npos) key_src += std::string(kTileSource) + kTileVjpSource;
   if (src.find("\"pyro_transport.cuh\"") != std::string::npos) key_src += kTransportSource;
   char hex[32];
   std::snprintf(hex, sizeof hex, "%016llx", (unsigned long long)fnv1a(key_src));
@@ -532,7 +533,7 @@ const char* group_kernel(const std::string& g) {
        : g == "cn" ? "pyro_cn_assemble" : g == "tr" ? "pyro_transport" : g == "wfwd" ? "pyro_omega_warp"
        : g == "wjvp" ? "pyro_jvp_warp" : g == "wvjp" ? "pyro_vjp_warp" : g == "wjac" ? "pyro_jacobian_cta"
        : g == "wjad" ? "pyro_jacobian_adiabatic_cta" : g == "tile" ? "pyro_omega_tile" : g == "ttr" ? "pyro_transport_tile"
-       : g == "tjvp" ? "pyro_jvp_tile" : "pyro_jacobian";
+       : g == "tjvp" ? "pyro_jvp_tile" : g == "tvjp" ? "pyro_vjp_tile" : "pyro_jacobian";
 }
 
 // Compile (in parallel threads, cached on disk) and load the named derivative
@@ -578,6 +579,10 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
     if (todo[i][0] == 'w') {
       G.block = 32 * h->emitted.warp_wpb.at(todo[i]);
       G.smem = h->emitted.smem_dyn_bytes_warp.at(todo[i]);
+    }
+    if (todo[i] == "tvjp") {
+      G.block = 32 * h->emitted.vjp_tile_warps;
+      G.smem = h->emitted.smem_dyn_bytes_vjp_tile;
     }
     if (todo[i] == "tjvp") {
       G.block = 32 * h->emitted.jvp_tile_warps;
@@ -625,7 +630,7 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
       h->emitted.stats[todo[i] + "_active_clusters"] = ncl;
     }
     if (h->emitted.stats["deriv_store_global"] > 0 && todo[i] != "jac" && todo[i] != "jad" && todo[i] != "cn" &&
-        todo[i] != "tile" && todo[i] != "ttr" && todo[i] != "tjvp" && todo[i][0] != 'w') {
+        todo[i] != "tile" && todo[i] != "ttr" && todo[i] != "tjvp" && todo[i] != "tvjp" && todo[i][0] != 'w') {
       size_t bytes = (size_t)h->num_sms * nb * 4 * h->m.n_species() * h->opt.deriv_block * sizeof(double);
       cudaError_t e = cudaMalloc(&G.store, bytes);
       if (e != cudaSuccess) return fail(PYRO_ECUDA, std::string("species-array store allocation: ") + cudaGetErrorString(e));
@@ -704,13 +709,29 @@ int launch_cta(const pyro_mech* h, const pyro_mech::Group& G, int64_t n, void* s
   return PYRO_OK;
 }
 
-// the kernels of a handle's JVP: the tile kernel with the per-thread kernel for the states
+// the kernels of a handle's "jvp" or "vjp": the tile kernel with the per-thread kernel for the states
 // it leaves open, or (variant=warp, or a mechanism beyond the tables) one FP64 kernel
-std::vector<std::string> jvp_groups(const pyro_mech* h) {
-  if (h->opt.warp) return {"wjvp"};
-  auto it = h->emitted.stats.find("jvp_tile");
-  if (it == h->emitted.stats.end() || it->second <= 0) return {"jvp"};
-  return {"jvp", "tjvp"};
+std::vector<std::string> product_groups(const pyro_mech* h, const std::string& which) {
+  if (h->opt.warp) return {"w" + which};
+  auto it = h->emitted.stats.find(which + "_tile");
+  if (it == h->emitted.stats.end() || it->second <= 0) return {which};
+  return {which, "t" + which};
+}
+
+int launch_deriv(const pyro_mech* h, const pyro_mech::Group& G, int64_t n, void* stream, void** params);
+
+// Launch a product on device pointers: params ends with the FP64 kernel's open_only flag
+int launch_product(pyro_mech* h, const std::vector<std::string>& gs, int64_t n, void* stream, void** params, int* open_only) {
+  const pyro_mech::Group& G = h->groups[gs[0]];
+  if (h->opt.warp) return launch_warp(h, G, n, stream, params);
+  *open_only = gs.size() > 1 ? 1 : 0;
+  if (*open_only) {
+    const pyro_mech::Group& t = h->groups[gs[1]];
+    const unsigned grid = (unsigned)std::min((n + 31) / 32, (int64_t)h->num_sms * t.blocks_per_sm);
+    CUresult r = driver().LaunchKernel(t.f, grid, 1, 1, t.block, 1, 1, t.smem, as_stream(stream), params, nullptr);
+    if (r != CUDA_SUCCESS) return fail(PYRO_ECUDA, "kernel launch: " + cu_err(r));
+  }
+  return launch_deriv(h, G, n, stream, params);
 }
 
 // the dense Jacobian groups of a handle: block per state (variant=warp, where
@@ -1057,15 +1078,14 @@ int pyro_mech_prepare(const pyro_mech* hc, const char* kernels) {
   std::string k = kernels ? kernels : "all";
   std::vector<std::string> names;
   if (k == "all") {
-    names = {h->opt.warp ? "wvjp" : "vjp", jac_group(h, false)};
-    for (auto& g : jvp_groups(h)) names.push_back(g);
+    names = {jac_group(h, false)};
+    for (const char* which : {"jvp", "vjp"}) for (auto& g : product_groups(h, which)) names.push_back(g);
   }
   else {
     std::string item;
     std::stringstream ss(k);
     while (std::getline(ss, item, ',')) {
-      if (item == "jvp") { for (auto& g : jvp_groups(h)) names.push_back(g); }
-      else if (item == "vjp") names.push_back(h->opt.warp ? "wvjp" : "vjp");
+      if (item == "jvp" || item == "vjp") { for (auto& g : product_groups(h, item)) names.push_back(g); }
       else if (item == "jacobian" || item == "jac") names.push_back(jac_group(h, false));
       else if (item == "jacobian_adiabatic" || item == "jad") names.push_back(jac_group(h, true));
       else if (item == "cn" || item == "crank_nicolson") names.push_back("cn");
@@ -1088,24 +1108,16 @@ int pyro_jvp(const pyro_mech* hc, int64_t n, const double* rho, const double* T,
     return fail(PYRO_EINVAL, "pyro_jvp: bad arguments");
   if (n == 0) return PYRO_OK;
   if (int rc = check_device(h)) return rc;
-  const std::vector<std::string> gs = jvp_groups(h);
-  const std::string g = gs[0];
+  const std::vector<std::string> gs = product_groups(h, "jvp");
   if (int rc = ensure_groups(h, gs)) return rc;
   const int64_t NS = h->m.n_species();
   return with_args(h, n, {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false}, {d_rho, 1, 8, true, false},
                        {d_T, 1, 8, true, false}, {d_Y, NS, 8, true, false}, {d_omega, NS, 8, false, true}},
                    stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
                      long long nn = nc;
-                     int open_only = gs.size() > 1 ? 1 : 0;
-                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &d[5], &d[6], &h->groups[g].store, &open_only};
-                     if (h->opt.warp) return launch_warp(h, h->groups[g], nc, st, params);
-                     if (open_only) {
-                       const pyro_mech::Group& t = h->groups["tjvp"];
-                       const unsigned grid = (unsigned)std::min((nc + 31) / 32, (int64_t)h->num_sms * t.blocks_per_sm);
-                       CUresult r = driver().LaunchKernel(t.f, grid, 1, 1, t.block, 1, 1, t.smem, as_stream(st), params, nullptr);
-                       if (r != CUDA_SUCCESS) return fail(PYRO_ECUDA, "kernel launch: " + cu_err(r));
-                     }
-                     return launch_deriv(h, h->groups[g], nc, st, params);
+                     int open_only = 0;
+                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &d[5], &d[6], &h->groups[gs[0]].store, &open_only};
+                     return launch_product(h, gs, nc, st, params, &open_only);
                    }, h->opt.warp);
 }
 
@@ -1116,16 +1128,16 @@ int pyro_vjp(const pyro_mech* hc, int64_t n, const double* rho, const double* T,
     return fail(PYRO_EINVAL, "pyro_vjp: bad arguments");
   if (n == 0) return PYRO_OK;
   if (int rc = check_device(h)) return rc;
-  const std::string g = h->opt.warp ? "wvjp" : "vjp";
-  if (int rc = ensure_groups(h, {g})) return rc;
+  const std::vector<std::string> gs = product_groups(h, "vjp");
+  if (int rc = ensure_groups(h, gs)) return rc;
   const int64_t NS = h->m.n_species();
   return with_args(h, n, {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false}, {omega_bar, NS, 8, true, false},
                        {rho_bar, 1, 8, false, true}, {T_bar, 1, 8, false, true}, {Y_bar, NS, 8, false, true}},
                    stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
                      long long nn = nc;
-                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &d[5], &d[6], &h->groups[g].store};
-                     if (h->opt.warp) return launch_warp(h, h->groups[g], nc, st, params);
-                     return launch_deriv(h, h->groups[g], nc, st, params);
+                     int open_only = 0;
+                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &d[5], &d[6], &h->groups[gs[0]].store, &open_only};
+                     return launch_product(h, gs, nc, st, params, &open_only);
                    }, h->opt.warp);
 }
 

@@ -1,4 +1,4 @@
-"""The JVP's tile kernel against the oracle where its dispatch or its number formats can go
+"""The JVP's and the VJP's tile kernels against the oracle where its dispatch or its number formats can go
 wrong: ragged tiles, states outside its tables beside ordinary ones, absent, negative and tiny
 mass fractions, zero and huge tangents, and every reaction class.  Tolerance: 1e-11 of each
 entry's gross scale (as in test_gpu_derivatives), with that suite's absolute floor of 1e-250."""
@@ -82,3 +82,52 @@ def test_nan_stays_in_its_state(mechs):
     a[4][12] = np.inf
     g = _check(m, orc, a, skip=(10, 11, 12))
     assert np.isnan(g[4, 10]) and np.isnan(g[4, 11]) and not np.isfinite(g[:, 12]).all()
+
+
+def _check_vjp(m, orc, rho, T, Y, wb, skip=()):
+    g = np.vstack([x.cpu().numpy().reshape(-1, T.size) for x in m.vjp(_t(rho), _t(T), _t(Y), _t(wb))])
+    o = np.vstack([np.asarray(x).reshape(-1, T.size) for x in orc.vjp(rho, T, Y, wb)])
+    sc = orc.vjp_scale(rho, T, Y, wb)
+    fine = np.isfinite(o).all(axis=0) & np.isfinite(sc).all(axis=0)
+    keep = np.setdiff1d(np.arange(T.size)[fine], skip)
+    assert keep.size >= 0.9 * T.size
+    assert np.all(np.isfinite(g[:, keep]))
+    assert np.all(np.abs(g - o)[:, keep] <= 1e-11 * sc[:, keep] + 1e-250)
+    return g
+
+
+@pytest.mark.parametrize("name,idx", [("h2", 0), ("gri", 1), ("pdep", 7)])
+@pytest.mark.parametrize("n", [1, 31, 33, 70])
+def test_vjp_ragged_tiles(mechs, name, idx, n):
+    m, orc = mechs[name]
+    assert m.stat("vjp_tile") == 1
+    rho, T, Y = _inputs(orc, idx, n, 71 + n)[:3]
+    _check_vjp(m, orc, rho, T, Y, np.random.default_rng(n).standard_normal((orc.N, n)))
+
+
+@pytest.mark.parametrize("name,idx", [("h2", 0), ("gri", 1), ("pdep", 7)])
+def test_vjp_open_states_and_compositions(mechs, name, idx):
+    m, orc = mechs[name]
+    rho, T, Y = _inputs(orc, idx, 128, 72)[:3]
+    rng = np.random.default_rng(73)
+    N = orc.N
+    wb = rng.standard_normal((N, 128))
+    T[[3, 40, 41]] = [190.0, 5000.0, 5400.0]
+    rho[5] = 1e-22
+    Y[:, 32:64] = np.where(rng.random((N, 32)) < 0.6, 0.0, Y[:, 32:64])
+    Y[:, 64:96] *= np.where(rng.random((N, 32)) < 0.3, -1e-6, 1.0)
+    Y[:, 96:112] = 10.0 ** rng.uniform(-60, -1, (N, 16))
+    wb[:, 50] = 0.0
+    wb[:, 51] *= 1e30
+    _check_vjp(m, orc, rho, T, Y, wb)
+
+
+def test_vjp_nan_stays_in_its_state(mechs):
+    m, orc = mechs["gri"]
+    rho, T, Y = _inputs(orc, 1, 64, 74)[:3]
+    wb = np.random.default_rng(75).standard_normal((orc.N, 64))
+    Y[4, 10] = np.nan
+    wb[4, 11] = np.nan
+    T[12] = np.nan
+    g = _check_vjp(m, orc, rho, T, Y, wb, skip=(10, 11, 12))
+    assert np.isnan(g[1, 10]) and np.isnan(g[1, 11]) and np.isnan(g[1, 12])
