@@ -24,7 +24,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # device sources compiled at run time (NVRTC), embedded as strings
 EMBED = {"pyro_device_math.cuh": "kDeviceMathSource", "pyro_fixed_math.cuh": "kFixedMathSource",
          "pyro_tile.cuh": "kTileSource", "pyro_transport.cuh": "kTransportSource",
-         "pyro_tile_jvp.cuh": "kTileJvpSource", "pyro_tile_vjp.cuh": "kTileVjpSource"}
+         "pyro_tile_jvp.cuh": "kTileJvpSource", "pyro_tile_vjp.cuh": "kTileVjpSource",
+         "pyro_tile_jac.cuh": "kTileJacSource"}
 
 
 def _embed_sources() -> str:

@@ -1134,9 +1134,16 @@ void emit_jacobian_kernel(Src& s, const Mechanism& m, const std::vector<SpeciesC
          "// per-reaction partials to the block's scratch, phase 2 assembles the rows.\n";
     s << "extern \"C\" __global__ void __launch_bounds__(" << blk << ") pyro_jacobian(i64 n, const double* __restrict__ g_rho,\n"
          "    const double* __restrict__ g_T, const double* __restrict__ g_Y, double* __restrict__ g_J,\n"
-         "    double* __restrict__ g_scratch) {\n" << prologue <<
+         "    double* __restrict__ g_scratch, int open_only) {\n"
+         "  // open_only: only the states that the tile kernel left open (pyro_tile_jac.cuh)\n"
+         "  if (open_only) {\n    bool any = false;\n"
+         "    #pragma unroll 8\n"
+         "    for (i64 p = (i64)blockIdx.x * BLKD + threadIdx.x; p < n; p += (i64)gridDim.x * BLKD)\n"
+         "      any |= __double_as_longlong(g_J[p]) == " << kTileOpen << ";\n"
+         "    if (!__syncthreads_or(any)) return;\n  }\n" << prologue <<
          "  double* W = g_scratch + (i64)blockIdx.x * " << stride << " * BLKD + t;\n"
          "  for (i64 p = (i64)blockIdx.x * BLKD + t; p < n; p += (i64)gridDim.x * BLKD) {\n"
+         "    if (open_only && __double_as_longlong(g_J[p]) != " << kTileOpen << ") continue;\n"
          "    const double* Yp = g_Y + p;\n    double* Jp = g_J + p;\n"
          "    const double rho = g_rho[p], T = g_T[p];\n";
   } else if (mode == JacMode::ADIA) {
@@ -2449,6 +2456,14 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
       out.group_sources["tvjp"] = v.source;
       out.vjp_tile_warps = v.warps;
       out.smem_dyn_bytes_vjp_tile = v.smem_bytes;
+    }
+    const TileEmit q = common_tmid(m) ? emit_tile_unit(m, TileKind::Jac) : TileEmit();
+    out.stats["jacobian_tile"] = q.source.empty() ? 0 : 1;
+    if (!q.source.empty()) {
+      out.group_sources["tjac"] = q.source;
+      out.jac_tile_warps = q.warps;
+      out.smem_dyn_bytes_jac_tile = q.smem_bytes;
+      out.jac_tile_scratch_bytes = q.scratch_bytes;
     }
   }
   out.stats["deriv_block"] = opt.deriv_block;

@@ -44,6 +44,8 @@ struct EmitResult {
   int transport_warps = 0;                // warps per block of the transport tile kernel
   int smem_dyn_bytes_transport_tile = 0;  // its dynamic shared memory
   int vjp_tile_warps = 0, smem_dyn_bytes_vjp_tile = 0;   // the same of the VJP's
+  int jac_tile_warps = 0, smem_dyn_bytes_jac_tile = 0;   // of the dense Jacobian's
+  int jac_tile_scratch_bytes = 0;         // its global scratch per block
   int jvp_tile_warps = 0;                 // warps per block of the JVP's tile kernel
   int smem_dyn_bytes_jvp_tile = 0;        // its dynamic shared memory
   int tile_warps = 0;                     // warps per block of the tile kernel

@@ -94,7 +94,8 @@ std::vector<std::string> as_d(const std::vector<double>& v) {
 }  // namespace
 
 TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
-  const bool deriv = what != TileKind::Rates, vjp = what == TileKind::Vjp;
+  const bool deriv = what != TileKind::Rates, jac = what == TileKind::Jac;
+  const bool vjp = what == TileKind::Vjp || jac;   // units that look at every reaction's products
   TileEmit out;
   const int N = m.n_species(), NR = m.n_reactions();
   if (N < 1 || N > 1022 || NR < 1) { out.why = "no reactions, or more than 1022 species"; return out; }
@@ -237,7 +238,8 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
   // (2^18 states): one block of 24 warps 5.6 ms, of 16 warps 6.4 ms.
   int mrows = 0;                                 // reactions with an [M] adjoint
   for (int j = 0; j < NR; ++j) if (classes(m.reactions[j])) ++mrows;
-  const int fixed_bytes = vjp ? 8192 + 1024 * (N + 1) + 256 * (mrows + 2) + 3 * 24 * 256 + 32 * (5 * 8 + 3 * 8 + 8 + 4) + 256
+  const int fixed_bytes = jac ? 8192 + 1280 * (N + 1) + 6 * 24 * 256 + 32 * (4 * 8 + 3 * 8 + 8 + 4) + 256
+                        : vjp ? 8192 + 1024 * (N + 1) + 256 * (mrows + 2) + 3 * 24 * 256 + 32 * (5 * 8 + 3 * 8 + 8 + 4) + 256
                         : deriv ? 8192 + 1024 * (N + 1) + 32 * (8 * 8 + 3 * 8 + 8 + 4) + 256 : 8192 + 512 * (N + 1) + 2064 + 256;
   int warps = rows_all < 48 ? 4 : rows_all < 120 ? 8 : 12;
   int minb = 24 / warps + (warps == 4 ? 2 : 0);
@@ -456,7 +458,63 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
   // adjoint lists: per owned species its factor occurrences (row of Db, the other factors'
   // offsets) and its efficiency terms (row of the [M] adjoint, coefficient)
   std::vector<int> vl, v1, v2, v3;
-  if (vjp) {
+  // dense Jacobian: per species row the terms of column T and of u_k, and the stream of terms
+  // per column (see pyro_tile_jac.cuh); the last row is the temperature's
+  std::vector<int> jk, jl, jt, je, jx;
+  std::vector<double> jc;
+  if (jac) {
+    for (int w = 0; w < warps; ++w) for (int i = 0; i < kpo; ++i) jk.push_back(i < (int)owned[w].size() ? owned[w][i] : -1);
+    auto terms_of = [&](int g, int times, std::vector<std::vector<int>>& col) {   // times: nu of the row
+      const Reaction& r = m.reactions[groups[g][0]];
+      for (int side = 0; side < (r.reversible ? 2 : 1); ++side) {
+        const std::vector<int> f = side_factors(side ? r.products : r.reactants);
+        for (size_t q = 0; q < f.size(); ++q) {
+          std::vector<int> o;
+          for (size_t z = 0; z < f.size(); ++z) if (z != q) o.push_back(f[z]);
+          if (o.empty()) o.push_back(N);
+          const int minus = (times < 0) != (side == 1) ? 1 : 0;
+          for (int t = 0; t < std::abs(times); ++t) {
+            col[f[q]].push_back(row_of[g] * 256 | minus | (o.size() > 1 ? 2 : 0));
+            col[f[q]].push_back(o[0] | (o.size() > 1 ? o[1] << 16 : 0));
+          }
+        }
+      }
+      const int j = groups[g][0];
+      if (mrow_of[j] >= 0)
+        for (auto& e : r.efficiencies) {
+          if (e.second == 1.0) continue;
+          col[e.first].push_back(mrow_of[j] * 256 | 4);
+          col[e.first].push_back((int)jc.size());
+          jc.push_back(times * (e.second - 1.0));
+        }
+    };
+    // a stream of two-term units: the columns first, first + step, ...
+    auto flush = [&](std::vector<std::vector<int>>& col, int first, int step) {
+      je.push_back((int)jx.size() / 4);
+      for (int c = first; c < N; c += step) {
+        if (col[c].empty()) { col[c].push_back(16); col[c].push_back(0); }
+        col[c][col[c].size() - 2] |= 8;
+        jx.insert(jx.end(), col[c].begin(), col[c].end());
+      }
+      while (jx.size() % 4) { jx.push_back(16); jx.push_back(0); }
+    };
+    for (int k = 0; k < N; ++k) {
+      std::vector<std::vector<int>> col(N);
+      jl.push_back((int)jt.size());
+      auto add = [&](int row, int nu) { for (int q = 0; q < std::abs(nu); ++q) jt.push_back(row * 256 | (nu < 0 ? 1 : 0)); };
+      for (auto& t : terms[k]) { add(row_of[t.first], t.second); terms_of(t.first, t.second, col); }
+      jl.push_back((int)jt.size());
+      jl.push_back((int)jt.size());
+      for (auto& t : terms[k]) if (mrow_of[groups[t.first][0]] >= 0) add(mrow_of[groups[t.first][0]], t.second);
+      jl.push_back((int)jt.size());
+      flush(col, 0, 1);
+    }
+    std::vector<std::vector<int>> col(N);
+    for (size_t g = 0; g < groups.size(); ++g) terms_of((int)g, 1, col);
+    for (int w = 0; w < warps; ++w) flush(col, w, warps);
+    for (int q = 0; q < 16; ++q) jx.push_back(16);   // the streams are read ahead
+  }
+  if (vjp && !jac) {
     for (int w = 0; w < warps; ++w)
       for (int i = 0; i < kpo; ++i) {
         if (i >= (int)owned[w].size()) { for (int q = 0; q < 8; ++q) vl.push_back(q ? 0 : -1); continue; }
@@ -513,12 +571,16 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
     array(o, "pfx::Log2Entry", "t_log2", l2);
   }
   array(o, "__align__(16) long long", "t_sp", as_ll(sp));
-  o << "__device__ const __align__(16) float t_ef[" << 12 * N << "] = {" << ef.str() << "};\n";
-  array(o, "__align__(16) double", "t_ed", as_d(ed));
+  if (!deriv) {
+    o << "__device__ const __align__(16) float t_ef[" << 12 * N << "] = {" << ef.str() << "};\n";
+    array(o, "__align__(16) double", "t_ed", as_d(ed));
+  }
   array(o, "double", "t_iw", as_d(iw));
-  array(o, "__align__(16) long long", "t_ex", as_ll(ex));
-  for (int& q : xs) q += 61;                     // f of the sums: the column's scale and Y's 61
-  array(o, "int", "t_exs", xs);
+  if (!deriv) {
+    array(o, "__align__(16) long long", "t_ex", as_ll(ex));
+    for (int& q : xs) q += 61;                   // f of the sums: the column's scale and Y's 61
+    array(o, "int", "t_exs", xs);
+  }
   array(o, "__align__(16) long long", "t_rx", as_ll(rx));
   array(o, "__align__(16) long long", "t_ax", as_ll(ax));
   array(o, "int", "t_seg", seg);
@@ -530,7 +592,21 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
     array(o, "__align__(16) double", "t_rd", as_d(rd));
     array(o, "double", "t_fx", as_d(fxa));
     array(o, "double", "t_h", as_d(hc));
-    if (vjp) {
+    if (jac) {
+      std::vector<double> cp;
+      for (auto& sp : m.species) {
+        const SpeciesCoef c = species_coef(sp);
+        for (int r = 0; r < 2; ++r) { cp.insert(cp.end(), c.cp[r], c.cp[r] + 5); cp.insert(cp.end(), c.cpd[r], c.cpd[r] + 4); cp.push_back(0.0); }
+      }
+      o << "#define T_MROWS " << mrows << "\n#define T_NROWS " << rows << "\n#define T_R " << lit((double)R_GAS) << "\n";
+      array(o, "double", "t_cp", as_d(cp));
+      array(o, "int", "t_jk", jk);
+      array(o, "__align__(16) int", "t_jl", jl);
+      array(o, "int", "t_jt", jt);
+      array(o, "int", "t_je", je);
+      array(o, "__align__(16) int", "t_jx", jx);
+      array(o, "double", "t_jc", as_d(jc));
+    } else if (vjp) {
       o << "#define T_MROWS " << mrows << "\n";
       array(o, "__align__(16) int", "t_vl", vl);
       array(o, "__align__(8) int", "t_v1", v1);
@@ -543,16 +619,17 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
     if (kv.first == 8) continue;
     const int c = kv.second;
     o << " \\\n  { const int a = __ldg(seg + " << c << "), b = __ldg(seg + " << c + 1 << "); if (a < b) "
-      << (vjp ? "vjp_plain<" : deriv ? "jvp_plain<" : "tile_plain<") << (kv.first & 2 ? 3 : 2) << ", " << (kv.first & 1 ? "true" : "false")
-      << (vjp ? ">(s, a, b, u, v, invT, invT2, Tb, lane); }" : deriv ? ">(s, a, b, u, v, u1, u2, lane); }" : ", SGN>(s, a, b, u, v, lane); }");
+      << (jac ? "jac_plain<" : vjp ? "vjp_plain<" : deriv ? "jvp_plain<" : "tile_plain<") << (kv.first & 2 ? 3 : 2) << ", " << (kv.first & 1 ? "true" : "false")
+      << (jac ? ">(s, a, b, u, v, invT, invT2, sum, lane); }" : vjp ? ">(s, a, b, u, v, invT, invT2, Tb, lane); }" : deriv ? ">(s, a, b, u, v, u1, u2, lane); }" : ", SGN>(s, a, b, u, v, lane); }");
   }
-  o << (vjp ? "\n#include \"pyro_tile_vjp.cuh\"\n" : deriv ? "\n#include \"pyro_tile_jvp.cuh\"\n" : "\n#include \"pyro_tile.cuh\"\n");
+  o << (jac ? "\n#include \"pyro_tile_jac.cuh\"\n" : vjp ? "\n#include \"pyro_tile_vjp.cuh\"\n" : deriv ? "\n#include \"pyro_tile_jvp.cuh\"\n" : "\n#include \"pyro_tile.cuh\"\n");
   out.source = o.str();
   out.warps = warps;
   out.smem_bytes = fixed_bytes + tile_rows * 256;
   out.t_lo = t_lo;
   out.chunks = chunks;
   out.rows = rows;
+  out.scratch_bytes = jac ? (2 * tile_rows + 2 * (mrows + 1)) * 256 : 0;
   return out;
 }
 

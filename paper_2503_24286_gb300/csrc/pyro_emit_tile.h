@@ -16,6 +16,7 @@ struct TileEmit {
   int smem_bytes = 0;      // dynamic shared memory per block
   double t_lo = 0.0;       // states at or below it are left to the FP64 kernel
   int chunks = 0, rows = 0;
+  int scratch_bytes = 0;   // global scratch per block (dense Jacobian)
 };
 
 // Dynamic shared memory an SM can hold, and what a resident block costs beside its own.
@@ -24,8 +25,9 @@ constexpr int kSmemPerBlock = 1024;
 constexpr int kSmemMaxBlock = 227 * 1024;
 
 // Kernels over the tables: net production rates (pyro_tile.cuh), Jacobian-vector product
-// (pyro_tile_jvp.cuh), vector-Jacobian product (pyro_tile_vjp.cuh).
-enum class TileKind { Rates, Jvp, Vjp };
+// (pyro_tile_jvp.cuh), vector-Jacobian product (pyro_tile_vjp.cuh), dense Jacobian
+// (pyro_tile_jac.cuh).
+enum class TileKind { Rates, Jvp, Vjp, Jac };
 TileEmit emit_tile_unit(const Mechanism& m, TileKind kind = TileKind::Rates);
 
 struct TransportTile {
@@ -41,5 +43,6 @@ extern const char* kTileSource;
 extern const char* kTransportSource;
 extern const char* kTileJvpSource;
 extern const char* kTileVjpSource;
+extern const char* kTileJacSource;
 
 }  // namespace pyro

@@ -117,10 +117,10 @@ const char* kArch = "sm_103a";
 bool nvrtc_compile(const std::string& src, std::vector<char>& cubin, std::string& log) {
   nvrtcProgram prog;
   const char* hdrs[] = {kDeviceMathSource, kFixedMathSource, kTileSource, kTransportSource,
-                        kTileJvpSource, kTileVjpSource};
+                        kTileJvpSource, kTileVjpSource, kTileJacSource};
   const char* names[] = {"pyro_device_math.cuh", "pyro_fixed_math.cuh", "pyro_tile.cuh", "pyro_transport.cuh",
-                         "pyro_tile_jvp.cuh", "pyro_tile_vjp.cuh"};
-  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 6, hdrs, names) != NVRTC_SUCCESS) {
+                         "pyro_tile_jvp.cuh", "pyro_tile_vjp.cuh", "pyro_tile_jac.cuh"};
+  if (nvrtcCreateProgram(&prog, src.c_str(), "pyro_mech.cu", 7, hdrs, names) != NVRTC_SUCCESS) {
     log = "nvrtcCreateProgram failed";
     return false;
   }
@@ -161,6 +161,7 @@ int compile_cached(const std::string& src, bool use_cache, std::vector<char>& cu
   if (src.find("\"pyro_tile.cuh\"") != std::string::npos) key_src += kTileSource;
   if (src.find("\"pyro_tile_jvp.cuh\"") != std::string::npos) key_src += std::string(kTileSource) + kTileJvpSource;
   if (src.find("\"pyro_tile_vjp.cuh\"") != std::string::npos) key_src += std::string(kTileSource) + kTileVjpSource;
+  if (src.find("\"pyro_tile_jac.cuh\"") != std::string::npos) key_src += std::string(kTileSource) + kTileJacSource;
   if (src.find("\"pyro_transport.cuh\"") != std::string::npos) key_src += kTransportSource;
   char hex[32];
   std::snprintf(hex, sizeof hex, "%016llx", (unsigned long long)fnv1a(key_src));
@@ -533,7 +534,8 @@ const char* group_kernel(const std::string& g) {
        : g == "cn" ? "pyro_cn_assemble" : g == "tr" ? "pyro_transport" : g == "wfwd" ? "pyro_omega_warp"
        : g == "wjvp" ? "pyro_jvp_warp" : g == "wvjp" ? "pyro_vjp_warp" : g == "wjac" ? "pyro_jacobian_cta"
        : g == "wjad" ? "pyro_jacobian_adiabatic_cta" : g == "tile" ? "pyro_omega_tile" : g == "ttr" ? "pyro_transport_tile"
-       : g == "tjvp" ? "pyro_jvp_tile" : g == "tvjp" ? "pyro_vjp_tile" : "pyro_jacobian";
+       : g == "tjvp" ? "pyro_jvp_tile" : g == "tvjp" ? "pyro_vjp_tile"
+       : g == "tjac" ? "pyro_jacobian_tile" : "pyro_jacobian";
 }
 
 // Compile (in parallel threads, cached on disk) and load the named derivative
@@ -579,6 +581,10 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
     if (todo[i][0] == 'w') {
       G.block = 32 * h->emitted.warp_wpb.at(todo[i]);
       G.smem = h->emitted.smem_dyn_bytes_warp.at(todo[i]);
+    }
+    if (todo[i] == "tjac") {
+      G.block = 32 * h->emitted.jac_tile_warps;
+      G.smem = h->emitted.smem_dyn_bytes_jac_tile;
     }
     if (todo[i] == "tvjp") {
       G.block = 32 * h->emitted.vjp_tile_warps;
@@ -630,10 +636,14 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
       h->emitted.stats[todo[i] + "_active_clusters"] = ncl;
     }
     if (h->emitted.stats["deriv_store_global"] > 0 && todo[i] != "jac" && todo[i] != "jad" && todo[i] != "cn" &&
-        todo[i] != "tile" && todo[i] != "ttr" && todo[i] != "tjvp" && todo[i] != "tvjp" && todo[i][0] != 'w') {
+        todo[i] != "tile" && todo[i] != "ttr" && todo[i] != "tjvp" && todo[i] != "tvjp" && todo[i] != "tjac" && todo[i][0] != 'w') {
       size_t bytes = (size_t)h->num_sms * nb * 4 * h->m.n_species() * h->opt.deriv_block * sizeof(double);
       cudaError_t e = cudaMalloc(&G.store, bytes);
       if (e != cudaSuccess) return fail(PYRO_ECUDA, std::string("species-array store allocation: ") + cudaGetErrorString(e));
+    }
+    if (todo[i] == "tjac") {   // per-block scratch of the rows (dR/dT, [M] terms)
+      cudaError_t e = cudaMalloc(&G.store, (size_t)h->num_sms * nb * h->emitted.jac_tile_scratch_bytes);
+      if (e != cudaSuccess) return fail(PYRO_ECUDA, std::string("Jacobian scratch allocation: ") + cudaGetErrorString(e));
     }
     if (todo[i] == "cn") {
       for (const char* nm : {"pyro_cn_prep", "pyro_cn_solve", "pyro_cn_finish", "pyro_cn_residual"}) {
@@ -716,6 +726,15 @@ std::vector<std::string> product_groups(const pyro_mech* h, const std::string& w
   auto it = h->emitted.stats.find(which + "_tile");
   if (it == h->emitted.stats.end() || it->second <= 0) return {which};
   return {which, "t" + which};
+}
+
+// the kernels of the dense Jacobian: as above, or the block-per-state kernel of variant=warp
+std::string jac_group(const pyro_mech* h, bool adiabatic);
+std::vector<std::string> jac_groups(const pyro_mech* h) {
+  const std::string g = jac_group(h, false);
+  auto it = h->emitted.stats.find("jacobian_tile");
+  if (g != "jac" || it == h->emitted.stats.end() || it->second <= 0) return {g};
+  return {g, "tjac"};
 }
 
 int launch_deriv(const pyro_mech* h, const pyro_mech::Group& G, int64_t n, void* stream, void** params);
@@ -1078,7 +1097,7 @@ int pyro_mech_prepare(const pyro_mech* hc, const char* kernels) {
   std::string k = kernels ? kernels : "all";
   std::vector<std::string> names;
   if (k == "all") {
-    names = {jac_group(h, false)};
+    names = jac_groups(h);
     for (const char* which : {"jvp", "vjp"}) for (auto& g : product_groups(h, which)) names.push_back(g);
   }
   else {
@@ -1086,7 +1105,7 @@ int pyro_mech_prepare(const pyro_mech* hc, const char* kernels) {
     std::stringstream ss(k);
     while (std::getline(ss, item, ',')) {
       if (item == "jvp" || item == "vjp") { for (auto& g : product_groups(h, item)) names.push_back(g); }
-      else if (item == "jacobian" || item == "jac") names.push_back(jac_group(h, false));
+      else if (item == "jacobian" || item == "jac") { for (auto& g : jac_groups(h)) names.push_back(g); }
       else if (item == "jacobian_adiabatic" || item == "jad") names.push_back(jac_group(h, true));
       else if (item == "cn" || item == "crank_nicolson") names.push_back("cn");
       else if (item == "warp" || item == "wfwd") names.push_back("wfwd");
@@ -1149,8 +1168,9 @@ int pyro_jacobian(const pyro_mech* hc, int64_t n, const double* rho, const doubl
     return fail(PYRO_EINVAL, "the dense Jacobian kernels need all species to share one NASA-7 T_mid");
   if (n == 0) return PYRO_OK;
   if (int rc = check_device(h)) return rc;
-  const std::string g = jac_group(h, false);
-  if (int rc = ensure_groups(h, {g})) return rc;
+  const std::vector<std::string> gs = jac_groups(h);
+  const std::string& g = gs[0];
+  if (int rc = ensure_groups(h, gs)) return rc;
   const pyro_mech::Group& G = h->groups[g];
   const bool cta = g[0] == 'w';
   int NP = h->m.n_species() + 1;
@@ -1160,7 +1180,15 @@ int pyro_jacobian(const pyro_mech* hc, int64_t n, const double* rho, const doubl
   return with_args(h, n, {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false}, {J, (int64_t)NP * NP, 8, false, true}},
                    stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
                      long long nn = nc;
-                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &h->d_jac_scratch};
+                     int open_only = gs.size() > 1 ? 1 : 0;
+                     if (open_only) {
+                       pyro_mech::Group& t = h->groups[gs[1]];
+                       void* pt[] = {&nn, &d[0], &d[1], &d[2], &d[3], &t.store};
+                       const unsigned grid = (unsigned)std::min((nc + 31) / 32, (int64_t)h->num_sms * t.blocks_per_sm);
+                       CUresult r = driver().LaunchKernel(t.f, grid, 1, 1, t.block, 1, 1, t.smem, as_stream(st), pt, nullptr);
+                       if (r != CUDA_SUCCESS) return fail(PYRO_ECUDA, "kernel launch: " + cu_err(r));
+                     }
+                     void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &h->d_jac_scratch, &open_only};
                      return cta ? launch_cta(h, G, nc, st, params) : launch_deriv(h, G, nc, st, params);
                    }, cta);
 }

@@ -1,4 +1,4 @@
-"""The JVP's and the VJP's tile kernels against the oracle where its dispatch or its number formats can go
+"""The tile kernels of the JVP, the VJP and the dense Jacobian against the oracle where its dispatch or its number formats can go
 wrong: ragged tiles, states outside its tables beside ordinary ones, absent, negative and tiny
 mass fractions, zero and huge tangents, and every reaction class.  Tolerance: 1e-11 of each
 entry's gross scale (as in test_gpu_derivatives), with that suite's absolute floor of 1e-250."""
@@ -131,3 +131,48 @@ def test_vjp_nan_stays_in_its_state(mechs):
     T[12] = np.nan
     g = _check_vjp(m, orc, rho, T, Y, wb, skip=(10, 11, 12))
     assert np.isnan(g[1, 10]) and np.isnan(g[1, 11]) and np.isnan(g[1, 12])
+
+
+def _check_jac(m, orc, rho, T, Y, skip=()):
+    NP = orc.N + 1
+    J = m.jacobian(_t(rho), _t(T), _t(Y)).cpu().numpy().reshape(NP, NP, -1)
+    Jo = orc.jacobian(rho, T, Y).reshape(NP, NP, -1)
+    G = orc.jacobian_gross(rho, T, Y)[:, 1:]
+    fine = np.isfinite(Jo).all(axis=(0, 1)) & np.isfinite(G).all(axis=(0, 1))
+    keep = np.setdiff1d(np.arange(T.size)[fine], skip)
+    assert keep.size >= 0.8 * T.size
+    assert np.all(np.isfinite(J[..., keep]))
+    assert np.all(np.abs(J - Jo)[..., keep] <= 1e-11 * G[..., keep] + 1e-250)
+    return J
+
+
+@pytest.mark.parametrize("name,idx", [("h2", 0), ("gri", 1), ("pdep", 7)])
+@pytest.mark.parametrize("n", [1, 31, 33])
+def test_jacobian_ragged_tiles(mechs, name, idx, n):
+    m, orc = mechs[name]
+    assert m.stat("jacobian_tile") == 1
+    _check_jac(m, orc, *_inputs(orc, idx, n, 81 + n)[:3])
+
+
+@pytest.mark.parametrize("name,idx", [("h2", 0), ("gri", 1), ("pdep", 7)])
+def test_jacobian_open_states_and_compositions(mechs, name, idx):
+    m, orc = mechs[name]
+    rho, T, Y = _inputs(orc, idx, 48, 82)[:3]
+    rng = np.random.default_rng(83)
+    N = orc.N
+    T[[3, 40, 41]] = [190.0, 5000.0, 5400.0]
+    rho[5] = 1e-22
+    Y[:, 8:20] = np.where(rng.random((N, 12)) < 0.6, 0.0, Y[:, 8:20])
+    Y[:, 20:30] *= np.where(rng.random((N, 10)) < 0.3, -1e-6, 1.0)
+    Y[:, 30:36] = 10.0 ** rng.uniform(-60, -1, (N, 6))
+    _check_jac(m, orc, rho, T, Y)
+
+
+def test_jacobian_nan_stays_in_its_state(mechs):
+    m, orc = mechs["gri"]
+    rho, T, Y = _inputs(orc, 1, 40, 84)[:3]
+    Y[4, 10] = np.nan
+    T[12] = np.nan
+    J = _check_jac(m, orc, rho, T, Y, skip=(10, 12))
+    # (the inert species takes part in no reaction: its row stays zero)
+    assert np.isnan(J[..., 10]).any() and np.isnan(J[0, :, 12]).all()
