@@ -1,5 +1,9 @@
 // Emitter: mechanism -> CUDA C specialised to that mechanism (sm_103a).
 //
+// Where a mechanism fits the tile kernels' tables (pyro_emit_tile.cpp), they evaluate
+// almost every state and the per-thread kernels emitted here the states that those leave
+// open (their open_only argument).
+//
 // Work split: one thread per state point, straight-line code per species and per
 // reaction with every mechanism constant folded into immediates.  Per-point
 // species quantities are staged in shared memory in [species][thread] layout
@@ -92,10 +96,13 @@ void emit_tsolve(Src& s, const Mechanism& m, const std::vector<SpeciesCoef>& C, 
   // Tables, one row per species (rows past the last one are zero).  FP32: the energy
   // coefficients d_0..d_5 of both ranges and the enthalpy's d_1 + 1/W.  FP64 and integer:
   // per range d_0..d_5, d_1 + 1/W.  An integer column m is scaled by 2^s_m with its largest
-  // coefficient in [2^(hb-1), 2^hb), hb = min(57, 62 - ceil(log2 N)): the sums of
-  // products of halves, the high one shifted by 7, then stay below 2^63 while sum |Y| < 2.
+  // coefficient in [2^(hb-1), 2^hb), hb = min(57, 62 - ceil(log2 n)): the sums of
+  // products of halves over n species, the high one shifted by 7, then stay below 2^63
+  // while sum |Y| < 2.  Above 64 rows the sums are taken in runs of n = 32 (hb = 57; by all
+  // of 160 species hb was 54, and the mean error of T 2.2e-15; now 1.2e-16).
+  const int run = NP > 64 ? 32 : N;
   int hb = 57;
-  while ((1 << (62 - hb)) < N) --hb;
+  while ((1 << (62 - hb)) < run) --hb;
   auto coef = [&](int k, int r, int q) { return q < 6 ? C[k].d[r][q] : C[k].d[r][1] + 1.0 / m.species[k].W; };
   int sc[7];
   for (int q = 0; q < 7; ++q) {
@@ -142,12 +149,13 @@ __device__ __noinline__ void ts_collapse64(const double* __restrict__ Yp, i64 n,
 
 // The same on the integer pipe, exact up to the 2^-61 of Y and the coefficients' 2^-hb.
 // The FP64 form takes 6 N = 318 FP64 instructions for 53 species, 6,000 cycles of an SM per
-// warp against ~2,000 of the integer form: 2^20 temperatures 0.72 ms with FP64.
+// warp: 2^20 temperatures 725 us with FP64, 513 us in this form (bound by instruction issue).
 template <bool ENTH>
 __device__ __forceinline__ void ts_collapse(const double* __restrict__ Yp, i64 n, bool hi, double (&B)[6]) {
-  i64 h[6], l[6];
+  i64 h[6], l[6], s[6];
+  auto fold = [&](int q) { return (h[q] << 7) + ((l[q] + 0x1000000ll) >> 25); };   // h 2^64 + l 2^32 in units of 2^57
 #pragma unroll
-  for (int q = 0; q < 6; ++q) h[q] = l[q] = 0;
+  for (int q = 0; q < 6; ++q) h[q] = l[q] = s[q] = 0;
 #pragma unroll 1
   for (int k0 = 0; k0 < NSP; k0 += 8) {
     double y[8];
@@ -168,10 +176,14 @@ __device__ __forceinline__ void ts_collapse(const double* __restrict__ Yp, i64 n
         l[q] += (i64)pfx::mulhi_s(cl, v.lo);
       }
     }
+    if (TS_ROWS > 64 && (k0 & 24) == 24) {       // a run of 32 species
+#pragma unroll
+      for (int q = 0; q < 6; ++q) { s[q] += fold(q); h[q] = l[q] = 0; }
+    }
   }
 #pragma unroll
-  for (int q = 0; q < 6; ++q)      // h 2^64 + l 2^32 = (h 2^7 + l 2^-25) 2^57
-    B[q] = pfx::scaled((h[q] << 7) + ((l[q] + 0x1000000ll) >> 25), 57 - __ldg(ts_s + (ENTH && q == 1 ? 6 : q)));
+  for (int q = 0; q < 6; ++q)
+    B[q] = pfx::scaled(s[q] + fold(q), 57 - __ldg(ts_s + (ENTH && q == 1 ? 6 : q)));
 }
 
 // Newton inversion of e = sum_k Y_k e_k(T) (Sec. A.3.1, Eq. delta_temp), or with

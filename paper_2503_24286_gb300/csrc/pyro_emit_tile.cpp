@@ -161,19 +161,6 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
   std::vector<i64> sp((size_t)N * 16);
   std::vector<double> hc;                        // h_k/(RT) = h0 + ... + h4 T^4 + h5/T
   std::vector<double> ed((size_t)N * 12), iw(N);
-  // integer energy coefficients: column q scaled by 2^xs[q], the largest in [2^(hb-1), 2^hb),
-  // so that sums over the species stay below 2^63 while sum |Y| < 2 (TileDot)
-  std::vector<i64> ex((size_t)N * 12);
-  std::vector<int> xs(6, 0);
-  {
-    int hb = 57;
-    while ((1 << (62 - hb)) < N) --hb;
-    for (int q = 0; q < 6; ++q) {
-      double mx = 0.0;
-      for (auto& sp : m.species) { const SpeciesCoef C = species_coef(sp); for (int r = 0; r < 2; ++r) mx = std::max(mx, std::fabs(C.d[r][q])); }
-      if (mx > 0.0) xs[q] = hb - 1 - std::ilogb(mx);
-    }
-  }
   std::ostringstream ef;
   for (int k = 0; k < N; ++k) {
     const Species& s = m.species[k];
@@ -194,10 +181,7 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
       q[6] = fx.coef((ld)a[5] * LOG2E / T_V);
       q[7] = 0;
       hc.insert(hc.end(), C.h[r], C.h[r] + 6);
-      for (int i = 0; i < 6; ++i) {
-        ed[((size_t)k * 2 + r) * 6 + i] = C.d[r][i];
-        ex[((size_t)k * 2 + r) * 6 + i] = fx.pair(llroundl(ldexpl((ld)C.d[r][i], xs[i])));
-      }
+      for (int i = 0; i < 6; ++i) ed[((size_t)k * 2 + r) * 6 + i] = C.d[r][i];
     }
     for (int r = 0; r < 2; ++r) for (int i = 0; i < 6; ++i) ef << (k + r + i ? "," : "") << litf(C.d[r][i]);
   }
@@ -246,6 +230,22 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
   auto red = [](int w) { return w * 256 + 6 * 256 + 14 * 128 + w * 13 * 128; };   // scratch of the temperature solve, in the rows
   while (minb > 1 && fixed_bytes + std::max(rows_all * 256, red(warps)) > kSmemPerSm / minb - kSmemPerBlock) --minb;
   if (minb == 1) warps = 24;
+
+  // integer energy coefficients: column q scaled by 2^xs[q], the largest in [2^(hb-1), 2^hb),
+  // so that a warp's sums over its species stay below 2^63 while sum |Y| < 2 (TileDot).  By
+  // the number of all species, hb was 54 for 160 of them: the largest coefficients are the
+  // light species', ~100 times the mixture's, and the mean error of T was 2.2e-15; now it is 1.5e-16 (FP64 sums 5.4e-16).
+  std::vector<i64> ex((size_t)N * 12);
+  std::vector<int> xs(6, 0);
+  int hb = 57;
+  while ((1 << (62 - hb)) < (N + warps - 1) / warps) --hb;
+  for (int q = 0; q < 6; ++q) {
+    double mx = 0.0;
+    for (int i = q; i < 12 * N; i += 6) mx = std::max(mx, std::fabs(ed[i]));
+    if (mx > 0.0) xs[q] = hb - 1 - std::ilogb(mx);
+    for (int i = q; i < 12 * N; i += 6) ex[i] = fx.pair(llroundl(ldexpl((ld)ed[i], xs[q])));
+  }
+
   const int lim = std::min(kSmemMaxBlock, kSmemPerSm / minb - kSmemPerBlock) - fixed_bytes;
   const int max_rows = lim / 256;
   if (lim < red(warps) || max_rows < 8) { out.why = "species arrays do not fit in shared memory"; return out; }
