@@ -70,6 +70,13 @@ typedef struct pyro_mech pyro_mech;
  *   exp=4|2|4call|2call (device exponential: 4 FP64-pipe operations (default)
  *                        or 2 with the second-order terms in FP32 pairs; inlined
  *                        at every use, or one called body)
+ *                        -- of the per-thread kernels; where the mechanism fits the
+ *                        tile kernels' tables they evaluate almost every state: 32
+ *                        states per block with exponents in 64-bit fixed point
+ *                        (net production rates, and without variant=warp the JVP,
+ *                        the VJP and the dense Jacobian; transport), and the
+ *                        per-thread or per-warp kernel the states beyond those
+ *                        tables (T outside about 200..5000 K, NaN, ...)
  *   warp_exp=2|4        (the exponential of the warp-per-state kernels: 2 FP64-pipe
  *                        operations (default; their code is compact) or 4)
  *   variant=thread|warp (net production rates: one thread per state with
