@@ -31,8 +31,8 @@
 // third-body concentrations and the blending factors of falloff reactions.
 //
 // States outside the tables' range (temperature outside (T_LO, T_HI), NaN,
-// infinite or subnormal mass fractions or ones from 2, densities beyond 2^-60..2^20,
-// [M] <= 0) get TILE_OPEN in their first output; the caller then launches the FP64
+// infinite or subnormal mass fractions or ones from 2, densities beyond 2^-60..2^20, a
+// falloff or PLOG reaction with [M] <= 0) get TILE_OPEN in their first output; the caller then launches the FP64
 // kernel, which evaluates the states so marked.
 #include "pyro_device_math.cuh"
 #include "pyro_fixed_math.cuh"
@@ -389,10 +389,14 @@ __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, in
       asm volatile("prefetch.global.L1 [%0];" ::"l"(pre));
     }
     const int ne = (int)__ldg(ax);
-    // log2 [M] of the reaction (PLOG: of the total concentration)
+    // log2 [M] of the reaction (PLOG: of the total concentration).  A third body's [M] is a
+    // factor of the rate and may be zero or negative (efficiencies of 0 whose sum cancels,
+    // undershoots); the other classes need a positive one.
+    const bool third = kind == TK_THREEBODY;
     const double M = rho * tile_mS(ax + 16, ne, ysum, Yp, n);
-    if (!tile_normal_pos(M)) s.sc->bad[lane] = 1;
-    const i64 lgM = pfx::log2_of(M, t_log2);
+    const bool normal = tile_normal_pos(third ? fabs(M) : M), none = third && M == 0.0;
+    if (!normal && !none) s.sc->bad[lane] = 1;
+    const i64 lgM = pfx::log2_of(normal ? fabs(M) : 1.0, t_log2);
     i64 X;
     if (kind == TK_PLOG) {
       // log2 k linear in log2 p between the bracketing nodes, end nodes outside
@@ -409,7 +413,7 @@ __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, in
     } else {
       X = tile_K(__ldg(r), __ldg(r + 1), __ldg(r + 2), u, v);
     }
-    if (kind == TK_THREEBODY) X += lgM;
+    if (third) X += lgM;
     if (kind >= TK_LINDEMANN && kind <= TK_SRI) {
       const i64 lgPr = tile_K(__ldg(ax + 2), __ldg(ax + 3), __ldg(ax + 4), u, v) + lgM;
       // log2(Pr/(1+Pr)) = min(lgPr, 0) - log2(1 + 2^-|lgPr|)
@@ -428,8 +432,9 @@ __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, in
           const i64 x = pfx::mul_add(as_pair(__ldg(e + 1)), t, pfx::mul_add(as_pair(__ldg(e + 2)), v, 0ll)) & ~1ll;
           S += pfx::exp2_lg(x + __ldg(e), s.exp2);
         }
-        if (!tile_normal_pos(S)) s.sc->bad[lane] = 1;
-        const i64 lS = pfx::log2_of(S, t_log2);
+        const bool pos = tile_normal_pos(S);
+        if (!pos) s.sc->bad[lane] = 1;
+        const i64 lS = pfx::log2_of(pos ? S : 1.0, t_log2);
         // Troe: log F = log F_cent den^2/(den^2 + x^2), all logarithms to base 10;
         // SRI: F = d S^(1/(1 + log10^2 Pr)) T^e
         double x = pfx::to_double(lgPr) * 0.30102999566398119521, den2 = 1.0;
@@ -443,7 +448,7 @@ __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, in
         if (kind == TK_SRI) X += pfx::mul_add(as_pair(__ldg(ax + 15)), u, __ldg(ax + 14));
       }
     }
-    X &= ~1ll;
+    X = (X & ~1ll) | (i64)(third && M < 0.0);
     // factors
     i64 Xf = 0, Xr = np ? 0ll : pfx::LG_ZERO;
     for (int q = 0; q < nr; ++q) {
@@ -455,7 +460,8 @@ __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, in
       const int k = (int)((q == 0 ? (fa >> 48) : (fb >> (16 * (q - 1)))) & 0xffff) * 32;
       Xr += alp[k];
     }
-    s.R[(int)((fb >> 32) & 0xffff) * 32 + lane] = tile_rate<true, true>(X + Xf, X + Xr, s.exp2);
+    const i64 rate = tile_rate<true, true>(X + Xf, X + Xr, s.exp2);
+    s.R[(int)((fb >> 32) & 0xffff) * 32 + lane] = none ? 0ll : rate;
   }
 }
 
@@ -618,7 +624,7 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
       __syncthreads();
     }
     const Pair u = s.sc->u[lane], v = s.sc->v[lane];
-    const bool open = s.sc->bad[lane] != 0, signs = s.sc->neg != 0;
+    const bool signs = s.sc->neg != 0;
 #pragma unroll 1
     for (int ch = rank; ch < (split ? rank + 1 : NCH); ++ch) {
       const int* seg = t_seg + (ch * NW + w) * (NCLS + 1);
@@ -638,6 +644,7 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         }
       }
       __syncthreads();
+      const bool open = s.sc->bad[lane] != 0;         // behind the barrier: reactions set it too
       tile_sums(s.R + lane, ch, w, [&](int k, double v) {
         if (split) {
           ((double*)s.lam)[k * 32 + lane] = v;       // the species arrays are free after the only chunk
