@@ -135,7 +135,7 @@ TransportTile emit_transport_tile(const Mechanism& m) {
   for (auto& R : recs) pt.insert(pt.end(), R.begin(), R.end());
   for (int i = 0; i < 8; ++i) pt.push_back(0);
 
-  const int smem = 5 * N * 256 + 4 * nw * 256 + 3 * 256 + 256 + 128 + 64;
+  const int smem = 5 * N * 256 + 4 * nw * 256 + nw * 128 + 3 * 256 + 256 + 128 + 64;
   if (smem > kSmemMaxBlock) return out;
   int minb = std::max(1, std::min({kSmemPerSm / (smem + kSmemPerBlock), 832 / (32 * nw)}));
 

@@ -14,7 +14,7 @@
 //    of a tournament: the pairs of a round share no species, so the warps update the
 //    sums of both species of a pair without conflicts, with a barrier per round.
 // States outside the tables' range (T outside (TT_LO, TT_HI), mole fractions or scaled
-// x/P beyond 2 in magnitude, NaN) get TILE_OPEN in the first output that is given and
+// x/P beyond 2 in magnitude, sum |x| from 2, NaN) get TILE_OPEN in the first output that is given and
 // are evaluated by the FP64 kernel launched behind.
 #include "pyro_device_math.cuh"
 #include "pyro_fixed_math.cuh"
@@ -30,7 +30,9 @@ __device__ __forceinline__ Pair tt_pair(i64 v) {
   return p;
 }
 
-// sum of c y: h 2^64 + l 2^32 (products of the low halves, below 2^-54 of the sum, left out)
+// sum of c y: h 2^64 + l 2^32 (products of the low halves, below 2^-54 of the sum, left out).
+// With |c| < 2^57 and y = x 2^61 the word h << 7 stays below 2^61 sum |x|, and l below
+// 2^60 sum |x| + N 2^55.
 struct TtDot {
   i64 h, l;
   __device__ __forceinline__ void add(i64 c, Pair y) {
@@ -65,6 +67,7 @@ __device__ __forceinline__ double tt_rcp(i64 v, int s) {
 
 struct TtShared {
   double ys[NW * 32], mu[NW * 32], ka[NW * 32], kh[NW * 32];
+  float xa[NW * 32];                           // sum |x|
   double rys[32], td[32], sqT[32];
   Pair t[32];
   int bad[32];
@@ -121,6 +124,7 @@ pyro_transport_tile(i64 n, const double* __restrict__ g_T, const double* __restr
     __syncthreads();
     const double td = sh.td[lane], rys = sh.rys[lane];
     double ka = 0.0, kh = 0.0;
+    float xa = 0.f;
     bool bad = false;
 #pragma unroll 1
     for (int k = w; k < NSP; k += NW) {
@@ -131,7 +135,7 @@ pyro_transport_tile(i64 n, const double* __restrict__ g_T, const double* __restr
       const double K = fma(td, fma(td, fma(td, fma(td, c4.y, c4.x), c3.y), c3.x), c2.y);
       const double rP = pdm::rcp(P), v = rP * x, q = v * rP;
       const double vs = v * TT_SV, ws = q * TT_SW;
-      bad |= !(fabs(x) < 1.9 && fabs(vs) < 1.9 && fabs(ws) < 1.9);
+      bad |= !(fabs(vs) < 1.9 && fabs(ws) < 1.9);
       sx[k * 32 + lane] = x;
       sP[k * 32 + lane] = P;
       fx[k * 32 + lane] = pfx::fix61(x);
@@ -139,7 +143,9 @@ pyro_transport_tile(i64 n, const double* __restrict__ g_T, const double* __restr
       fw[k * 32 + lane] = pfx::fix61(ws);
       ka = fma(x, K, ka);
       kh = fma(x, pdm::rcp(K), kh);
+      xa += fabsf(pdm::to_float_trunc(x));
     }
+    sh.xa[w * 32 + lane] = xa;
     sh.ka[w * 32 + lane] = ka;
     sh.kh[w * 32 + lane] = kh;
     if (bad) sh.bad[lane] = 1;
@@ -170,6 +176,11 @@ pyro_transport_tile(i64 n, const double* __restrict__ g_T, const double* __restr
       double ka = 0.0, kh = 0.0, mu = 0.0;
 #pragma unroll
       for (int i = 0; i < NW; ++i) { ka += sh.ka[i * 32 + lane]; kh += sh.kh[i * 32 + lane]; }
+      // Wilke's integer sums: their top word stays below 2^63 while sum |x| < 2 (TtDot)
+      float xs = 0.f;
+#pragma unroll
+      for (int i = 0; i < NW; ++i) xs += sh.xa[i * 32 + lane];
+      if (!(xs < 2.f)) sh.bad[lane] = 1;
       if (g_mu) {
 #pragma unroll
         for (int i = 0; i < NW; ++i) mu += sh.mu[i * 32 + lane];
