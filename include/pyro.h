@@ -69,26 +69,31 @@ typedef struct pyro_mech pyro_mech;
  *   deriv_block=<threads per block of the derivative kernels, default 64>
  *   exp=4|2|4call|2call (device exponential: 4 FP64-pipe operations (default)
  *                        or 2 with the second-order terms in FP32 pairs; inlined
- *                        at every use, or one called body)
- *                        -- of the per-thread kernels; where the mechanism fits the
- *                        tile kernels' tables they evaluate almost every state: 32
- *                        states per block with exponents in 64-bit fixed point
- *                        (net production rates, and without variant=warp the JVP,
- *                        the VJP and the dense Jacobian; transport), and the
- *                        per-thread or per-warp kernel the states beyond those
- *                        tables (T outside about 200..5000 K, NaN, ...)
+ *                        at every use, or one called body), of the per-thread kernels
+ *   tile=auto|0         (auto, default: where the mechanism fits their tables, the
+ *                        tile kernels -- 32 states per block, exponents in 64-bit
+ *                        fixed point -- evaluate the net production rates,
+ *                        transport and, without variant=warp, the JVP, the VJP and
+ *                        the dense Jacobian; states beyond the tables (T at or below
+ *                        pyro_mech_stat("tile_t_lo") or from 5000 K, NaN, fractions
+ *                        from 2 in magnitude, a falloff [M] <= 0, ...) are evaluated
+ *                        by the FP64 kernel launched behind, the only place where
+ *                        block=, exp=, variant= and store= then act on those calls;
+ *                        0: the FP64 kernels alone)
  *   warp_exp=2|4        (the exponential of the warp-per-state kernels: 2 FP64-pipe
  *                        operations (default; their code is compact) or 4)
- *   variant=thread|warp (net production rates: one thread per state with
+ *   variant=thread|warp (the FP64 kernels: one thread per state with
  *                        mechanism-specialised straight-line code (default),
  *                        or one warp per state (pyro_net_production_rates,
  *                        pyro_jvp, pyro_vjp): the lanes split the species and
  *                        the reactions, in chunks of 32 reactions emitted for
- *                        the mechanism's reaction classes -- the faster form for
- *                        large mechanisms such as 160 species / 1100 reactions;
- *                        pyro_jacobian and pyro_jacobian_adiabatic then run one
- *                        block of 8 warps per state, in clusters of 4 blocks on
- *                        4 consecutive states, with no per-handle scratch).
+ *                        the mechanism's reaction classes -- the faster FP64 form
+ *                        for large mechanisms such as 160 species / 1100
+ *                        reactions (the JVP of a default handle, by its tile
+ *                        kernel, is faster still); pyro_jacobian and
+ *                        pyro_jacobian_adiabatic then run one block of 8 warps
+ *                        per state, in clusters of 4 blocks on 4 consecutive
+ *                        states, with no per-handle scratch).
  *                        variant=warp needs at most three factors on each side
  *                        of a reaction and one NASA-7 T_mid for all species
  *                        (PYRO_EINVAL otherwise)
@@ -211,8 +216,9 @@ int pyro_vjp(const pyro_mech* mech, int64_t n, const double* rho, const double* 
  * per-handle scratch buffer for the per-reaction partials (allocated on first
  * use, grown as needed; 8 B x pyro_mech_stat("jacobian_scratch_doubles_per_point")
  * x deriv_block (default 64) x the resident blocks: with the defaults ~0.6 GB for
- * 53 species, ~3 GB for 160 species and 1100 reactions): calls on one handle that use it (pyro_jacobian,
- * pyro_jacobian_adiabatic, pyro_cn_step) must not overlap on the GPU.  Handles
+ * 53 species, ~3 GB for 160 species and 1100 reactions; the tile kernel's rows
+ * beside it take ~30 MB for 53 species): calls on one handle that use it
+ * (pyro_jacobian, pyro_jacobian_adiabatic, pyro_cn_step) must not overlap on the GPU.  Handles
  * loaded with variant=warp use the block-per-state kernels instead, which keep
  * the partials in shared memory and need no scratch (their calls may overlap).
  * Needs all species to share one NASA-7 T_mid. */
@@ -334,11 +340,11 @@ int pyro_mlp_load(pyro_mech* mech, const char* path);
  *  - Every call on a device shares the one scratch array, which keeps the
  *    previous call's contents (the failure counter is cleared by each call):
  *    calls that overlap on the GPU (other streams, other host threads) race.
- *  - It runs the same kernel as pyro_net_production_rates on this handle (one
- *    thread or one warp per state, see variant=).  With the thread kernel and
- *    the species arrays in the handle's global scratch (store=global, e.g. 160
- *    species) it also uses that scratch, so it must not overlap on the GPU with
- *    a pyro_net_production_rates call on the same handle either.
+ *  - It runs the same kernels as pyro_net_production_rates on this handle (see
+ *    tile= and variant=).  With the thread kernel and the species arrays in the
+ *    handle's global scratch (store=global, e.g. 160 species) it also uses that
+ *    scratch, so it must not overlap on the GPU with a
+ *    pyro_net_production_rates call on the same handle either.
  *  - The call is synchronous (returns after the results are copied out) and
  *    returns PYRO_ENOCONV if a Newton solve failed (input_is_energy != 0). */
 #define PYRO_NOALLOC_SCRATCH_BYTES (32u << 20)

@@ -2399,7 +2399,7 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
   }
   out.stats["has_transport"] = m.has_transport ? 1 : 0;
   {
-    const TransportTile t = emit_transport_tile(m);
+    const TransportTile t = opt.tile ? emit_transport_tile(m) : TransportTile();
     out.stats["transport_tile"] = t.source.empty() ? 0 : 1;
     if (!t.source.empty()) {
       out.group_sources["ttr"] = t.source;
@@ -2444,7 +2444,8 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
   }
   {
     // tile kernel of the net production rates (the form that evaluates almost every state)
-    const TileEmit t = emit_tile_unit(m);
+    const TileEmit none;
+    const TileEmit t = opt.tile ? emit_tile_unit(m) : none;
     out.stats["tile"] = t.source.empty() ? 0 : 1;
     if (!t.source.empty()) {
       out.group_sources["tile"] = t.source;
@@ -2455,21 +2456,21 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
       out.stats["tile_warps"] = t.warps;
       out.stats["tile_chunks"] = t.chunks;
     }
-    const TileEmit j = emit_tile_unit(m, TileKind::Jvp);
+    const TileEmit j = opt.tile ? emit_tile_unit(m, TileKind::Jvp) : none;
     out.stats["jvp_tile"] = j.source.empty() ? 0 : 1;
     if (!j.source.empty()) {
       out.group_sources["tjvp"] = j.source;
       out.jvp_tile_warps = j.warps;
       out.smem_dyn_bytes_jvp_tile = j.smem_bytes;
     }
-    const TileEmit v = emit_tile_unit(m, TileKind::Vjp);
+    const TileEmit v = opt.tile ? emit_tile_unit(m, TileKind::Vjp) : none;
     out.stats["vjp_tile"] = v.source.empty() ? 0 : 1;
     if (!v.source.empty()) {
       out.group_sources["tvjp"] = v.source;
       out.vjp_tile_warps = v.warps;
       out.smem_dyn_bytes_vjp_tile = v.smem_bytes;
     }
-    const TileEmit q = common_tmid(m) ? emit_tile_unit(m, TileKind::Jac) : TileEmit();
+    const TileEmit q = opt.tile && common_tmid(m) ? emit_tile_unit(m, TileKind::Jac) : none;
     out.stats["jacobian_tile"] = q.source.empty() ? 0 : 1;
     if (!q.source.empty()) {
       out.group_sources["tjac"] = q.source;

@@ -28,6 +28,7 @@ struct EmitOptions {
   int warp_exp_ops = 2;       // the same for the warp-per-state kernels (their code is compact, so
                               // the 2-operation form does not outgrow the instruction cache)
   bool exp_call = false;      // one called body instead of inlining at every use
+  bool tile = true;           // emit the tile kernels of a mechanism that fits their tables
 };
 
 struct EmitResult {

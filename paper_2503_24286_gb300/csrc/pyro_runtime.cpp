@@ -194,13 +194,14 @@ struct Options {
   bool device = true;     // false: parse, validate, emit and compile only (no CUDA device needed)
   int deriv_block = 64;   // threads per block of the derivative kernels
   int store = 0;          // 0 auto, 1 shared memory, 2 global scratch (per-state species arrays)
-  bool warp = false;      // net production rates: warp per state (table-driven) instead of thread per state
+  bool warp = false;      // FP64 kernels: warp per state instead of thread per state
   int exp_ops = 4;        // exponential flavour (4 or 2 FP64 ops)
   int warp_exp_ops = 2;   // the warp-per-state kernels' exponential (compact code: 2 FP64 ops by default)
   bool exp_call = false;  // exponential as a called function
   bool cn_chord = false;  // Crank-Nicolson: keep a factorisation for several iterations (chord) instead of full Newton
   int cn_refresh = 4;     // chord: re-assemble and re-factor every cn_refresh-th iteration
   int jac_rows = 0;       // Jacobian row assembly: 0 auto (tables above 64 species), 1 inline, 2 tables
+  bool tile = true;       // the tile kernels where the mechanism fits their tables; false: the FP64 kernels alone
 };
 
 bool parse_options(const char* s, Options& o, std::string& err) {
@@ -232,6 +233,7 @@ bool parse_options(const char* s, Options& o, std::string& err) {
       else { err = "exp=2|4|2call|4call"; return false; }
     }
     else if (k == "jac_rows") { if (v == "auto") o.jac_rows = 0; else if (v == "inline") o.jac_rows = 1; else if (v == "table") o.jac_rows = 2; else { err = "jac_rows=auto|inline|table"; return false; } }
+    else if (k == "tile") { if (v == "auto") o.tile = true; else if (v == "0") o.tile = false; else { err = "tile=auto|0"; return false; } }
     else if (k == "cn_refresh") { o.cn_refresh = std::atoi(v.c_str()); if (o.cn_refresh < 1 || o.cn_refresh > 1000) { err = "cn_refresh must be in [1, 1000]"; return false; } }
     else if (k == "cn_newton") { if (v == "full") o.cn_chord = false; else if (v == "chord") o.cn_chord = true; else { err = "cn_newton=full|chord"; return false; } }
     else if (k == "variant") { if (v == "thread") o.warp = false; else if (v == "warp") o.warp = true; else { err = "variant=thread|warp"; return false; } }
@@ -848,6 +850,7 @@ int pyro_mech_load(const char* mech_path, const char* options, pyro_mech** out) 
   eo.exp_ops = h->opt.exp_ops;
   eo.warp_exp_ops = h->opt.warp_exp_ops;
   eo.exp_call = h->opt.exp_call;
+  eo.tile = h->opt.tile;
   {
     const int N = h->m.n_species();
     const size_t lim = 160 * 1024;

@@ -87,3 +87,14 @@ def test_mechanisms_that_do_not_fit_the_tables_keep_the_fp64_kernel(mech_files, 
     assert B.Mechanism(handmech.write(mech, str(tmp_path), "order4.txt"), "device=0").stat("tile") == 0
     mech = handmech.abcd_mechanism(theta=3.0e6)
     assert B.Mechanism(handmech.write(mech, str(tmp_path), "theta.txt"), "device=0").stat("tile") == 0
+
+
+def test_the_tile_option(mech_files):
+    """tile=0 leaves a handle on the FP64 kernels alone; other values are refused."""
+    from paper_2503_24286_gb300 import binding as B
+    m = B.Mechanism(mech_files[0][0], "device=0;tile=0")
+    for key in ("tile", "jvp_tile", "vjp_tile", "jacobian_tile", "transport_tile"):
+        assert m.stat(key) == 0
+    assert B.Mechanism(mech_files[0][0], "device=0;tile=auto").stat("tile") == 1
+    with pytest.raises(B.PyroError):
+        B.Mechanism(mech_files[0][0], "device=0;tile=2")
