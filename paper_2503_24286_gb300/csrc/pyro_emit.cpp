@@ -89,9 +89,8 @@ __device__ __forceinline__ void pyro_load_tables(double* se, double* sl) {
 // temperature solve
 // ---------------------------------------------------------------------------
 
-
-void emit_tsolve(Src& s, const Mechanism& m, const std::vector<SpeciesCoef>& C, const EmitOptions& opt,
-                 std::map<std::string, double>& st) {
+// Tables of the mixture sums, and the sums over them in rolled loops (ts_collapse64, ts_collapse)
+void emit_tsolve_tables(Src& s, const Mechanism& m, const std::vector<SpeciesCoef>& C) {
   const int N = m.n_species(), NP = (N + 7) / 8 * 8;
   // Tables, one row per species (rows past the last one are zero).  FP32: the energy
   // coefficients d_0..d_5 of both ranges and the enthalpy's d_1 + 1/W.  FP64 and integer:
@@ -126,8 +125,6 @@ void emit_tsolve(Src& s, const Mechanism& m, const std::vector<SpeciesCoef>& C, 
         tx << (k || r || q ? "," : "") << (long long)(((unsigned long long)hi << 32) | (unsigned)lo) << "ll";
       }
   }
-  s << "#include \"pyro_fixed_math.cuh\"\n#define TS_ROWS " << NP << "\n#define TS_INV_R " << lit((double)(1.0L / R_GAS))
-    << "\n#define TS_INV_R_LO " << lit((double)(1.0L / R_GAS - (long double)(double)(1.0L / R_GAS))) << "\n";
   s << "__device__ const __align__(16) float ts_f[" << 16 * NP << "] = {" << tf.str() << "};\n";
   s << "__device__ const __align__(16) double ts_d[" << 16 * NP << "] = {" << td.str() << "};\n";
   s << "__device__ const __align__(16) long long ts_x[" << 16 * NP << "] = {" << tx.str() << "};\n";
@@ -185,7 +182,21 @@ __device__ __forceinline__ void ts_collapse(const double* __restrict__ Yp, i64 n
   for (int q = 0; q < 6; ++q)
     B[q] = pfx::scaled(s[q] + fold(q), 57 - __ldg(ts_s + (ENTH && q == 1 ? 6 : q)));
 }
+)";
+}
 
+// unrolled: the mixture sums as straight-line FP32 and FP64 code with every coefficient an
+// immediate (the Crank-Nicolson unit: its assembly kernel runs one warp per SM sub-partition in
+// 10 MB of straight-line code, and the rolled loops' table loads added latency to every Newton
+// iteration: 53 species, 2^18 states 178 ms a step, with this form 172 ms)
+void emit_tsolve(Src& s, const Mechanism& m, const std::vector<SpeciesCoef>& C, std::map<std::string, double>& st,
+                 bool unrolled) {
+  const int N = m.n_species();
+  if (!unrolled) s << "#include \"pyro_fixed_math.cuh\"\n#define TS_ROWS " << (N + 7) / 8 * 8 << "\n";
+  s << "#define TS_INV_R " << lit((double)(1.0L / R_GAS)) << "\n#define TS_INV_R_LO "
+    << lit((double)(1.0L / R_GAS - (long double)(double)(1.0L / R_GAS))) << "\n";
+  if (!unrolled) emit_tsolve_tables(s, m, C);
+  s << R"(
 // Newton inversion of e = sum_k Y_k e_k(T) (Sec. A.3.1, Eq. delta_temp), or with
 // ENTH of h = sum_k Y_k h_k(T) (the enthalpy variant: the linear coefficient of each
 // species polynomial gains 1/W_k, c_v becomes c_p); returns T, writes the iteration
@@ -194,7 +205,20 @@ template <bool ENTH>
 __device__ __forceinline__ double pyro_tsolve(const double* __restrict__ Yp, i64 n, double e,
     double T0, int max_iter, float tolf, int* iters) {
   float bl0=0.f,bl1=0.f,bl2=0.f,bl3=0.f,bl4=0.f,bl5=0.f,bh0=0.f,bh1=0.f,bh2=0.f,bh3=0.f,bh4=0.f,bh5=0.f;
-  float ysum = 0.f;
+)";
+  auto coef = [&](int k, int r, int q, bool enth) { return enth && q == 1 ? C[k].d[r][1] + 1.0 / m.species[k].W : C[k].d[r][q]; };
+  if (unrolled) {
+    for (int k = 0; k < N; ++k) {
+      s << "  { const float y = pdm::to_float_trunc(__ldg(Yp + (i64)" << k << " * n));";
+      for (int r = 0; r < 2; ++r)
+        for (int q = 0; q < 6; ++q) {
+          const std::string b = std::string(r ? "bh" : "bl") + std::to_string(q), c = litf(coef(k, r, q, false));
+          s << " " << b << " = fmaf(y, " << (q == 1 ? "(ENTH ? " + litf(coef(k, r, q, true)) + " : " + c + ")" : c) << ", " << b << ");";
+        }
+      s << " }\n";
+    }
+  } else {
+    s << R"(  float ysum = 0.f;
 #pragma unroll 1
   for (int k0 = 0; k0 < NSP; k0 += 8) {
     double yd[8];
@@ -213,7 +237,9 @@ __device__ __forceinline__ double pyro_tsolve(const double* __restrict__ Yp, i64
       bh2 = fmaf(y, c2.x, bh2); bh3 = fmaf(y, c2.y, bh3); bh4 = fmaf(y, c2.z, bh4); bh5 = fmaf(y, c2.w, bh5);
     }
   }
-  float Tf = pdm::to_float_trunc(T0);
+)";
+  }
+  s << R"(  float Tf = pdm::to_float_trunc(T0);
   const float eRf = pdm::to_float_trunc(e * TS_INV_R);
   int it32 = 0;
   if (opt_mixed) {
@@ -234,11 +260,25 @@ __device__ __forceinline__ double pyro_tsolve(const double* __restrict__ Yp, i64
   double T = opt_mixed ? pdm::to_double(Tf) : T0;
   bool hi = pdm::to_float_trunc(T) >= (float)TMID;
   double B[6];
-  const bool small = ysum > 0.25f && ysum < 2.f;          // sum |Y|; false for NaN
+)";
+  if (unrolled) {
+    s << "  auto collapse = [&] {\n    for (int q = 0; q < 6; ++q) B[q] = 0.0;\n";
+    for (int k = 0; k < N; ++k) {
+      s << "    { const double y = __ldg(Yp + (i64)" << k << " * n);";
+      for (int q = 0; q < 6; ++q) {
+        const double v[2] = {coef(k, 0, q, false), coef(k, 1, q, false)}, h[2] = {coef(k, 0, q, true), coef(k, 1, q, true)};
+        s << " B[" << q << "] = fma(y, " << (q == 1 ? "(ENTH ? " + sel(h) + " : " + sel(v) + ")" : sel(v)) << ", B[" << q << "]);";
+      }
+      s << " }\n";
+    }
+  } else {
+    s << R"(  const bool small = ysum > 0.25f && ysum < 2.f;          // sum |Y|; false for NaN
   auto collapse = [&] {
     if (small) ts_collapse<ENTH>(Yp, n, hi, B);
     else { double b[6]; ts_collapse64<ENTH>(Yp, n, hi, b); for (int q = 0; q < 6; ++q) B[q] = b[q]; }
-    // B_0 - e/R first: the formation energies cancel there, and the residual is rounded
+)";
+  }
+  s << R"(    // B_0 - e/R first: the formation energies cancel there, and the residual is rounded
     // at the size of c_v T only
     B[0] = fma(e, -TS_INV_R_LO, fma(e, -TS_INV_R, B[0]));
   };
@@ -2198,7 +2238,7 @@ EmitResult emit_module(const Mechanism& m, const EmitOptions& opt) {
   for (auto& sp : m.species) C.push_back(species_coef(sp));
   emit_prelude(s, m, opt);
   s << "#define opt_mixed " << (opt.mixed_newton ? 1 : 0) << "\n";
-  emit_tsolve(s, m, C, opt, out.stats);
+  emit_tsolve(s, m, C, out.stats, false);
 
   // ---- diagnostic math kernel -------------------------------------------------
   s << R"(
@@ -2419,7 +2459,7 @@ extern "C" __global__ void __launch_bounds__(BLK) pyro_temperature_h(i64 n, cons
     d << "#define CN_G " << kCnGroup << "\n#define CN_W " << cnw << "\n#define opt_mixed "
       << (opt.mixed_newton ? 1 : 0) << "\n";
     std::map<std::string, double> dummy;
-    emit_tsolve(d, m, C, opt, dummy);
+    emit_tsolve(d, m, C, dummy, true);
     emit_jacobian_kernel(d, m, C, opt.deriv_block, &ns2, JacMode::CN, opt.dgstore, opt.jac_table);
     emit_cn_kernels(d, m, C);
     if (opt.cn_residual) emit_cn_residual_kernel(d, m, C, opt.acc_mem);
