@@ -154,7 +154,7 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
   double t_lo = 0.0;
   for (double lo : {200.0, 225.0, 250.0, 275.0, 300.0, 350.0, 400.0}) if (fits_from(lo)) { t_lo = lo; break; }
   if (t_lo == 0.0) { out.why = "rate constants out of range above 400 K"; return out; }
-  const ld T_V = 0.9999L * (ld)t_lo;
+  const ld T_V = (double)(0.9999L * (ld)t_lo);   // a double: the kernel divides by T what the coefficients hold
 
   // ---- species tables ----------------------------------------------------------
   Fix fx;
@@ -426,6 +426,7 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
   std::vector<int> chunk_of(groups.size());
   for (int ch = 0; ch < chunks; ++ch) for (int g : in_chunk[ch]) chunk_of[g] = ch;
   std::vector<int> wl, wo, we, wc;
+  int hb_max = 0;
   for (int ch = 0; ch < chunks; ++ch)
     for (int w = 0; w < warps; ++w)
       for (int i = 0; i < kpo; ++i) {
@@ -444,8 +445,9 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
           ends[pass + 1] = (int)we.size();
         }
         wl.insert(wl.end(), ends, ends + 4);
-        int hb = 0;
-        while ((1 << hb) < sum) ++hb;
+        int hb = 3;                              // headroom bits of the sum, more than its terms take
+        while ((1 << hb) <= sum) ++hb;
+        hb_max = std::max(hb_max, hb);
         wo.push_back(i < (int)owned[w].size() ? owned[w][i] : -1);
         wo.push_back(hb + 256 * no);
       }
@@ -553,7 +555,7 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
   std::ostringstream o;
   o << "// Tile kernel of mechanism '" << m.name << "': " << N << " species, " << NR << " reactions.\n"
     << "#define NSP " << N << "\n#define NW " << warps << "\n#define TILE_MINB " << minb << "\n#define KPW " << kpw
-    << "\n#define KPO " << kpo << "\n#define NCH " << chunks << "\n#define NCLS " << ncls << "\n#define TILE_ROWS "
+    << "\n#define TILE_ROUND " << (hb_max > 7 ? 1 : 0) << "\n#define KPO " << kpo << "\n#define NCH " << chunks << "\n#define NCLS " << ncls << "\n#define TILE_ROWS "
     << tile_rows << "\n#define TMID " << lit(tmid) << "\n#define TILE_OPEN " << kTileOpen << "\n#define T_LO " << lit(t_lo) << "\n#define T_HI "
     << lit((double)T_HI) << "\n#define T_V " << lit((double)T_V) << "\n#define T_T " << lit((double)T_T)
     << "\n#define T_INV_R " << lit((double)(1.0L / R_GAS)) << "\n#define T_INV_R_LO "

@@ -12,7 +12,7 @@
 //      K_j(T) - sum nu' lambda + sum nu' alpha  and  ... + sum nu'' alpha,
 //      two exponentials and their difference, the rate of progress, in shared memory
 //      as one 64-bit word: 52 bits of signed integer and 12 of exponent (not
-//      normalised: its error is 2^-50 of the larger of the two rates);
+//      normalised: its error is 2^-51 of the larger of the two rates);
 //   3  per species the sum of its reactions' rates, aligned to the largest exponent
 //      met so far, normalised once into the output.
 // Bound: the integer pipes (53 species / 325 reactions: 130 k warp instructions a tile,
@@ -41,6 +41,17 @@ using pfx::Pair;
 typedef pfx::i64 i64;
 typedef pfx::u64 u64;
 
+// A rate is a 64-bit word r: read as an integer it is m 2^(e - 62 - RATE_E) with
+// e = r & RATE_M, |m| < 2^63.  The exponent's bits are the last bits of the integer: they lie
+// below its resolution and, near RATE_E/(RATE_M + 1) = 1/2 of one unit, are on average what
+// truncation took away.  12 exponent bits, or 11 (RATE_E 1023) for words made of doubles.
+#ifndef RATE_E
+#define RATE_E 2048
+#define RATE_M 4095
+#else
+#define RATE_M 2047
+#endif
+
 #ifndef TILE_DERIV
 struct TileScalars {
   double T[32], ysum[32];
@@ -51,13 +62,6 @@ struct TileScalars {
   int neg;                       // the tile has negative mass fractions or densities
 };
 
-// A rate is a 64-bit word r: read as an integer it is m 2^(e - 61 - RATE_E) with
-// e = r & 4095.  The exponent's bits are the last bits of the integer: they lie below
-// its resolution and, near RATE_E/4096 of one unit, are on average what truncation
-// took away.
-#ifndef RATE_E
-#define RATE_E 2048
-#endif
 struct TileSmem {
   u64* exp2;
   i64 *lam, *alp;   // [NSP + 1][32]: the species and a unit factor; alp first holds Y
@@ -148,23 +152,42 @@ __device__ __forceinline__ i64 tile_rate(i64 xf, i64 xr, const u64* tab) {
     const i64 sg = SGN ? -(xr & 1ll) : 0ll;
     const int ng = (int)(xr >> pfx::LG_F);
     e = max(e, ng);
-    // one's complement negation: off by one in 2^61
-    m = ((i64)tile_shr(f, e + 2 - nf) ^ sf) - ((i64)tile_shr(g, e + 2 - ng) ^ sg);
+    if (SGN) e += (int)(xf ^ xr) & 1;           // unlike signs: the terms add up to twice the larger
+    // one's complement negation: off by one in 2^62
+    m = ((i64)tile_shr(f, e + 1 - nf) ^ sf) - ((i64)tile_shr(g, e + 1 - ng) ^ sg);
   } else {
-    m = (i64)tile_shr(f, e + 2 - nf) ^ sf;
+    m = (i64)tile_shr(f, e + 1 - nf) ^ sf;
   }
-  return (m & ~4095ll) | (i64)(e + RATE_E);
+  return (m & ~(i64)RATE_M) | (i64)(e + RATE_E);
 }
 
 // the rate of a sum of two
 __device__ __forceinline__ i64 tile_add(i64 a, i64 b) {
-  const int ea = (int)a & 4095, eb = (int)b & 4095, e = max(ea, eb) + 1;
-  return ((tile_sar(a, e - ea) + tile_sar(b, e - eb)) & ~4095ll) | (i64)e;
+  const int ea = (int)a & RATE_M, eb = (int)b & RATE_M, e = max(ea, eb) + 1;
+  return ((tile_sar(a, e - ea) + tile_sar(b, e - eb)) & ~(i64)RATE_M) | (i64)e;
 }
 
 // K(T) = c + beta u + tau v of a reaction, lowest bit clear
 __device__ __forceinline__ i64 tile_K(i64 c, i64 beta, i64 tau, Pair u, Pair v) {
   return pfx::mul_add(as_pair(tau), v, pfx::mul_add(as_pair(beta), u, c)) & ~1ll;
+}
+
+// The temperature's factors of a state, T in (T_LO, T_HI): u = log2(T)/16, v = T_V/T and
+// t = T/T_T as fracs, and its lg.  The exponents of cold states are a few hundred, so an ulp of v
+// is an error of 1e-14 to 5e-14 in every rate: quotients get the remainder of the FP64
+// value in units of 2^-63, and u keeps the bits of the logarithm that lg has no room for.
+__device__ __forceinline__ i64 tile_quotient(double a, double b, double r) {     // a/b, r = 1/b
+  const double q = a * r;
+  return pfx::frac_of(q) + (i64)__double2int_rn(fma(-b, q, a) * r * 9223372036854775808.0);
+}
+__device__ __forceinline__ void tile_T(double T, Pair& u, Pair& v, Pair& t, i64& lgT) {
+  const u64 b = pfx::dbits(T);
+  const i64 e = (i64)(b >> 52) - 1023;
+  const i64 l = pfx::log2_mant((b & 0xfffffffffffffull) | 0x10000000000000ull, t_log2);      // f = 62
+  lgT = (e << pfx::LG_F) + (((l + 0x1000ll) >> 13) << 1);
+  u = pfx::split((e << 59) + ((l + 4) >> 3));
+  v = pfx::split(tile_quotient(T_V, T, pdm::rcp(T)));
+  t = pfx::split(tile_quotient(T, T_T, 1.0 / T_T));
 }
 
 #ifndef TILE_DERIV
@@ -468,7 +491,11 @@ __device__ __forceinline__ void tile_other(const TileSmem& s, int i0, int i1, in
 #endif  // TILE_DERIV
 
 // species sums of a chunk: per owned species the rows with nu = +1, with -1 (both padded to
-// multiples of 4 with the zero row) and with other nu; sink(species, sum)
+// multiples of 4 with the zero row) and with other nu; sink(species, sum).  Every term is cut
+// at the headroom hb of its list of n terms, a bias of at most n 2^(hb - 63) of the largest
+// term: 2^-51 for 55 terms (160 species' longest list), but 2^-47 from 250 terms.  Units with
+// such lists (TILE_ROUND: hb above 7) align four terms with 3 bits of headroom and round
+// their sum to hb, 5 instructions more for four terms (3 % of the kernel's time).
 struct TilePlus { static constexpr bool minus = false; };
 struct TileMinus { static constexpr bool minus = true; };
 template <class F>
@@ -487,7 +514,14 @@ __device__ __forceinline__ void tile_sums(const i64* rows, int ch, int w, F sink
     if (o.x < 0) break;
     qn = __ldg((const int4*)t_wl + (ch * NW + w) * KPO + i + 1);
     on = __ldg((const int2*)t_wo + (ch * NW + w) * KPO + i + 1);
-    const int hb = o.y & 0xff;
+#if TILE_ROUND
+    const int hb = 3, up = (o.y & 0xff) - 3;    // headroom of four terms, and the rest of the list's
+    const i64 half = (1ll << up) >> 1;
+    auto fold = [&](i64 b) { return tile_sar(b + half, up); };
+#else
+    const int hb = o.y & 0xff, up = 0;
+    auto fold = [&](i64 b) { return b; };
+#endif
     i64 a = 0;
     int e = 0;
     auto quad = [&](int j, auto sign) {
@@ -495,23 +529,23 @@ __device__ __forceinline__ void tile_sums(const i64* rows, int ch, int w, F sink
       rn = __ldg((const int4*)(t_we + j + 4));
       const i64 v0 = *(const i64*)(R + r.x), v1 = *(const i64*)(R + r.y), v2 = *(const i64*)(R + r.z),
                 v3 = *(const i64*)(R + r.w);
-      const int e0 = (int)v0 & 4095, e1 = (int)v1 & 4095, e2 = (int)v2 & 4095, e3 = (int)v3 & 4095;
+      const int e0 = (int)v0 & RATE_M, e1 = (int)v1 & RATE_M, e2 = (int)v2 & RATE_M, e3 = (int)v3 & RATE_M;
       const int en = max(max(e, max(e0, e1)), max(e2, e3)), t = en + hb;
       a = tile_sar(a, en - e);
       e = en;
-      const i64 b = (tile_sar(v0, t - e0) + tile_sar(v1, t - e1)) + (tile_sar(v2, t - e2) + tile_sar(v3, t - e3));
+      const i64 b = fold((tile_sar(v0, t - e0) + tile_sar(v1, t - e1)) + (tile_sar(v2, t - e2) + tile_sar(v3, t - e3)));
       if (decltype(sign)::minus) a -= b; else a += b;
     };
     _Pragma("unroll 2") for (int j = q.x; j < q.y; j += 4) quad(j, TilePlus());
     _Pragma("unroll 2") for (int j = q.y; j < q.z; j += 4) quad(j, TileMinus());
     for (int j = q.z; j < q.z + (o.y >> 8); ++j) {
       const i64 x = *(const i64*)(R + __ldg(t_we + j));
-      const int e0 = (int)x & 4095, en = max(e, e0);
-      a = tile_sar(a, en - e) + (i64)__ldg(t_wc + j) * tile_sar(x, en + hb - e0);
+      const int e0 = (int)x & RATE_M, en = max(e, e0);
+      a = tile_sar(a, en - e) + fold((i64)__ldg(t_wc + j) * tile_sar(x, en + hb - e0));
       e = en;
     }
     if (q.w > q.z) rn = __ldg((const int4*)(t_we + q.w));
-    sink(o.x, tile_to_double(a, e + hb - RATE_E, 61));
+    sink(o.x, tile_to_double(a, e + hb + up - RATE_E, 62));
   }
 }
 
@@ -578,13 +612,9 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         const unsigned re = ((unsigned)__double2hiint(rho) >> 20) & 0x7ff;
         const bool in = T > T_LO && T < T_HI && re >= 1023 - 60 && re <= 1023 + 20;
         const double Ts = in ? T : 1000.0;
-        const i64 lgT = pfx::log2_of(Ts, t_log2);
         s.sc->T[lane] = Ts;
-        s.sc->lgT[lane] = lgT;
+        tile_T(Ts, s.sc->u[lane], s.sc->v[lane], s.sc->t[lane], s.sc->lgT[lane]);
         s.sc->lgrho[lane] = pfx::log2_of(in ? fabs(rho) : 1.0, t_log2) | (i64)((u64)__double_as_longlong(rho) >> 63);
-        s.sc->u[lane] = pfx::split(lgT << 9);
-        s.sc->v[lane] = pfx::split(pfx::frac_of(T_V * pdm::rcp(Ts)));
-        s.sc->t[lane] = pfx::split(pfx::frac_of(Ts * (1.0 / T_T)));
         s.sc->bad[lane] = in ? 0 : 1;
         if (lane == 0) s.sc->neg = 0;
         __syncwarp();

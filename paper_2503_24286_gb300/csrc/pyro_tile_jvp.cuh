@@ -29,11 +29,12 @@ struct JvpSmem {
   JvpScalars* sc;
 };
 
-// a double as a rate word (0 below the normal range); e = 2047 marks overflow or NaN
+// a double as a rate word (0 below the normal range); e = 2047 marks overflow or NaN.  Its 53
+// bits fill the word but for one: the last one is rounded off by the exponent's bits (RATE_M).
 __device__ __forceinline__ i64 jvp_word(double x) {
   const int h = __double2hiint(x), e = (h >> 20) & 0x7ff;
-  const u64 m = ((u64)__double_as_longlong(x) & 0xfffffffffffffull) << 9 | 0x2000000000000000ull;   // 1.f 2^61
-  const i64 w = (((i64)m ^ (i64)(h >> 31)) & ~4095ll) | (i64)e;
+  const u64 m = ((u64)__double_as_longlong(x) & 0xfffffffffffffull) << 10 | 0x4000000000000000ull;   // 1.f 2^62
+  const i64 w = (((i64)m ^ (i64)(h >> 31)) & ~(i64)RATE_M) | (i64)e;
   return e == 0 ? 0ll : w;
 }
 __device__ __forceinline__ bool jvp_finite(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) != 0x7ff; }
@@ -262,7 +263,6 @@ pyro_jvp_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict_
       const bool in = T > T_LO && T < T_HI && re >= 1023 - 60 && re <= 1023 + 20 && rho > 0.0 && jvp_finite(drho) &&
                       jvp_finite(dT);
       const double Ts = in ? T : 1000.0, rs = in ? rho : 1.0;
-      const i64 lgT = pfx::log2_of(Ts, t_log2);
       JvpScalars& z = *s.sc;
       z.T[lane] = Ts;
       z.invT[lane] = pdm::rcp(Ts);
@@ -270,10 +270,7 @@ pyro_jvp_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict_
       z.drho[lane] = in ? drho : 0.0;
       z.drr[lane] = in ? drho * pdm::rcp(rs) : 0.0;
       z.dT[lane] = in ? dT : 0.0;
-      z.lgT[lane] = lgT;
-      z.u[lane] = pfx::split(lgT << 9);
-      z.v[lane] = pfx::split(pfx::frac_of(T_V * pdm::rcp(Ts)));
-      z.t[lane] = pfx::split(pfx::frac_of(Ts * (1.0 / T_T)));
+      tile_T(Ts, z.u[lane], z.v[lane], z.t[lane], z.lgT[lane]);
       z.bad[lane] = in ? 0 : 1;
     }
     __syncthreads();

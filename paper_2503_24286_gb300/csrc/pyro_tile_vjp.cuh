@@ -236,15 +236,11 @@ pyro_vjp_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict_
       const unsigned re = ((unsigned)__double2hiint(rho) >> 20) & 0x7ff;
       const bool in = T > T_LO && T < T_HI && re >= 1023 - 60 && re <= 1023 + 20 && rho > 0.0;
       const double Ts = in ? T : 1000.0;
-      const i64 lgT = pfx::log2_of(Ts, t_log2);
       VjpScalars& z = *s.sc;
       z.T[lane] = Ts;
       z.invT[lane] = pdm::rcp(Ts);
       z.rho[lane] = in ? rho : 1.0;
-      z.lgT[lane] = lgT;
-      z.u[lane] = pfx::split(lgT << 9);
-      z.v[lane] = pfx::split(pfx::frac_of(T_V * pdm::rcp(Ts)));
-      z.t[lane] = pfx::split(pfx::frac_of(Ts * (1.0 / T_T)));
+      tile_T(Ts, z.u[lane], z.v[lane], z.t[lane], z.lgT[lane]);
       z.bad[lane] = in ? 0 : 1;
     }
     __syncthreads();
