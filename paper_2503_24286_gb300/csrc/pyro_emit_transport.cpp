@@ -70,28 +70,31 @@ TransportTile emit_transport_tile(const Mechanism& m) {
   if (!(pmin > 0) || !std::isfinite((double)pmin)) return out;
   const int sv = ilogbl(pmin), sw = 2 * sv;      // x/P 2^sv, x/P^2 2^sw below one
 
-  // ---- Wilke's matrices, each scaled by a power of two: the largest coefficient below 2^hb,
-  // so that sums of products of halves stay below 2^63 (as in the mixture collapse)
+  // ---- Wilke's matrices, each row scaled by a power of two: the largest coefficient below 2^hb,
+  // so that sums of products of halves stay below 2^63 (as in the mixture collapse).  By row:
+  // the rows of heavy species are 10^-2 of the largest, and one scale for a matrix left
+  // mu with a mean error of 2.0e-15 (53 species; FP64 sums 3.4e-16)
   auto W = [&](int k) { return (ld)m.species[k].W; };
   auto wil = [&](int k, int j, int q) {
     const ld c = 1.0L / sqrtl(8.0L * (1.0L + W(k) / W(j))), g = powl(W(j) / W(k), 0.25L);
     return q == 0 ? c : q == 1 ? 2 * c * g : c * g * g;
   };
-  int hb = 57, f[3];
+  int hb = 57;
   while ((1 << (62 - hb)) < N) --hb;
+  std::vector<i64> wk((size_t)N * N * 4, 0), we;   // and per row the f of the three sums
+  for (int k = 0; k < N; ++k) we.insert(we.end(), 4, 0);
   for (int q = 0; q < 3; ++q) {
     ld mx = 0, mn = 1e300L;
-    for (int k = 0; k < N; ++k)
-      for (int j = 0; j < N; ++j) { mx = std::max(mx, wil(k, j, q)); mn = std::min(mn, wil(k, j, q)); }
-    if (mn < mx * 1e-4L) return out;             // few bits left for the smallest: the FP64 kernel
-    f[q] = hb - 1 - ilogbl(mx);
-  }
-  std::vector<i64> wk;
-  for (int k = 0; k < N; ++k)
-    for (int j = 0; j < N; ++j) {
-      for (int q = 0; q < 3; ++q) wk.push_back(halves(llroundl(ldexpl(wil(k, j, q), f[q]))));
-      wk.push_back(0);
+    for (int k = 0; k < N; ++k) {
+      ld row = 0;
+      for (int j = 0; j < N; ++j) { row = std::max(row, wil(k, j, q)); mn = std::min(mn, wil(k, j, q)); }
+      mx = std::max(mx, row);
+      const int f = hb - 1 - ilogbl(row);
+      for (int j = 0; j < N; ++j) wk[((size_t)k * N + j) * 4 + q] = halves(llroundl(ldexpl(wil(k, j, q), f)));
+      we[(size_t)k * 4 + q] = f + 61 + (q == 0 ? 0 : q == 1 ? sv : sw);     // the row's scale, that of x, x/P or x/P^2
     }
+    if (mn < mx * 1e-4L) return out;             // few bits left for the smallest: the FP64 kernel
+  }
 
   // ---- pairs in rounds of a tournament (circle method: player 0 stays) ------------------
   const int M = N + (N & 1), rounds = M - 1, ppr = M / 2;
@@ -143,9 +146,8 @@ TransportTile emit_transport_tile(const Mechanism& m) {
   o << "// Transport tile kernel of mechanism '" << m.name << "': " << N << " species.\n#define NSP " << N << "\n#define NW "
     << nw << "\n#define KPW " << (N + nw - 1) / nw << "\n#define TT_MINB " << minb << "\n#define TT_ROUNDS " << rounds
     << "\n#define TT_PER_WARP " << per << "\n#define TT_PAIRS_W " << rounds * per << "\n#define TT_LO " << lit(t_lo)
-    << "\n#define TT_HI " << lit(t_hi) << "\n#define TT_LGC " << (i64)llroundl(log2l(1000.0L) * 562949953421312.0L) * 2
-    << "ll\n#define TT_SV " << lit((double)ldexpl(1, sv)) << "\n#define TT_SW " << lit((double)ldexpl(1, sw)) << "\n#define TT_FA "
-    << f[0] + 61 << "\n#define TT_FB " << f[1] + 61 + sv << "\n#define TT_FE " << f[2] + 61 + sw << "\n#define TILE_OPEN " << kTileOpen << "\n#include \"pyro_fixed_math.cuh\"\n";
+    << "\n#define TT_HI " << lit(t_hi) << "\n#define TT_LGC " << (i64)llroundl(log2l(1000.0L) * 576460752303423488.0L)
+    << "ll\n#define TT_SV " << lit((double)ldexpl(1, sv)) << "\n#define TT_SW " << lit((double)ldexpl(1, sw)) << "\n#define TILE_OPEN " << kTileOpen << "\n#include \"pyro_fixed_math.cuh\"\n";
   auto d = [](double v) { return lit(v); };
   auto l = [](i64 v) { return std::to_string(v) + "ll"; };
   std::vector<double> iw;
@@ -153,6 +155,7 @@ TransportTile emit_transport_tile(const Mechanism& m) {
   array(o, "double", "tt_iw", iw, d);
   array(o, "double", "tt_fit", fit, d);
   array(o, "long long", "tt_wilke", wk, l);
+  array(o, "int", "tt_wf", we, [](i64 v) { return std::to_string(v); });
   array(o, "long long", "tt_pair_tab", pt, l);
   std::vector<int> idx(256);
   for (int j = 0; j < 256; ++j) idx[j] = j;

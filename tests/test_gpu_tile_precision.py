@@ -68,3 +68,15 @@ def test_rates_of_long_lists(mech_files, tmp_path):
     path = str(tmp_path / "long.txt")
     synth.write_mechanism(m, path)
     _rates(path, 0, 113)
+
+
+@pytest.mark.parametrize("idx", [0, 1])
+def test_transport(mech_files, idx):
+    tile, fp64, orc = _handles(mech_files[0][idx])
+    assert tile.stat("transport_tile") == 1 and fp64.stat("transport_tile") == 0
+    st = synth.config_states(idx, n=100, offset_seed=114)
+    ref = orc.transport(st.T, st.Y, long_double=True)
+    out = [[x.cpu().numpy() for x in m.transport(_t(st.T), _t(st.Y))] for m in (tile, fp64)]
+    for k in range(3):
+        a, b = _errors(out[0][k], ref[k]), _errors(out[1][k], ref[k])
+        assert a[0] <= b[0] and a[1] <= b[1], (k, a, b)
