@@ -109,7 +109,7 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
 
   // ---- temperature range: the lowest T_LO from which every rate's exponent at unit
   // concentrations is below 1190 (a product with one zero, 2^-2400, then vanishes) and
-  // above -8150 + 2460 per factor (a product of zeros stays in range: |lg| < 8192)
+  // above -8150 + 2460 per factor (a product of zeros stays in range: |lg| < 8192; with [M] 1030 higher)
   auto folded = [&](const Reaction& r, double A, double b, double theta) {
     Arr a{log2l((ld)A), (ld)b, (ld)theta};
     for (auto& p : r.reactants) a.c -= p.second * log2l((ld)m.species[p.first].W);
@@ -145,14 +145,16 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
           const ld K = arr_at(a, T) + g;         // log2 of the rate constant
           const ld X = arr_at(a, T) - f + r;     // reverse exponent at unit products
           const ld nf = (ld)side_factors(m.reactions[j].reactants).size(), np = (ld)side_factors(m.reactions[j].products).size();
-          if (!(K > -8150 + 2460 * nf && K < 1190 && X > -8150 + 2460 * np && X < 1190)) return false;
+          const int cls = classes(m.reactions[j]);
+          const ld M = cls > 0 && cls < 5 ? 1030 : 0;           // [M] from the smallest normal number
+          if (!(K > -8150 + 2460 * nf + M && K < 1190 && X > -8150 + 2460 * np + M && X < 1190)) return false;
         }
       }
     }
     return true;
   };
-  double t_lo = 0.0;
-  for (double lo : {200.0, 225.0, 250.0, 275.0, 300.0, 350.0, 400.0}) if (fits_from(lo)) { t_lo = lo; break; }
+  double t_lo = 0.0;                             // (in steps of 10 K: 160 species' lies at 290 K, below room temperature)
+  for (double lo = 200.0; lo <= 400.0 && t_lo == 0.0; lo += 10.0) if (fits_from(lo)) t_lo = lo;
   if (t_lo == 0.0) { out.why = "rate constants out of range above 400 K"; return out; }
   const ld T_V = (double)(0.9999L * (ld)t_lo);   // a double: the kernel divides by T what the coefficients hold
 

@@ -30,8 +30,8 @@
 // The FP64 pipe, which runs beside the integer work, keeps the Newton steps, the
 // third-body concentrations and the blending factors of falloff reactions.
 //
-// States outside the tables' range (temperature outside (T_LO, T_HI), NaN,
-// infinite or subnormal mass fractions or ones from 2, densities beyond 2^-60..2^20, a
+// States outside the tables' range (temperature outside (T_LO, T_HI), NaN or
+// infinite mass fractions or ones from 2, densities beyond 2^-60..2^20, a
 // falloff or PLOG reaction with [M] <= 0) get TILE_OPEN in their first output; the caller then launches the FP64
 // kernel, which evaluates the states so marked.
 #include "pyro_device_math.cuh"
@@ -60,6 +60,7 @@ struct TileScalars {
   float Tf[32];
   int bad[32];
   int neg;                       // the tile has negative mass fractions or densities
+  int none;                      // no state of the tile is inside the tables
 };
 
 struct TileSmem {
@@ -575,6 +576,12 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
     const i64 pc = p < n ? p : n - 1;
     const double* Yp = g_Y + pc;
     const double rho = __ldg(g_rho + pc);
+    // a tile without any state in the tables (a cold block): no work beside the FP64 kernel's
+    const double Tin = __ldg(g_Tin + pc);
+    if (!energy_mode && !__any_sync(0xffffffffu, Tin > T_LO && Tin < T_HI)) {
+      if (w == 0 && p < n && rank == 0) g_omega[p] = __longlong_as_double(TILE_OPEN);
+      continue;
+    }
     {
       {
         double y[KPW];
@@ -598,9 +605,9 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
       double T;
       bool ok = true;
       if (energy_mode) {
-        tile_energy(s, Yp, n, __ldg(g_Tin + pc), T_guess, max_iter, (float)tol, w, lane, T, ok);
+        tile_energy(s, Yp, n, Tin, T_guess, max_iter, (float)tol, w, lane, T, ok);
       } else {
-        T = __ldg(g_Tin + pc);
+        T = Tin;
         __syncthreads();
       }
       if (w == 0) {
@@ -616,7 +623,8 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         tile_T(Ts, s.sc->u[lane], s.sc->v[lane], s.sc->t[lane], s.sc->lgT[lane]);
         s.sc->lgrho[lane] = pfx::log2_of(in ? fabs(rho) : 1.0, t_log2) | (i64)((u64)__double_as_longlong(rho) >> 63);
         s.sc->bad[lane] = in ? 0 : 1;
-        if (lane == 0) s.sc->neg = 0;
+        const bool none = !__any_sync(0xffffffffu, in);
+        if (lane == 0) { s.sc->neg = 0; s.sc->none = none; }
         __syncwarp();
         if (__double_as_longlong(rho) < 0) s.sc->neg = 1;
       }
@@ -627,6 +635,11 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         s.sc->ysum[lane] = a;
       }
       __syncthreads();
+      if (s.sc->none) {                          // the same, its temperatures solved
+        if (w == 0 && p < n && rank == 0) g_omega[p] = __longlong_as_double(TILE_OPEN);
+        __syncthreads();
+        continue;
+      }
       // species: lambda_k and alpha_k
       const Pair u = s.sc->u[lane], v = s.sc->v[lane], t = s.sc->t[lane];
       const i64 lgrho = s.sc->lgrho[lane];
@@ -641,10 +654,16 @@ pyro_omega_tile(i64 n, const double* __restrict__ g_rho, const double* __restric
         q = pfx::horner(q, t, c2.x);
         q = tile_K(q, c2.y, c3.x, u, v);
         const u64 yb = (u64)s.alp[k * 32 + lane];
-        const int ye = (int)(yb >> 52) & 0x7ff;
+        int ye = (int)(yb >> 52) & 0x7ff;
         const bool zero = (yb << 1) == 0ull;
-        bad |= (ye == 0 && !zero) || ye > 1023;
-        i64 ly = pfx::log2_of(__longlong_as_double((i64)(yb & 0x7fffffffffffffffull)), t_log2);
+        bad |= ye > 1023;
+        u64 ym = (yb & 0xfffffffffffffull) | 0x10000000000000ull;
+        if (ye == 0) {                           // subnormal
+          const int sh = pfx::clz64(ym ^ 0x10000000000000ull) - 11;
+          ym = (ym ^ 0x10000000000000ull) << sh;
+          ye = 1 - sh;
+        }
+        i64 ly = ((i64)(ye - 1023) << pfx::LG_F) + (((pfx::log2_mant(ym, t_log2) + 0x1000ll) >> 13) << 1);
         ly = zero ? pfx::LG_ZERO : (ly | (i64)(yb >> 63));
         if ((i64)yb < 0 && !zero) s.sc->neg = 1;
         s.lam[k * 32 + lane] = q;

@@ -112,7 +112,8 @@ __device__ __forceinline__ void jvp_other(const JvpSmem& s, int i0, int i1, int 
       dmS = fma(__ldg(dYp + c.x * n), ax_d(c.y), dmS);
     }
     const double M = rho * mS, dM = fma(z.drho[lane], mS, rho * dmS);
-    if (!tile_normal_pos(M) || !jvp_finite(dM)) s.sc->bad[lane] = 1;
+    // (a third body's [M] is a factor: zero or negative as it may be)
+    if (!(kind == TK_THREEBODY ? jvp_finite(M) : tile_normal_pos(M)) || !jvp_finite(dM)) s.sc->bad[lane] = 1;
     const i64 lgM = pfx::log2_of(M, t_log2);
     i64 X;
     double tau, sM = 0.0;          // d ln kk/dT, d ln kk/d ln M
@@ -234,6 +235,12 @@ pyro_jvp_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict_
 #pragma unroll 1
   for (i64 tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const i64 p = tile * 32 + lane, pc = p < n ? p : n - 1;
+    // a tile without any state in the tables (a cold block): no work beside the FP64 kernel's
+    const double T_in = __ldg(g_T + pc);
+    if (!__any_sync(0xffffffffu, T_in > T_LO && T_in < T_HI)) {
+      if (w == 0 && p < n) g_dw[p] = __longlong_as_double(TILE_OPEN);
+      continue;
+    }
     const double *Yp = g_Y + pc, *dYp = g_dY + pc;
     {
       double y[KPW], dy[KPW], ys = 0.0, dys = 0.0;
@@ -258,7 +265,7 @@ pyro_jvp_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict_
       part[(w * 2 + 1) * 32 + lane] = dys;
     }
     if (w == 0) {
-      const double T = __ldg(g_T + pc), rho = __ldg(g_rho + pc), drho = __ldg(g_drho + pc), dT = __ldg(g_dT + pc);
+      const double T = T_in, rho = __ldg(g_rho + pc), drho = __ldg(g_drho + pc), dT = __ldg(g_dT + pc);
       const unsigned re = ((unsigned)__double2hiint(rho) >> 20) & 0x7ff;
       const bool in = T > T_LO && T < T_HI && re >= 1023 - 60 && re <= 1023 + 20 && rho > 0.0 && jvp_finite(drho) &&
                       jvp_finite(dT);

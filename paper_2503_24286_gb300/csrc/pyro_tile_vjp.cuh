@@ -86,7 +86,8 @@ __device__ __forceinline__ void vjp_other(const VjpSmem& s, int i0, int i1, int 
     const i64* ax = t_ax + __ldg(r + 5);
     const double* fx = t_fx + __ldg(r + 5);
     const double mS = tile_mS(ax + 16, (int)__ldg(ax), z.ysum[lane], Yp, n), M = rho * mS;
-    if (!tile_normal_pos(M)) s.sc->bad[lane] = 1;
+    // (a third body's [M] is a factor: zero or negative as it may be)
+    if (!(kind == TK_THREEBODY ? vjp_finite(M) : tile_normal_pos(M))) s.sc->bad[lane] = 1;
     const i64 lgM = pfx::log2_of(M, t_log2);
     i64 X;
     double tau, sM = 0.0;          // d ln kk/dT, d ln kk/d ln M
@@ -209,6 +210,12 @@ pyro_vjp_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict_
 #pragma unroll 1
   for (i64 tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const i64 p = tile * 32 + lane, pc = p < n ? p : n - 1;
+    // a tile without any state in the tables (a cold block): no work beside the FP64 kernel's
+    const double T_in = __ldg(g_T + pc);
+    if (!__any_sync(0xffffffffu, T_in > T_LO && T_in < T_HI)) {
+      if (w == 0 && p < n) g_rhob[p] = __longlong_as_double(TILE_OPEN);
+      continue;
+    }
     const double* Yp = g_Y + pc;
     bool bad = false;
     {
@@ -232,7 +239,7 @@ pyro_vjp_tile(i64 n, const double* __restrict__ g_rho, const double* __restrict_
       part[w * 32 + lane] = ys;
     }
     if (w == 0) {
-      const double T = __ldg(g_T + pc), rho = __ldg(g_rho + pc);
+      const double T = T_in, rho = __ldg(g_rho + pc);
       const unsigned re = ((unsigned)__double2hiint(rho) >> 20) & 0x7ff;
       const bool in = T > T_LO && T < T_HI && re >= 1023 - 60 && re <= 1023 + 20 && rho > 0.0;
       const double Ts = in ? T : 1000.0;

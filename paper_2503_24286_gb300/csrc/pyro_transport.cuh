@@ -102,6 +102,12 @@ pyro_transport_tile(i64 n, const double* __restrict__ g_T, const double* __restr
 #pragma unroll 1
   for (i64 tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const i64 p = tile * 32 + lane, pc = p < n ? p : n - 1;
+    // a tile without any state in the tables (a cold block): no work beside the FP64 kernel's
+    const double T = __ldg(g_T + pc);
+    if (!__any_sync(0xffffffffu, T > TT_LO && T < TT_HI)) {
+      if (w == 0 && p < n) (g_mu ? g_mu : g_kappa ? g_kappa : g_Dm)[p] = __longlong_as_double(TILE_OPEN);
+      continue;
+    }
     const double* Yp = g_Y + pc;
     {
       double y[KPW];
@@ -118,7 +124,6 @@ pyro_transport_tile(i64 n, const double* __restrict__ g_T, const double* __restr
       sh.ys[w * 32 + lane] = ys;
     }
     if (w == 0) {
-      const double T = __ldg(g_T + pc);
       const bool in = T > TT_LO && T < TT_HI;
       const double Ts = in ? T : 1000.0;
       const u64 b = pfx::dbits(Ts);
