@@ -315,6 +315,18 @@ struct ArgSpec {
   bool in, out;
 };
 
+// Whether an output of a call (but for number `except`) overlaps one of its inputs (d: the device
+// pointers, n states).  The FP64 kernels read a state's inputs before they write its outputs; the
+// tile kernels read some of them again, and leave states to an FP64 kernel behind them, after
+// outputs have been written.
+bool in_place(const std::vector<ArgSpec>& args, const std::vector<void*>& d, int64_t n, size_t except = ~size_t(0)) {
+  auto end = [&](size_t i) { return (const char*)d[i] + (size_t)args[i].rows * n * args[i].elem; };
+  for (size_t o = 0; o < args.size(); ++o)
+    for (size_t i = 0; i < args.size(); ++i)
+      if (o != except && args[o].out && args[i].in && d[o] && d[i] && (const char*)d[o] < end(i) && (const char*)d[i] < end(o)) return true;
+  return false;
+}
+
 // Classify the non-null pointers of a call: returns 1 (all device), 0 (all host) or -1 (mixed).
 int classify(const std::vector<const void*>& ptrs) {
   int kind = -2;
@@ -742,10 +754,11 @@ std::vector<std::string> jac_groups(const pyro_mech* h) {
 int launch_deriv(const pyro_mech* h, const pyro_mech::Group& G, int64_t n, void* stream, void** params);
 
 // Launch a product on device pointers: params ends with the FP64 kernel's open_only flag
-int launch_product(pyro_mech* h, const std::vector<std::string>& gs, int64_t n, void* stream, void** params, int* open_only) {
+int launch_product(pyro_mech* h, const std::vector<std::string>& gs, int64_t n, void* stream, void** params, int* open_only,
+                   bool alias) {
   const pyro_mech::Group& G = h->groups[gs[0]];
   if (h->opt.warp) return launch_warp(h, G, n, stream, params);
-  *open_only = gs.size() > 1 ? 1 : 0;
+  *open_only = gs.size() > 1 && !alias ? 1 : 0;
   if (*open_only) {
     const pyro_mech::Group& t = h->groups[gs[1]];
     const unsigned grid = (unsigned)std::min((n + 31) / 32, (int64_t)h->num_sms * t.blocks_per_sm);
@@ -769,7 +782,7 @@ std::string jac_group(const pyro_mech* h, bool adiabatic) {
 // the FP64 kernel (thread or warp per state) those that the tile kernel left open.
 // newton=fp64 keeps its own temperature iteration: solved first, then rates at T.
 int launch_rates(const pyro_mech* h, int64_t n, const void* rho, const void* T_or_e, int energy, const void* Y,
-                 void* T_out, void* omega, unsigned long long* fail_ctr, void* stream) {
+                 void* T_out, void* omega, unsigned long long* fail_ctr, void* stream, bool alias = false) {
   long long nn = n;
   double Tg = 1200.0, tol = 1e-10;
   int max_iter = 50, open_only = 0;
@@ -777,7 +790,7 @@ int launch_rates(const pyro_mech* h, int64_t n, const void* rho, const void* T_o
   const void* Tin = T_or_e;
   auto it = h->groups.find("tile");
   const bool tile = it != h->groups.end() && it->second.f;
-  if (tile) {
+  if (tile && !alias) {
     const pyro_mech::Group& G = it->second;
     if (energy && !h->opt.mixed) {
       void* pt[] = {&nn, &Tin, &Y, &none, &Tg, &max_iter, &tol, &T_out, &none, &fail_ctr};
@@ -787,7 +800,8 @@ int launch_rates(const pyro_mech* h, int64_t n, const void* rho, const void* T_o
     }
     const int64_t need = (n + 31) / 32, cap = (int64_t)h->num_sms * G.blocks_per_sm;
     // as long as every tile's cluster is resident at once, the chunks of a tile run in parallel
-    int split = need <= G.clusters ? 1 : 0;
+    // (every block of a cluster reads the energies, one writes the temperatures: not over them)
+    int split = need <= G.clusters && !(energy && T_out == T_or_e) ? 1 : 0;
     void* params[] = {&nn, &rho, &Tin, &energy, &Y, &T_out, &omega, &Tg, &max_iter, &tol, &fail_ctr, &split};
     CUlaunchConfig cfg;
     CUlaunchAttribute attr;
@@ -1084,10 +1098,13 @@ int pyro_net_production_rates(const pyro_mech* hc, int64_t n, const double* rho,
   if (n == 0) return PYRO_OK;
   if (int rc = check_device(h)) return rc;
   const int64_t NS = h->m.n_species();
-  int rc = with_args(h, n, {{rho, 1, 8, true, false}, {T_or_e, 1, 8, true, false}, {Y, NS, 8, true, false},
-                         {input_is_energy ? T_out : nullptr, 1, 8, false, true}, {omega, NS, 8, false, true}},
-                     stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
-                       return launch_rates(h, nc, d[0], d[1], input_is_energy ? 1 : 0, d[2], d[3], d[4], h->d_fail, st);
+  const std::vector<ArgSpec> args = {{rho, 1, 8, true, false}, {T_or_e, 1, 8, true, false}, {Y, NS, 8, true, false},
+                                     {input_is_energy ? T_out : nullptr, 1, 8, false, true}, {omega, NS, 8, false, true}};
+  int rc = with_args(h, n, args, stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
+                       // T over e: each block of the tile kernel reads its energies before it writes temperatures
+                       const bool T_over_e = d[3] && d[3] == d[1];
+                       return launch_rates(h, nc, d[0], d[1], input_is_energy ? 1 : 0, d[2], d[3], d[4], h->d_fail, st,
+                                           in_place(args, d, nc, T_over_e ? 3 : ~size_t(0)));
                      }, h->opt.warp || h->emitted.stats["omega_store_global"] <= 0);   // no per-block global scratch
   if (rc) return rc;
   return input_is_energy ? maybe_checked(h, stream) : PYRO_OK;
@@ -1133,13 +1150,14 @@ int pyro_jvp(const pyro_mech* hc, int64_t n, const double* rho, const double* T,
   const std::vector<std::string> gs = product_groups(h, "jvp");
   if (int rc = ensure_groups(h, gs)) return rc;
   const int64_t NS = h->m.n_species();
-  return with_args(h, n, {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false}, {d_rho, 1, 8, true, false},
-                       {d_T, 1, 8, true, false}, {d_Y, NS, 8, true, false}, {d_omega, NS, 8, false, true}},
-                   stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
+  const std::vector<ArgSpec> args = {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false},
+                                     {d_rho, 1, 8, true, false}, {d_T, 1, 8, true, false}, {d_Y, NS, 8, true, false},
+                                     {d_omega, NS, 8, false, true}};
+  return with_args(h, n, args, stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
                      long long nn = nc;
                      int open_only = 0;
                      void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &d[5], &d[6], &h->groups[gs[0]].store, &open_only};
-                     return launch_product(h, gs, nc, st, params, &open_only);
+                     return launch_product(h, gs, nc, st, params, &open_only, in_place(args, d, nc));
                    }, h->opt.warp);
 }
 
@@ -1153,13 +1171,14 @@ int pyro_vjp(const pyro_mech* hc, int64_t n, const double* rho, const double* T,
   const std::vector<std::string> gs = product_groups(h, "vjp");
   if (int rc = ensure_groups(h, gs)) return rc;
   const int64_t NS = h->m.n_species();
-  return with_args(h, n, {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false}, {omega_bar, NS, 8, true, false},
-                       {rho_bar, 1, 8, false, true}, {T_bar, 1, 8, false, true}, {Y_bar, NS, 8, false, true}},
-                   stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
+  const std::vector<ArgSpec> args = {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false},
+                                     {omega_bar, NS, 8, true, false}, {rho_bar, 1, 8, false, true}, {T_bar, 1, 8, false, true},
+                                     {Y_bar, NS, 8, false, true}};
+  return with_args(h, n, args, stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
                      long long nn = nc;
                      int open_only = 0;
                      void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4], &d[5], &d[6], &h->groups[gs[0]].store, &open_only};
-                     return launch_product(h, gs, nc, st, params, &open_only);
+                     return launch_product(h, gs, nc, st, params, &open_only, in_place(args, d, nc));
                    }, h->opt.warp);
 }
 
@@ -1180,10 +1199,11 @@ int pyro_jacobian(const pyro_mech* hc, int64_t n, const double* rho, const doubl
   const int64_t NS = h->m.n_species();
   if (!cta)
     if (int rc = ensure_jac_scratch(h, G, n)) return rc;
-  return with_args(h, n, {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false}, {J, (int64_t)NP * NP, 8, false, true}},
-                   stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
+  const std::vector<ArgSpec> args = {{rho, 1, 8, true, false}, {T, 1, 8, true, false}, {Y, NS, 8, true, false},
+                                     {J, (int64_t)NP * NP, 8, false, true}};
+  return with_args(h, n, args, stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
                      long long nn = nc;
-                     int open_only = gs.size() > 1 ? 1 : 0;
+                     int open_only = gs.size() > 1 && !in_place(args, d, nc) ? 1 : 0;
                      if (open_only) {
                        pyro_mech::Group& t = h->groups[gs[1]];
                        void* pt[] = {&nn, &d[0], &d[1], &d[2], &d[3], &t.store};
@@ -1209,12 +1229,12 @@ int pyro_transport(const pyro_mech* hc, int64_t n, const double* T, const double
   if (int rc = ensure_groups(h, tile ? std::vector<std::string>{"tr", "ttr"} : std::vector<std::string>{"tr"})) return rc;
   pyro_mech::Group& G = h->groups["tr"];
   const int64_t NS = h->m.n_species();
-  return with_args(h, n, {{T, 1, 8, true, false}, {Y, NS, 8, true, false}, {mu, 1, 8, false, true},
-                          {kappa, 1, 8, false, true}, {D_mix, NS, 8, false, true}},
-                   stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
+  const std::vector<ArgSpec> args = {{T, 1, 8, true, false}, {Y, NS, 8, true, false}, {mu, 1, 8, false, true},
+                                     {kappa, 1, 8, false, true}, {D_mix, NS, 8, false, true}};
+  return with_args(h, n, args, stream, [&](std::vector<void*>& d, int64_t nc, void* st) {
                      long long nn = nc;
-                     int open_only = tile ? 1 : 0;
-                     if (tile) {   // 32 states per block; the FP64 kernel then takes the states it left open
+                     int open_only = tile && !in_place(args, d, nc) ? 1 : 0;
+                     if (open_only) {   // 32 states per block; the FP64 kernel then takes the states it left open
                        const pyro_mech::Group& t = h->groups["ttr"];
                        void* params[] = {&nn, &d[0], &d[1], &d[2], &d[3], &d[4]};
                        const unsigned grid = (unsigned)std::min((nc + 31) / 32, (int64_t)h->num_sms * t.blocks_per_sm);
