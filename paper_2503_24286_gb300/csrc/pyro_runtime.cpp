@@ -490,6 +490,9 @@ int check_device(const pyro_mech* h) {
   if (cudaGetDevice(&dev) != cudaSuccess) return fail(PYRO_ECUDA, "cudaGetDevice failed");
   if (dev != h->device) return fail(PYRO_EINVAL, "mechanism was loaded on device " + std::to_string(h->device) +
                                                    " but the current device is " + std::to_string(dev));
+  // the kernels are launched through the driver, which needs the context current in this thread
+  // (a thread that has made no runtime call of its own has none)
+  if (cudaSetDevice(dev) != cudaSuccess) return fail(PYRO_ECUDA, "cudaSetDevice failed");
   return PYRO_OK;
 }
 
