@@ -19,6 +19,7 @@
 #include <mutex>
 #include <sstream>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -555,6 +556,17 @@ const char* group_kernel(const std::string& g) {
        : g == "tjac" ? "pyro_jacobian_tile" : "pyro_jacobian";
 }
 
+// Start a thread; false where the system has none left (the caller then does the work itself)
+template <class F>
+bool start_thread(std::vector<std::thread>& th, F f) {
+  try {
+    th.emplace_back(f);
+    return true;
+  } catch (const std::system_error&) {
+    return false;
+  }
+}
+
 // Compile (in parallel threads, cached on disk) and load the named derivative
 // kernel groups that are not loaded yet.
 int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
@@ -569,13 +581,13 @@ int ensure_groups(pyro_mech* h, const std::vector<std::string>& names) {
   std::vector<std::vector<char>> cubins(todo.size());
   std::vector<int> rcs(todo.size(), PYRO_OK);
   std::vector<std::string> errs(todo.size());
+  auto compile = [&](size_t i) {
+    rcs[i] = compile_cached(h->emitted.group_sources.at(todo[i]), h->opt.cache, cubins[i]);
+    if (rcs[i]) errs[i] = pyro_last_error();
+  };
   std::vector<std::thread> th;
-  for (size_t i = 0; i < todo.size(); ++i) {
-    th.emplace_back([&, i] {
-      rcs[i] = compile_cached(h->emitted.group_sources.at(todo[i]), h->opt.cache, cubins[i]);
-      if (rcs[i]) errs[i] = pyro_last_error();
-    });
-  }
+  for (size_t i = 0; i < todo.size(); ++i)
+    if (i + 1 == todo.size() || !start_thread(th, [&, i] { compile(i); })) compile(i);
   for (auto& t : th) t.join();
   if (!h->module) {   // compile-only handle: record the build, load nothing
     for (size_t i = 0; i < todo.size(); ++i) {
@@ -883,11 +895,11 @@ int pyro_mech_load(const char* mech_path, const char* options, pyro_mech** out) 
   // compile (or fetch from the cache)
   std::vector<char> cubin;
   const bool tile = h->emitted.stats["tile"] > 0;
-  std::thread tile_compile;   // the tile kernel's unit beside the main one (fetched from the cache below)
+  std::vector<std::thread> tile_compile;   // the tile kernel's unit beside the main one (fetched from the cache below)
   if (tile && h->opt.cache)
-    tile_compile = std::thread([&] { std::vector<char> c; compile_cached(h->emitted.group_sources.at("tile"), true, c); });
+    start_thread(tile_compile, [&] { std::vector<char> c; compile_cached(h->emitted.group_sources.at("tile"), true, c); });
   const int crc = compile_cached(h->emitted.source, h->opt.cache, cubin);
-  if (tile_compile.joinable()) tile_compile.join();
+  for (auto& t : tile_compile) t.join();
   if (crc) { delete h; return crc; }
   h->emitted.stats["cubin_bytes"] = (double)cubin.size();
   if (!h->opt.device) {
