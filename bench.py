@@ -20,6 +20,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -58,15 +59,32 @@ def sm_max_mhz_of(gpu_index: int) -> float:
     except (OSError, ValueError, IndexError, subprocess.SubprocessError):
         return SM_MAX_MHZ_DEFAULT
 
-# DRAM traffic of one launch of the timed kernel, from an ncu capture of this
-# kernel source (hash of the emitted source); None once the kernel changes.
-PROFILED_TRAFFIC = {
-    # 2^19-state ncu captures scaled by 8 to a 2^22-state launch
-    "953a6879ca9d63b7": 3.334e9,
-    "a24d27e8509fd73d": 3.330e9,
-    # 2^20-state capture (dram__bytes_read.sum + dram__bytes_write.sum) scaled by 4
-    "d480c6fd1d99f5f7": 3.497e9,
+# One launch of the timed kernel from an ncu capture of its sources (kernel_source_hash): DRAM
+# bytes of a 2^22-state launch and warp instructions per state; none once a source changes.
+PROFILED = {
+    # a capture of 2^20 states, energy input: 4,326,255,393 warp instructions, 461.6 MB read, 412.2 MB written
+    "9c7031c8c8f4e7e5": {"dram_bytes": 3.495e9, "warp_instructions_per_state": 4126.0},
 }
+
+# what the tile kernel of the net production rates is made of, beside the emitted tables
+TILE_SOURCES = ("pyro_tile.cuh", "pyro_fixed_math.cuh", "pyro_device_math.cuh", "pyro_emit_tile.cpp")
+
+
+def kernel_source_hash(mech) -> str:
+    """Of the emitted FP64 source and the tile kernel's sources, their comments left out."""
+    h = hashlib.sha256(mech.source().encode())
+    csrc = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_2503_24286_gb300", "csrc")
+    for name in TILE_SOURCES:
+        with open(os.path.join(csrc, name)) as f:
+            lines = (re.sub(r"//.*", "", line).strip() for line in f)
+            h.update("\n".join(line for line in lines if line).encode())
+    return h.hexdigest()[:16]
+
+
+def fp64_fraction(mech, tile_stat, flops_per_s, peak):
+    """The FP64 kernel's operations against the FP64 peak; None where a tile kernel evaluates the
+    states, which does most of that work on the integer pipe."""
+    return None if mech.stat(tile_stat) > 0 else flops_per_s / peak
 
 
 def _dist():
@@ -253,15 +271,16 @@ def derivative_rates(mech, synth, dev, stream, args, rank):
         res[name + "_ms"] = ms
         res[name + "_per_s"] = n / (ms * 1e-3)
     res["jacobian_out_GB_per_s"] = 54 * 54 * 8 * n / (res["jacobian_ms"] * 1e-3) / 1e9
-    # FP64 roofline of each derivative kernel: the emitter's static FP64 flops per
-    # state x states/s, against the FP64 peak (Jacobian-evals/s vs FP64 roofline)
-    for name, key in (("jvp", "jvp_fp64_flops_per_point"), ("vjp", "vjp_fp64_flops_per_point"),
-                      ("jacobian", "jacobian_fp64_flops_per_point"),
-                      ("omega_isothermal", "omega_fp64_flops_per_point")):
+    # the FP64 form's work: the emitter's static FP64 flops per state x states/s (what the FP64
+    # kernels would have to do at this rate); a fraction of the peak only where they run
+    for name, key, tile in (("jvp", "jvp_fp64_flops_per_point", "jvp_tile"),
+                            ("vjp", "vjp_fp64_flops_per_point", "vjp_tile"),
+                            ("jacobian", "jacobian_fp64_flops_per_point", "jacobian_tile"),
+                            ("omega_isothermal", "omega_fp64_flops_per_point", "tile")):
         f = mech.stat(key)
         res[name + "_fp64_flops_per_state_static"] = f
-        res[name + "_gflops"] = f * res[name + "_per_s"] / 1e9
-        res[name + "_frac"] = f * res[name + "_per_s"] / (args.fp64_peak * 1e9)
+        res[name + "_fp64_form_gflops"] = f * res[name + "_per_s"] / 1e9
+        res[name + "_frac"] = fp64_fraction(mech, tile, f * res[name + "_per_s"], args.fp64_peak * 1e9)
     del J
     return res
 
@@ -351,11 +370,11 @@ def start_large_compile(path):
 
 def large_mechanism_rates(path, synth, dev, stream, args, rank):
     """160 species / 1100 reactions at 2^21 states: T from e + omega, and the JVP and
-    VJP (intermediates recomputed, nothing stored), each with one thread per state
-    (emitted straight-line code, species arrays in a global scratch) against one
-    warp per state (lanes split the reactions); also the warp variant of the
-    forward on the 53-species workload.  Each row with its FP64 roofline fraction
-    (emitter's static FP64 flops per state)."""
+    VJP (intermediates recomputed, nothing stored), by the tile kernel (default handle;
+    the VJP of this mechanism does not fit it), by the FP64 kernels alone (tile=0)
+    with one thread per state (emitted straight-line code, species arrays in a
+    global scratch) and with one warp per state (lanes split the reactions).  The
+    FP64 rows with their roofline fraction (emitter's static FP64 flops per state)."""
     import torch
     from paper_2503_24286_gb300 import binding as B
     cfg = synth.CONFIGS[4]
@@ -363,8 +382,9 @@ def large_mechanism_rates(path, synth, dev, stream, args, rank):
     res = {"workload": "synthetic 160 species / 1100 reactions (80 third-body, 60 Troe), %d states, "
                        "T ~ U[300, 2800] K, p ~ U[1, 40] atm; T from e + omega, JVP and VJP (unit-scale random "
                        "seed vectors)" % n}
-    mt = B.Mechanism(path)
-    mw = B.Mechanism(path, "variant=warp")
+    m0 = B.Mechanism(path)
+    mt = B.Mechanism(path, "tile=0")
+    mw = B.Mechanism(path, "tile=0;variant=warp")
     T, p, Y = synth.generate_states_torch(160, n, cfg["T"], cfg["p_atm"], synth.STATE_SEED_BASE + 4 + 7919 * rank, dev)
     rho = mt.density(p, T, Y)
     e = mt.internal_energy(T, Y)
@@ -389,11 +409,11 @@ def large_mechanism_rates(path, synth, dev, stream, args, rank):
     f_fwd = mt.stat("omega_fp64_flops_per_point") + 2 * mt.stat("tsolve_collapse_fp64_ops") + \
         3 * 2 * mt.stat("tsolve_iter_fp64_ops_mixed")
     res["fp64_flops_per_state_static"] = f_fwd
-    for tag, m in (("thread_per_state", mt), ("warp_per_state", mw)):
+    for tag, m in (("tile", m0), ("thread_per_state", mt), ("warp_per_state", mw)):
         ms = timed(lambda: m.net_production_rates(rho, Y, e=e, T_out=To, out=w))
         res[tag + "_ms"] = ms
         res[tag + "_states_per_s"] = n / (ms * 1e-3)
-        res[tag + "_frac"] = f_fwd * n / (ms * 1e-3) / peak
+        res[tag + "_frac"] = fp64_fraction(m, "tile", f_fwd * n / (ms * 1e-3), peak)
         assert m.nonconverged() == 0
     g = torch.Generator(device=dev)
     g.manual_seed(7)
@@ -403,7 +423,7 @@ def large_mechanism_rates(path, synth, dev, stream, args, rank):
     w_bar = torch.randn((160, n), dtype=torch.float64, device=dev, generator=g)
     args.large_compile.join()
     deriv = {}
-    for tag, m in (("thread_per_state", mt), ("warp_per_state", mw)):
+    for tag, m in (("tile", m0), ("thread_per_state", mt), ("warp_per_state", mw)):
         try:
             if tag == "warp_per_state" and m.stat("deriv_warp_per_state") <= 0:
                 deriv[tag] = {"unavailable": "no warp-per-state derivative kernels for this mechanism"}
@@ -420,7 +440,7 @@ def large_mechanism_rates(path, synth, dev, stream, args, rank):
             r[name + "_ms"] = ms
             r[name + "_states_per_s"] = n / (ms * 1e-3)
             r[name + "_fp64_flops_per_state_static"] = fl
-            r[name + "_frac"] = fl * n / (ms * 1e-3) / peak
+            r[name + "_frac"] = fp64_fraction(m, name + "_tile", fl * n / (ms * 1e-3), peak)
         deriv[tag] = r
     res["derivatives"] = deriv
     # dense Jacobians, one block of 8 warps per state (variant=warp), on --large-jac-points
@@ -597,7 +617,7 @@ def pressure_dependent_rates(synth, dev, stream, args, rank):
     return {"workload": "53 species / 325 reactions with 10 SRI falloff and 20 PLOG (3-5 nodes in [0.1, 100] atm) "
                         "reactions, %d states, T ~ U[300, 2800] K, p ~ U[0.5, 20] atm; T from e + omega" % n,
             "ms": ms, "states_per_s": n / (ms * 1e-3), "fp64_flops_per_state_static": flops,
-            "fp64_frac": flops * n / (ms * 1e-3) / (args.fp64_peak * 1e9)}
+            "fp64_frac": fp64_fraction(m, "tile", flops * n / (ms * 1e-3), args.fp64_peak * 1e9)}
 
 
 def transport_rates(mech, synth, dev, stream, args, rank):
@@ -632,7 +652,7 @@ def transport_rates(mech, synth, dev, stream, args, rank):
     return {"workload": "53 species, %d states, T ~ U[300, 2800] K, Dirichlet Y; mu (Wilke), kappa, D_km" % n,
             "ms": ms, "states_per_s": n / (ms * 1e-3),
             "fp64_ops_per_state_static": ops,
-            "fp64_pipe_frac": ops * n / (ms * 1e-3) / (args.fp64_peak * 1e9 / 2)}
+            "fp64_pipe_frac": fp64_fraction(mech, "transport_tile", ops * n / (ms * 1e-3), args.fp64_peak * 1e9 / 2)}
 
 
 def run_rows_only(args):
@@ -783,7 +803,7 @@ def run_ours(args):
     warp53 = None
     large = None
     if not args.no_large:
-        mw = B.Mechanism(path, "variant=warp")
+        mw = B.Mechanism(path, "tile=0;variant=warp")
         for _ in range(3):
             mw.net_production_rates(rho, Y, e=e, T_out=T, out=omega)
         torch.cuda.synchronize(dev)
@@ -812,12 +832,24 @@ def run_ours(args):
         cn = crank_nicolson_rates(synth, dev, stream, args, rank)
 
     # --- roofline of the timed kernel ---------------------------------------------------
+    # the tile kernel: warp instructions (profiled for these sources) against the issue slots of
+    # the SMs; the FP64 kernel alone: its static FP64 operations against the FP64 pipe
     flops_fwd = mech.stat("omega_fp64_flops_per_point")
     flops_ts = 2 * mech.stat("tsolve_collapse_fp64_ops") + 3 * 2 * mech.stat("tsolve_iter_fp64_ops_mixed")
     flops_pt = flops_fwd + flops_ts
-    achieved = flops_pt * n / (ms * 1e-3) / 1e9
-    src_hash = hashlib.sha256(mech.source().encode()).hexdigest()[:16]
-    traffic = PROFILED_TRAFFIC.get(src_hash)
+    src_hash = kernel_source_hash(mech)
+    prof = PROFILED.get(src_hash, {})
+    traffic = prof.get("dram_bytes")
+    if tile:
+        bound, unit, peak = "issue", "G warp instructions/s", 4 * n_sm * sm_max * 1e-3
+        peak_source = "4 warp instructions/SM/clk x %d SMs (device) x %.0f MHz (nvidia-smi clocks.max.sm)" % (n_sm, sm_max)
+        ops_pt = prof.get("warp_instructions_per_state")
+    else:
+        bound, unit, peak = "alu", "GFLOP/s", args.fp64_peak
+        peak_source = ("FP64 pipe: 2 lanes/SM/clk (DFMA microbenchmark) x %d SMs (device) x %.0f MHz (nvidia-smi "
+                       "clocks.max.sm) x 2 flops/DFMA" % (n_sm, sm_max))
+        ops_pt = flops_pt
+    achieved = ops_pt * n / (ms * 1e-3) / 1e9 if ops_pt else None
     clocks = clk.summary()
 
     line = None
@@ -829,15 +861,13 @@ def run_ours(args):
                 "warmup": args.warmup, "ms_per_step": ms_max, "higher_is_better": True, "scaling": "weak",
                 "vs_baseline": None, "dtype": "f64", "data": "synthetic", "config": workload_config(n),
                 "parallelism": "points sharded across ranks, no collective" if world > 1 else "1 GPU",
-                "roofline": {"bound": "alu", "achieved": achieved, "peak": args.fp64_peak, "unit": "GFLOP/s",
-                             "frac": achieved / args.fp64_peak, "traffic": traffic,
-                             "note": ("achieved counts the FP64 operations of the FP64 form; the tile kernel does most "
-                                      "of them on the integer pipe, so frac may exceed 1" if tile else None),
-                             "peak_source": "FP64 pipe: 2 lanes/SM/clk (DFMA microbenchmark) x %d SMs (device) x "
-                                            "%.0f MHz (nvidia-smi clocks.max.sm) x 2 flops/DFMA" % (n_sm, sm_max),
-                             "flops_per_state": flops_pt,
-                             "frac_at_sampled_clock": (achieved / (args.fp64_peak * clocks["sm_mhz"] / sm_max)
-                                                       if clocks.get("sm_mhz") else None)},
+                "roofline": {"bound": bound, "achieved": achieved, "peak": peak, "unit": unit,
+                             "frac": achieved / peak if achieved else None, "traffic": traffic,
+                             "peak_source": peak_source, "operations_per_state": ops_pt,
+                             "fp64_form_flops_per_state": flops_pt,
+                             "fp64_form_gflops": flops_pt * n / (ms * 1e-3) / 1e9,
+                             "frac_at_sampled_clock": (achieved / (peak * clocks["sm_mhz"] / sm_max)
+                                                       if achieved and clocks.get("sm_mhz") else None)},
                 "cpu_baseline": {"value": rate_cpu, "unit": "states/s", "cores": cores, "kind": "oracle",
                                  "sample": "%d states of the same workload (seeded), T solve + omega, %.1f s"
                                            % (args.cpu_sample, dt),
