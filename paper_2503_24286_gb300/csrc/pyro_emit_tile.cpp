@@ -221,7 +221,10 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
   // warps an SM 7.3 ms, one of 24 warps 7.6, two of 8 warps 7.9, one of 16 warps 7.8; with
   // the rows in more than one chunk two blocks lose (8.3 ms and more).  10 species / 21
   // reactions: eight blocks of 4 warps 0.81 ms, four of 8 warps 0.96 ms; 160 / 1100
-  // (2^18 states): one block of 24 warps 5.6 ms, of 16 warps 6.4 ms.
+  // (2^18 states): one block of 24 warps 5.6 ms, of 16 warps 6.4 ms.  Between them, 16 to 30
+  // species: 60 rows, 4096 states by 4, 8 and 12 warps 38.5, 32.7, 33.0 us, 2^20 states 1.76,
+  // 1.77, 1.90 ms; 80 rows 43.9, 36.6, 35.8 us, 2.33, 2.39, 2.36 ms; 110 rows 54.3, 38.8, 37.5
+  // us, 3.11, 3.19, 3.02 ms: 8 warps are within 6 % of the best at every size.
   int mrows = 0;                                 // reactions with an [M] adjoint
   for (int j = 0; j < NR; ++j) if (classes(m.reactions[j])) ++mrows;
   const int fixed_bytes = jac ? 8192 + 1280 * (N + 1) + 6 * 24 * 256 + 32 * (4 * 8 + 3 * 8 + 8 + 4) + 256
@@ -335,7 +338,7 @@ TileEmit emit_tile_unit(const Mechanism& m, TileKind what) {
             rec[6] = (i64)mrow;
             mrow_of[j] = mrow++;
             rec[5] = (i64)ax.size();
-            if (cls) {
+            {                                    // auxiliary data
               std::vector<i64> x(16, 0);
               std::vector<double> fd(16, 0.0);
               if (cls == 5) {

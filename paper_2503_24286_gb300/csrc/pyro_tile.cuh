@@ -15,12 +15,13 @@
 //      normalised: its error is 2^-51 of the larger of the two rates);
 //   3  per species the sum of its reactions' rates, aligned to the largest exponent
 //      met so far, normalised once into the output.
-// Bound: the integer pipes (53 species / 325 reactions: 130 k warp instructions a tile,
-// issue 0.54 a cycle, multiply pipe 54 % and FP64 pipe 33 % of their limits averaged over the
-// phases, which load them in turn; DRAM 1 %).  Measured against one thread per state, whose
+// Bound: the integer pipes (53 species / 325 reactions: 132 k warp instructions a tile,
+// issue 0.53 a cycle, ALU pipe 43 % and FP64 pipe 32 % of their limits averaged over the
+// phases, which load them in turn; DRAM 2 %).  Measured against one thread per state, whose
 // 7,270 FP64 instructions a state ran at the FP64 pipe's limit: 2^22 states of 53 species,
-// energy input, 57.2 -> 26.8 ms; one state 332 -> 47 us; 160 species, 2^18 states (against
-// one warp per state) 12.9 -> 5.4 ms.  Leaving the exponential's last product and the
+// energy input, 57.2 -> 26.4 ms; one state 332 -> 47 us; 160 species, 2^18 states (against
+// one warp per state) 12.9 -> 5.4 ms.  Errors against extended precision: rates 1.5e-15 of a
+// state's norm on average (FP64 kernel 1.0e-14), T 1.8e-16 (6.1e-16).  Leaving the exponential's last product and the
 // difference of the two rates to FP64 was slower (7.24 against 7.11 ms per 2^20 states).
 //
 // All warps of a block run the same code at about the same time and the loops over

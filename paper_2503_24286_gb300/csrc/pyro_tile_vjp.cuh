@@ -6,8 +6,8 @@
 // and stores Db; the adjoints of the activities are then gathered per species,
 //   abar_i = sum_j +-Db_j (product of the side's other factors),
 // in a fixed order, with no conflicts between warps: 17 FP64 instructions a reaction of two
-// factors a side in all, against some 40 of the per-thread kernel (2^18 states 8.6 -> 5.2 ms,
-// bound by the FP64 pipe).  [M] adjoints likewise.
+// factors a side in all, against some 40 of the per-thread kernel (2^18 states 8.6 -> 5.3 ms,
+// FP64 pipe 81 of its 84 %).  [M] adjoints likewise.
 // States outside the tables' range, with non-finite inputs or results, get TILE_OPEN in
 // rho_bar and are evaluated by the FP64 kernel.
 #define TILE_DERIV

@@ -3,7 +3,7 @@
 //
 // Included by the emitted unit, which defines the tables (tt_*) and sizes.  The
 // per-thread kernel spent 24.5 k FP64 instructions a state on 53 species: 19 cycles of
-// an SM each, 13.1 ms per 2^18 states.  This kernel takes 5.9 ms, about half of it FP64-bound
+// an SM each, 13.1 ms per 2^18 states.  This kernel takes 6.2 ms, about half of it FP64-bound
 // (two FMAs a pair, the species fits), half integer work.  Here
 //  * Wilke's sums (three products with constant N x N matrices) are integer dot
 //    products: mole fractions and x/P, x/P^2 in fixed point, sums exact to 2^-54;
