@@ -3,7 +3,7 @@
 //
 // Included by the emitted unit, which defines the tables (tt_*) and sizes.  The
 // per-thread kernel spent 24.5 k FP64 instructions a state on 53 species: 19 cycles of
-// an SM each, 13.1 ms per 2^18 states.  This kernel takes 6.2 ms, about half of it FP64-bound
+// an SM each, 13.1 ms per 2^18 states.  This kernel takes 6.0 ms, about half of it FP64-bound
 // (two FMAs a pair, the species fits), half integer work.  Here
 //  * Wilke's sums (three products with constant N x N matrices) are integer dot
 //    products: mole fractions and x/P, x/P^2 in fixed point, sums exact to 2^-54;
@@ -30,18 +30,20 @@ __device__ __forceinline__ Pair tt_pair(i64 v) {
   return p;
 }
 
-// sum of c y: h 2^64 + l 2^32 (of the products of the low halves their upper half: left out
-// altogether, they alone were a mean error of 4.0e-16 of mu, FP64 sums 3.2e-16).
+// sum of c y: h 2^64 + l 2^32 (LOW: and the upper half of the products of the low halves;
+// left out of the sums of x/P^2, whose y are the smallest, they are a mean error of 3.8e-16
+// of mu, of x/P 1.2e-16, of x 1e-17, FP64 sums altogether 3.2e-16; all three 4 % of the kernel's
+// time, the one 1 %).
 // With |c| < 2^57 and y = x 2^61 the word h << 7 stays below 2^61 sum |x|, and l below
 // 2^60 sum |x| + N 2^55.
-struct TtDot {
+template <bool LOW> struct TtDot {
   i64 h, l;
   __device__ __forceinline__ void add(i64 c, Pair y) {
     const int ch = (int)(c >> 32), cl = (int)c;
     h += (i64)ch * y.hi;
     l += (i64)ch * y.lo;
     l += (i64)cl * y.hi;
-    l += (i64)pfx::mulhi_s(cl, y.lo);
+    if (LOW) l += (i64)pfx::mulhi_s(cl, y.lo);
   }
   __device__ __forceinline__ double value(int f) const { return pfx::scaled((h << 7) + (l >> 25), 57 - f); }
 };
@@ -174,7 +176,8 @@ pyro_transport_tile(i64 n, const double* __restrict__ g_T, const double* __restr
       double mu = 0.0;
 #pragma unroll 1
       for (int k = w; k < NSP; k += NW) {
-        TtDot a, b, e;
+        TtDot<false> a, b;
+        TtDot<true> e;
         a.h = a.l = b.h = b.l = e.h = e.l = 0;
         const longlong2* c = (const longlong2*)(tt_wilke + k * NSP * 4);
 #pragma unroll 4
